@@ -139,8 +139,10 @@ typedef struct rddmc_leak_params {
  *                 persistent grid of ctas_per_sm * #SM CTAs of threads_per_cta
  *                 threads (a multiple of 32, at most 256); `chunk` transitions
  *                 (multiple of 4) between warp refills.
- *   table_in_smem 1: stage the fast row heads in shared memory when they fit;
- *                 0: gather them from global memory (L1/L2).
+ *   table_in_smem 1: stage the fast row heads in shared memory when they fit
+ *                 (the dust weight method; the other walks read a denser table
+ *                 through L1, which measured faster); 0: gather them from
+ *                 global memory (L1/L2).
  *   time_slice_us wall-time slice (0 = none): a thread that reaches a chunk
  *                 boundary more than this many microseconds after its CTA
  *                 started saves its packet and takes no new one.  Needs saved
@@ -274,9 +276,9 @@ int rddmc_reset_tallies(const rddmc_grid* grid, void* d_tallies, size_t tally_by
 /*
  * rddmc_launch_packets -- walk packets (Sec. 2.3) with one persistent kernel.
  * Each thread holds one packet: it draws one word of the packet's transition
- * stream per transition, gathers the 8-byte head of its state's row (its two
- * frequency thresholds) and, unless the word falls in a plain frequency move,
- * the full 16/32-byte row, and takes the
+ * stream per transition, gathers the frequency thresholds around its state (16
+ * bytes for two transitions, or the 8-byte head of each row) and, unless the
+ * words fall in plain frequency moves, the full 16/32-byte row, and takes the
  * outcome whose threshold interval holds the word (the categorical form of the
  * competing exponentials of eq. l_min_1/2: the argmin of independent
  * exponentials with rates k_X is X with probability k_X / sum k).  Packets

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "grid.h"
+#include "pairs.cuh"
 
 using namespace rddmc;
 
@@ -214,6 +215,7 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     g->off_abs = off; off += align256((uint64_t)g->n_class * J * 4);
     g->off_wq = off; off += align256((uint64_t)g->n_class * J * 8);
     g->off_ka = off; off += align256((uint64_t)g->n_class * J * 4);
+    g->off_pair = off + 256; off += g->pairs() ? 256 + align256((uint64_t)g->n_class * J * 16 + kPairPad) : 0;
     g->table_bytes = off;
     *out = g;
     return RDDMC_OK;

@@ -1,0 +1,110 @@
+// pairs.cuh -- two frequency moves per gather: the pair table of the DDMC walk
+// and the transition stream it consumes.
+//
+// Frequency moves dominate a thick line, and two of them in a row visit only
+// the states s-1, s and s+1.  The pair of row s is 16 bytes,
+//   {T[s-1], T[s], T[s+1], guard},
+// T the row's first threshold (w < T: bin - 1) and guard the smallest fast
+// threshold of the three rows (0 when one of them has a frequency outcome that
+// is not a plain move).  When both words are below the guard, both transitions
+// are frequency moves and the pair decides them; otherwise the walk takes the
+// rows one by one.  Rows outside the class block are never reached (the end
+// bins have no move past them: T = 0 at the bottom, T = the fast threshold at
+// the top) and do not enter the guard.
+#pragma once
+#include <cstdint>
+
+#include "rddmc_internal.cuh"
+
+namespace rddmc {
+
+struct alignas(16) Pair {
+    uint32_t m1, z, p1, guard;
+};
+
+// The walk keeps a state as the byte offset 16 s of its pair, so that a gather
+// takes a uniform base and a 32-bit offset and needs no 64-bit address product
+// (kPairRows keeps offsets below 2^31).  Two moves change the offset by -32, 0
+// or 32: they add 32 per upward move, and the constant -32 rides on the next
+// gather's address, so a move is one predicated add.
+//
+// Four frequency moves on the words of r from offset o0: two gathers through L1
+// (the table is read-only during a walk).  up2 and up4 return 32 times the
+// upward moves of the first two and of all four transitions; ok2 and ok4 whether
+// those were frequency moves.  Offsets stay inside the pair region and its pads
+// whatever the table holds: o0 is clamped by the caller, the second gather lies
+// within two rows of it (kPairPad bytes before and after the region).
+constexpr int kPairPad = 32;
+
+__device__ __forceinline__ Pair load_pair(const Pair* base, uint32_t offset, int shift) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(base) + offset + shift));
+    return Pair{v.x, v.y, v.z, v.w};
+}
+
+__device__ __forceinline__ void walk_four(const Pair* base, const uint4& r, uint32_t o0, uint32_t& o2, uint32_t& o4,
+                                          bool& ok2, bool& ok4) {
+    const Pair a = load_pair(base, o0, 0);
+    const bool d0 = r.x >= a.z;
+    const bool d1 = r.y >= (d0 ? a.p1 : a.m1);
+    o2 = o0;
+    if (d0) o2 += 32u;
+    if (d1) o2 += 32u;
+    const Pair b = load_pair(base, o2, -32);
+    const bool d2 = r.z >= b.z;
+    const bool d3 = r.w >= (d2 ? b.p1 : b.m1);
+    o4 = o2;
+    if (d2) o4 += 32u;
+    if (d3) o4 += 32u;
+    ok2 = max(r.x, r.y) < a.guard;
+    ok4 = ok2 && max(r.z, r.w) < b.guard;
+}
+
+// Consecutive transition blocks of one packet for a fixed high word of the
+// block index: Philox4x32-10 of (b, b_hi, p_lo, p_hi) with what the first three
+// rounds owe to the packet and b_hi alone computed once, and the first product
+// of the block index carried from block to block as a sum.  Three of the twenty
+// 32x32->64 products and three of the xors leave the loop that way (a wide
+// product takes the multiply pipe twice as long as any other instruction takes
+// its pipe, and that pipe is what the loop saturates).  K: a kernel's
+// parameter block with the round keys rk0[10], rk1[10], read from the constant
+// bank at fixed offsets (through a pointer they would be copied to local memory).
+struct TransitionStream {
+    uint32_t e0, e1, e2, e3;
+    unsigned long long w0;  // first product of the next block
+
+    template <class K>
+    __device__ __forceinline__ void init(uint32_t b, uint32_t b_hi, uint32_t p_lo, uint32_t p_hi, const K& P) {
+        const unsigned long long w1 = wide(0xCD9E8D57u, p_lo);
+        const unsigned long long w2 = wide(0xD2511F53u, hi(w1) ^ b_hi ^ P.rk0[0]);
+        e0 = p_hi ^ P.rk1[0];
+        e1 = lo(w1) ^ P.rk0[1];
+        e2 = hi(w2) ^ P.rk1[1];
+        e3 = lo(w2) ^ P.rk1[2];
+        w0 = wide(0xD2511F53u, b);
+    }
+
+    template <class K>
+    __device__ __forceinline__ uint4 next(const K& P) {
+        const unsigned long long w1 = wide(0xCD9E8D57u, hi(w0) ^ e0);
+        const unsigned long long w2 = wide(0xD2511F53u, hi(w1) ^ e1), w3 = wide(0xCD9E8D57u, lo(w0) ^ e2);
+        w0 += 0xD2511F53u;
+        uint4 c = make_uint4(hi(w3) ^ lo(w1) ^ P.rk0[2], lo(w3), hi(w2) ^ e3, lo(w2));
+#pragma unroll
+        for (int r = 3; r < 10; ++r) {
+            const unsigned long long a0 = wide(0xD2511F53u, c.x), a1 = wide(0xCD9E8D57u, c.z);
+            c = make_uint4(hi(a1) ^ c.y ^ P.rk0[r], lo(a1), hi(a0) ^ c.w ^ P.rk1[r], lo(a0));
+        }
+        return c;
+    }
+
+private:
+    static __device__ __forceinline__ unsigned long long wide(uint32_t a, uint32_t b) {
+        unsigned long long r;
+        asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+        return r;
+    }
+    static __device__ __forceinline__ uint32_t hi(unsigned long long v) { return (uint32_t)(v >> 32); }
+    static __device__ __forceinline__ uint32_t lo(unsigned long long v) { return (uint32_t)v; }
+};
+
+}  // namespace rddmc

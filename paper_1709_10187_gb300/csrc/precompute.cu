@@ -15,6 +15,7 @@
 #include <cstring>
 
 #include "grid.h"
+#include "pairs.cuh"
 #include "voigt.cuh"
 
 namespace rddmc {
@@ -126,6 +127,23 @@ __global__ void rows_kernel(const TableHeader h, const ClassDesc* __restrict__ c
     }
 }
 
+// The walk's pair of each row (pairs.cuh) from the fast heads of the three rows
+// around it in its class block.
+__global__ void pair_kernel(const uint2* __restrict__ fast, Pair* __restrict__ pair, int J, int64_t nrow) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= nrow) return;
+    const int j = (int)(r % J);
+    uint32_t t[3], guard = 0xffffffffu;
+#pragma unroll
+    for (int i = -1; i <= 1; ++i) {
+        const bool in = j + i >= 0 && j + i < J;
+        const uint2 f = in ? fast[r + i] : make_uint2(0u, 0xffffffffu);
+        t[i + 1] = f.x;
+        guard = min(guard, f.y);
+    }
+    pair[r] = Pair{t[0], t[1], t[2], guard};
+}
+
 // Split points (u1, u0) of the three-part rejection envelope of the parallel
 // atom velocity, f(u) = e^{-u^2} / (a^2 + (x-u)^2) (Sec. 5.2), for |x| = i/16:
 //   u < u1: e^{-u^2} g(u1);  u1 <= u <= u0: c g(u), c = max e^{-u^2} on [u1,u0];
@@ -192,6 +210,10 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
         rows_kernel<3><<<(unsigned)blocks, threads, 0, s>>>(h, cd, edges, phi, rows, fast, tau_row, rk, abs_thr,
                                                             dusty, wq, ka_row, weighted, nrow);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (g.pairs()) {
+        pair_kernel<<<(unsigned)((nrow + 255) / 256), 256, 0, s>>>(fast, (Pair*)(base + g.off_pair), g.J, nrow);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     // the u_par envelope table serves only the continuous MC of the hybrid scheme
     if (g.params.mode == RDDMC_MODE_HYBRID)
         upar_kernel<<<(kUparN + 127) / 128, 128, 0, s>>>((float2*)(base + g.off_upar), g.a);

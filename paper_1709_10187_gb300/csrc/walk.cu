@@ -8,11 +8,15 @@
 // o = #{k : w >= thr_k} of the state's row: the categorical form of the
 // competing exponentials of eq. l_min_1/2.
 //
-// Frequency moves dominate (the core of the line, Sec. 4.2), so the fast path
-// reads only the state's 8-byte fast head {thr0, thr1 or 0} (through L1, or
-// staged in shared memory): when w < thr1 the packet moves one bin down
-// (w < thr0) or up.  A group of four transitions runs as one branch-free chain
-// of head loads, checked at its end.
+// Frequency moves dominate (the core of the line, Sec. 4.2).  Where the table
+// has pairs (pairs.cuh: up to kPairRows rows), two transitions are one 16-byte
+// gather and two compares: a group of four is two dependent gathers instead of
+// four, checked at its end, and a transition whose word reaches its pair's
+// guard is taken row by row with the rest of its group, plain moves (frequency
+// or spatial) in a short step and other outcomes in the generic one.  Larger
+// tables and the dust weight method read the 8-byte fast heads {thr0, thr1 or
+// 0}: four transitions run as a chain of head loads (w < thr1: one bin down
+// when w < thr0, else up).
 // Everything else -- spatial moves, Doppler rebins, escapes through exterior
 // faces, and frequency outcomes that are not plain moves (their head holds 0)
 // -- goes through one generic step that reads the full row (through L1) and
@@ -39,8 +43,13 @@ namespace {
 // weight method: -ln(1e-10) in 2^-40 units, the elimination weight of Sec. 2.6
 constexpr unsigned long long kLwMin = 25317190836906ull;
 
+// Resident 256-thread CTAs per SM the register budget targets.  Three (80
+// registers) keep the pair loop's two blocks of words and its stream constants
+// in registers; four (64) spill them: 27.7 against 28.2 ms on two 4096-step
+// slices of 4e6 packets (256 x 512 slab), 0.56 against 0.67 s on 1e5 packets of
+// the 64 x 128 slab to escape, 46 against 53 ms on the 32^3 clumpy medium.
 #ifndef RDDMC_WALK_MIN_BLOCKS
-#define RDDMC_WALK_MIN_BLOCKS 4  // resident 256-thread CTAs per SM the register budget targets
+#define RDDMC_WALK_MIN_BLOCKS 3
 #endif
 
 // ---------------------------------------------------------------- hybrid MC
@@ -293,16 +302,43 @@ __device__ __forceinline__ bool prop_takes(const WalkParams& P, unsigned cell, u
     return l >= P.prop_llo && l <= P.prop_lhi;
 }
 
-template <int NDIM, bool SMEM_ROWS, bool HYBRID, bool PROPOSE, bool WEIGHT>
-__global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const WalkParams P) {
+// Per-thread counters in shared memory.
+enum Loc64 { L_STEPS = 0, L_EDRAW = 1, L_MC = 2, kLoc64 = 3 };
+enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6 };
+
+// How a kernel instantiation reads frequency moves: fast heads through L1 or
+// from shared memory, or pairs through L1.
+enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2 };
+
+// What bounds it: dispatch.  A Philox block costs 17 wide products (3.65 cycles
+// of the multiply pipe each) and 19 xors, measured at 81 cycles per warp and
+// scheduler alone; the choice and its bookkeeping add about 50.  Pairs took the
+// four dependent 8-byte gathers of a group, which held the L1 at its random
+// gather rate, down to two.  __grid_constant__: the escape functions take the
+// parameter block's address, and without it every read of P went to a local
+// copy (9 local loads per group).  Two 4096-step slices of 4e6 packets on the
+// 256 x 512 slab: 32.5 ms with heads, 27.7 ms.
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
+__global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const __grid_constant__ WalkParams P) {
     constexpr int RW = NDIM == 1 ? 1 : 2;  // uint4 per row
+    constexpr bool SMEM_ROWS = PATH == HEADS_SMEM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long* s_cnt = reinterpret_cast<unsigned long long*>(smem_raw);  // kCounters
     unsigned long long* s_face = s_cnt + kCounters;                              // 8
     unsigned long long* s_sb = s_face + 8;                                        // kNsb
     unsigned long long* s_hist = s_sb + kNsb;                                     // J+2 if in smem
     const int nhist = P.J + 2;
-    uint2* s_fast = reinterpret_cast<uint2*>(s_hist + (P.hist_in_smem ? ((nhist + 1) & ~1) : 0));
+    // this thread's counters: touched once per packet or event, so they live in
+    // shared memory and leave their registers to the transition loop
+    unsigned long long* loc64 = s_hist + (P.hist_in_smem ? ((nhist + 1) & ~1) : 0) + threadIdx.x;
+    unsigned* loc32 = reinterpret_cast<unsigned*>(loc64 - threadIdx.x + kLoc64 * blockDim.x) + threadIdx.x;
+    uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + kLoc32 * blockDim.x);
+    auto cnt64 = [&](int i) -> unsigned long long& { return loc64[i * blockDim.x]; };
+    auto cnt32 = [&](int i) -> unsigned& { return loc32[i * blockDim.x]; };
+#pragma unroll
+    for (int i = 0; i < kLoc64; ++i) cnt64(i) = 0ull;
+#pragma unroll
+    for (int i = 0; i < kLoc32; ++i) cnt32(i) = 0u;
 
     for (int i = threadIdx.x; i < kCounters + 8 + kNsb; i += blockDim.x) s_cnt[i] = 0ull;
     if (P.hist_in_smem)
@@ -316,13 +352,33 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
     const unsigned lane = threadIdx.x & 31u;
     const unsigned J = (unsigned)P.J;
     const unsigned nr1 = (unsigned)P.n_rows - 1u;
+    const uint32_t omax = 16u * nr1;  // the last row's pair
     const unsigned long long t_begin = P.time_slice_ns ? global_ns() : 0ull;
     bool have = false, exhausted = false;
     unsigned long long pid = 0, t = 0, e = 0, t_stop = 0;
     unsigned long long lw = 0;  // weight method: -ln(packet weight) in 2^-40 units
     unsigned cell = 0, cls = 0, s = 0;  // s = cls * J + bin: the row of the state
-    unsigned long long n_steps = 0, n_edraw = 0, n_mc = 0;
-    unsigned n_emit = 0, n_esc = 0, n_abort = 0, n_clamp = 0, status_bits = 0, n_conv = 0;
+
+    // A packet's transitions and event draws in this launch: its counters when
+    // the lane lets it go less those it came with (a new packet's are 0, and
+    // its source draw counts).
+    auto take = [&]() {
+        cnt64(L_STEPS) -= t;
+        cnt64(L_EDRAW) -= e;
+    };
+    auto release = [&]() {
+        cnt64(L_STEPS) += t;
+        cnt64(L_EDRAW) += e;
+        have = false;
+    };
+    auto excursion = [&](unsigned bin, int face) -> McResult {
+        unsigned long long n_mc = 0;
+        unsigned n_conv = 0;
+        const McResult res = mc_excursion<NDIM>(P, cell, bin, face, pid, e, n_mc, n_conv);
+        cnt64(L_MC) += n_mc;
+        cnt32(L_CONV) += n_conv;
+        return res;
+    };
 
     // Outcome of an MC excursion: back to DDMC (returns false) or finished.
     auto after_mc = [&](const McResult& res) -> bool {
@@ -337,10 +393,10 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             else atomicAdd(&P.tally[kHistOff + res.hist], 1ull);
             if (res.sb >= 0) smem_tally(s_sb, (unsigned)res.sb);
             smem_tally(s_face, (unsigned)res.face);
-            ++n_esc;
+            ++cnt32(L_ESC);
             return true;
         }
-        ++n_abort;
+        ++cnt32(L_ABORT);
         return true;
     };
 
@@ -376,10 +432,9 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         if (o < 2u) {
             if (act == ACT_MOVE) { s += o ? 1u : 0xffffffffu; return faded(); }
             if (HYBRID && act == ACT_TO_MC)  // leak into a thin bin of this cell
-                return after_mc(mc_excursion<NDIM>(P, cell, o ? min(bin + 1u, J - 1u) : (bin ? bin - 1u : 0u), -1,
-                                                   pid, e, n_mc, n_conv));
-            status_bits |= (unsigned)STATUS_UNSUPPORTED_EVENT;
-            ++n_abort;
+                return after_mc(excursion(o ? min(bin + 1u, J - 1u) : (bin ? bin - 1u : 0u), -1));
+            cnt32(L_STATUS) |= (unsigned)STATUS_UNSUPPORTED_EVENT;
+            ++cnt32(L_ABORT);
             return true;
         }
         const unsigned face = o - 2u;
@@ -400,14 +455,14 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                 atomicAdd(&P.tally[P.hist_off_w], ww);
                 atomicAdd(&P.tally[P.hist_off_w + 1 + eb.hist], ww);
             }
-            ++n_esc;
+            ++cnt32(L_ESC);
             return true;
         }
         if (act == ACT_TO_MC) {
             if (HYBRID)  // leak into a thin neighbour cell
-                return after_mc(mc_excursion<NDIM>(P, cell, bin, (int)face, pid, e, n_mc, n_conv));
-            status_bits |= (unsigned)STATUS_UNSUPPORTED_EVENT;
-            ++n_abort;
+                return after_mc(excursion(bin, (int)face));
+            cnt32(L_STATUS) |= (unsigned)STATUS_UNSUPPORTED_EVENT;
+            ++cnt32(L_ABORT);
             return true;
         }
         unsigned nbin = bin;
@@ -415,8 +470,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             const Rebin rb = P.rebin[min(cls, (unsigned)P.n_class - 1u) * (2u * NDIM) + face];
             const unsigned w1 = event_word(pid, e++, P.k0, P.k1);
             int jn = (int)bin + rb.m + (w1 >= rb.thr ? 1 : 0);
-            if (jn < 0) { jn = 0; ++n_clamp; }
-            if (jn > (int)J - 1) { jn = (int)J - 1; ++n_clamp; }
+            if (jn < 0) { jn = 0; ++cnt32(L_CLAMP); }
+            if (jn > (int)J - 1) { jn = (int)J - 1; ++cnt32(L_CLAMP); }
             nbin = (unsigned)jn;
         }
         const unsigned ax = face >> 1;
@@ -425,6 +480,39 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         cls = __ldg(&P.cell_class[cell]);
         s = cls * J + nbin;
         return faded();
+    };
+
+    // The transitions q .. 3 of words r, row by row: a plain move (frequency or
+    // spatial) in place, any other outcome through the generic step.  Returns 4,
+    // or the index of the transition that finished the packet.
+    auto by_rows = [&](const uint4& r, unsigned q) -> unsigned {
+        do {
+            const unsigned w = word_of(r, q);
+            const unsigned ri = min(s, nr1);
+            const uint4 a = __ldg(&rows[ri * RW]);
+            unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
+            if (NDIM == 3) {
+                const uint4 b = __ldg(&rows[ri * RW + 1]);
+                o += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
+            }
+            const bool plain = ((a.w >> (2u * o)) & 3u) == ACT_MOVE && !(P.dust && o == 2u * NDIM + 1u);
+            if (plain) {
+                if (o < 2u) {
+                    s += o ? 1u : 0xffffffffu;
+                } else {
+                    const unsigned ax = (o - 2u) >> 1;
+                    const unsigned stride =
+                        NDIM == 1 ? 1u : (ax == 0 ? 1u : (ax == 1 ? (unsigned)P.n0 : (unsigned)P.n01));
+                    cell = min((o & 1u) ? cell + stride : cell - stride, (unsigned)P.ncell - 1u);
+                    const unsigned c1 = __ldg(&P.cell_class[cell]);
+                    s += (c1 - cls) * J;
+                    cls = c1;
+                }
+            } else if (generic(w)) {
+                return q;
+            }
+        } while (++q < 4u);
+        return 4u;
     };
 
     for (;;) {
@@ -448,6 +536,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                         t = P.st_t[pid];
                         e = P.st_e[pid];
                         if (WEIGHT) lw = P.st_lw[pid];
+                        take();
                         have = true;
                     } else if (st == PK_FRESH) {
                         // event draw 0: bit 31-a picks the centre cell on axis a, bit 28 the bin
@@ -461,7 +550,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                         t = 0;
                         e = 1;
                         lw = 0;
-                        ++n_emit;
+                        ++cnt32(L_EMIT);
                         have = true;
                     }
                     if (have) {
@@ -473,11 +562,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                             // a thin source state starts as MC
                             const uint4 a0 = __ldg(&rows[min(s, nr1) * RW]);
                             if (a0.w & FLAG_THIN) {
-                                const unsigned long long e0 = e;
-                                const McResult res = mc_excursion<NDIM>(P, cell, min(bin, J - 1u), -1, pid, e, n_mc,
-                                                                        n_conv);
-                                n_edraw += e - e0;
-                                if (after_mc(res)) have = false;
+                                if (after_mc(excursion(min(bin, J - 1u), -1))) release();
                             }
                         }
                     }
@@ -494,7 +579,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             P.st_e[pid] = e;
             if (WEIGHT) P.st_lw[pid] = lw;
             P.st_status[pid] = PK_INFLIGHT;
-            have = false;
+            release();
             exhausted = true;
             continue;
         }
@@ -515,7 +600,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             k0q = __shfl_sync(grp, k0q, lead);
             const unsigned long long k = k0q + (unsigned long long)__popc(grp & ((1u << lane) - 1u));
             P.prop_qpid[min(k, P.n_packets - 1ull)] = pid;
-            have = false;
+            release();
             continue;
         }
 
@@ -525,78 +610,118 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                                          : t + (unsigned long long)P.chunk;
         lim = lim < t_stop ? lim : t_stop;
         lim = lim < P.max_steps ? lim : P.max_steps;
-        const unsigned long long t0 = t;
-        const unsigned long long e0 = e;
         bool fin = false;
         {
             const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
             unsigned long long blk = t >> 2;
             const unsigned ng = (unsigned)((lim - t) >> 2);  // full groups of four
-            uint4 rn = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
-            unsigned g = 0;
-            while (g < ng) {
-                const uint4 r = rn;
-                ++blk;
-                rn = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
-                unsigned q;
+            if constexpr (PATH == PAIRS) {
+                const unsigned long long blk_end = blk + ng;
+                while (blk < blk_end) {  // one pass, or two when the block index crosses a multiple of 2^32
+                    const uint32_t bh = (uint32_t)(blk >> 32);
+                    const unsigned long long wrap = ((unsigned long long)bh + 1ull) << 32;
+                    unsigned left = (unsigned)((blk_end < wrap ? blk_end : wrap) - blk);
+                    blk += left;
+                    TransitionStream ts;
+                    ts.init((uint32_t)blk - left, bh, pl, ph, P);
+                    uint4 ra = ts.next(P), rb;
+                    uint32_t o = 16u * s;
+                    // one group of four on r while the next block is drawn into rn;
+                    // true when the packet finished
+                    auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
+                        uint32_t o2, o4;
+                        bool ok2, ok4;
+                        walk_four(P.pair, r, o, o2, o4, ok2, ok4);
+                        rn = ts.next(P);
+                        if (ok4) {
+                            o = min(o4 - 64u, omax);
+                            return false;
+                        }
+                        s = (ok2 ? o2 - 32u : o) >> 4;
+                        const unsigned q = by_rows(r, ok2 ? 2u : 0u);
+                        o = min(16u * s, omax);
+                        t = 4ull * (blk - behind) + q + 1ull;
+                        return q < 4u;
+                    };
+                    // two groups per pass, the blocks changing places: no register
+                    // moves and one loop test per eight transitions
+                    if (left & 1u) {
+                        if (group(ra, rb, left)) { fin = true; goto chunk_done; }
+                        ra = rb;
+                    }
+                    for (left &= ~1u; left; left -= 2u) {
+                        if (group(ra, rb, left) || group(rb, ra, left - 1u)) { fin = true; goto chunk_done; }
+                    }
+                    s = o >> 4;
+                }
+                t = 4ull * blk;
+            } else {
+                uint4 rn = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
+                unsigned g = 0;
+                while (g < ng) {
+                    const uint4 r = rn;
+                    ++blk;
+                    rn = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
+                    unsigned q;
 #define RDDMC_FAST(W, Q)                                                                  \
-    {                                                                                     \
-        const uint2 f_ = SMEM_ROWS ? fast[min(s, nr1)] : __ldg(&fast[min(s, nr1)]);       \
-        const unsigned long long wq_ = WEIGHT ? __ldg(&P.wq[min(s, nr1)]) : 0ull;         \
-        if ((W) < f_.y && (!WEIGHT || lw + wq_ <= kLwMin)) {                              \
-            if (WEIGHT) lw += wq_;                                                        \
-            s += ((W) >= f_.x) ? 1u : 0xffffffffu;                                        \
-        } else {                                                                          \
-            q = (Q);                                                                      \
-            goto slow;                                                                    \
-        }                                                                                 \
-    }
-                if (!WEIGHT) {
-                    // The group's four transitions as one branch-free chain: each
-                    // head is loaded at the state the previous transition would
-                    // reach by a frequency move (index clamped, so a speculative
-                    // state past a non-move stays in bounds), then the chain is
-                    // checked.  With no branch between the loads the scheduler
-                    // fills their latency with the next group's Philox rounds.
-                    const unsigned s0 = s;
-                    const uint2 f0 = SMEM_ROWS ? fast[min(s0, nr1)] : __ldg(&fast[min(s0, nr1)]);
-                    const unsigned s1 = s0 + ((r.x >= f0.x) ? 1u : 0xffffffffu);
-                    const uint2 f1 = SMEM_ROWS ? fast[min(s1, nr1)] : __ldg(&fast[min(s1, nr1)]);
-                    const unsigned s2 = s1 + ((r.y >= f1.x) ? 1u : 0xffffffffu);
-                    const uint2 f2 = SMEM_ROWS ? fast[min(s2, nr1)] : __ldg(&fast[min(s2, nr1)]);
-                    const unsigned s3 = s2 + ((r.z >= f2.x) ? 1u : 0xffffffffu);
-                    const uint2 f3 = SMEM_ROWS ? fast[min(s3, nr1)] : __ldg(&fast[min(s3, nr1)]);
-                    const unsigned s4 = s3 + ((r.w >= f3.x) ? 1u : 0xffffffffu);
-                    const bool ok0 = r.x < f0.y, ok1 = r.y < f1.y, ok2 = r.z < f2.y, ok3 = r.w < f3.y;
-                    if (ok0 && ok1 && ok2 && ok3) {
-                        s = s4;
-                        ++g;
-                        continue;
+        {                                                                                     \
+            const uint2 f_ = SMEM_ROWS ? fast[min(s, nr1)] : __ldg(&fast[min(s, nr1)]);       \
+            const unsigned long long wq_ = WEIGHT ? __ldg(&P.wq[min(s, nr1)]) : 0ull;         \
+            if ((W) < f_.y && (!WEIGHT || lw + wq_ <= kLwMin)) {                              \
+                if (WEIGHT) lw += wq_;                                                        \
+                s += ((W) >= f_.x) ? 1u : 0xffffffffu;                                        \
+            } else {                                                                          \
+                q = (Q);                                                                      \
+                goto slow;                                                                    \
+            }                                                                                 \
+        }
+                    if (!WEIGHT) {
+                        // The group's four transitions as one branch-free chain: each
+                        // head is loaded at the state the previous transition would
+                        // reach by a frequency move (index clamped, so a speculative
+                        // state past a non-move stays in bounds), then the chain is
+                        // checked.  With no branch between the loads the scheduler
+                        // fills their latency with the next group's Philox rounds.
+                        const unsigned s0 = s;
+                        const uint2 f0 = SMEM_ROWS ? fast[min(s0, nr1)] : __ldg(&fast[min(s0, nr1)]);
+                        const unsigned s1 = s0 + ((r.x >= f0.x) ? 1u : 0xffffffffu);
+                        const uint2 f1 = SMEM_ROWS ? fast[min(s1, nr1)] : __ldg(&fast[min(s1, nr1)]);
+                        const unsigned s2 = s1 + ((r.y >= f1.x) ? 1u : 0xffffffffu);
+                        const uint2 f2 = SMEM_ROWS ? fast[min(s2, nr1)] : __ldg(&fast[min(s2, nr1)]);
+                        const unsigned s3 = s2 + ((r.z >= f2.x) ? 1u : 0xffffffffu);
+                        const uint2 f3 = SMEM_ROWS ? fast[min(s3, nr1)] : __ldg(&fast[min(s3, nr1)]);
+                        const unsigned s4 = s3 + ((r.w >= f3.x) ? 1u : 0xffffffffu);
+                        const bool ok0 = r.x < f0.y, ok1 = r.y < f1.y, ok2 = r.z < f2.y, ok3 = r.w < f3.y;
+                        if (ok0 && ok1 && ok2 && ok3) {
+                            s = s4;
+                            ++g;
+                            continue;
+                        }
+                        // the first transition that is not a plain frequency move
+                        // takes the generic step from the state before it
+                        q = !ok0 ? 0u : (!ok1 ? 1u : (!ok2 ? 2u : 3u));
+                        s = !ok0 ? s0 : (!ok1 ? s1 : (!ok2 ? s2 : s3));
+                        goto slow;
                     }
-                    // the first transition that is not a plain frequency move
-                    // takes the generic step from the state before it
-                    q = !ok0 ? 0u : (!ok1 ? 1u : (!ok2 ? 2u : 3u));
-                    s = !ok0 ? s0 : (!ok1 ? s1 : (!ok2 ? s2 : s3));
-                    goto slow;
-                }
-                RDDMC_FAST(r.x, 0u)
-                RDDMC_FAST(r.y, 1u)
-                RDDMC_FAST(r.z, 2u)
-                RDDMC_FAST(r.w, 3u)
+                    RDDMC_FAST(r.x, 0u)
+                    RDDMC_FAST(r.y, 1u)
+                    RDDMC_FAST(r.z, 2u)
+                    RDDMC_FAST(r.w, 3u)
 #undef RDDMC_FAST
-                ++g;
-                continue;
-            slow:
-                for (; q < 4u; ++q) {
-                    if (generic(word_of(r, q))) {
-                        fin = true;
-                        t += 4ull * g + q + 1ull;
-                        goto chunk_done;
+                    ++g;
+                    continue;
+                slow:
+                    for (; q < 4u; ++q) {
+                        if (generic(word_of(r, q))) {
+                            fin = true;
+                            t += 4ull * g + q + 1ull;
+                            goto chunk_done;
+                        }
                     }
+                    ++g;
                 }
-                ++g;
+                t += 4ull * ng;
             }
-            t += 4ull * ng;
             // at most three transitions left before the watchdog limit
             while (t < lim) {
                 const unsigned long long b = t >> 2;
@@ -607,14 +732,12 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             }
         }
     chunk_done:
-        n_steps += t - t0;
-        n_edraw += e - e0;
         if (fin) {
-            have = false;
+            release();
             if (P.save_state) P.st_status[pid] = PK_DONE;
         } else if (t >= P.max_steps) {
-            ++n_abort;
-            have = false;
+            ++cnt32(L_ABORT);
+            release();
             if (P.save_state) P.st_status[pid] = PK_DONE;
         } else if (t >= t_stop) {
             P.st_cell[pid] = cell;
@@ -623,13 +746,13 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             P.st_e[pid] = e;
             if (WEIGHT) P.st_lw[pid] = lw;
             P.st_status[pid] = PK_INFLIGHT;
-            have = false;
+            release();
         }
     }
 
     // ---- flush: warp sums of the per-thread counters, then CTA totals to HBM
-    n_edraw += n_emit;  // the source draw of each emitted packet
-    unsigned long long v[9] = {n_emit, n_esc, n_abort, n_steps, n_clamp, n_edraw, status_bits, n_mc, n_conv};
+    unsigned long long v[9] = {cnt32(L_EMIT),  cnt32(L_ESC),   cnt32(L_ABORT),  cnt64(L_STEPS), cnt32(L_CLAMP),
+                               cnt64(L_EDRAW), cnt32(L_STATUS), cnt64(L_MC),    cnt32(L_CONV)};
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         unsigned long long x = v[i];
@@ -663,27 +786,38 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         if (s_sb[i]) atomicAdd(&P.tally[kHistOff + nhist + i], s_sb[i]);
 }
 
-template <int NDIM, bool SMEM, bool HYBRID, bool PROPOSE, bool WEIGHT>
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
 cudaError_t launch_variant(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<NDIM, SMEM, HYBRID, PROPOSE, WEIGHT>,
+    cudaError_t e = cudaFuncSetAttribute(walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (!ctas) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, walk_kernel<NDIM, SMEM, HYBRID, PROPOSE, WEIGHT>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>,
                                                           threads, smem);
         if (e != cudaSuccess) return e;
     }
     if (ctas < 1) ctas = 1;
-    walk_kernel<NDIM, SMEM, HYBRID, PROPOSE, WEIGHT><<<(unsigned)(ctas * nsm), threads, smem, s>>>(P);
+    walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT><<<(unsigned)(ctas * nsm), threads, smem, s>>>(P);
     return cudaGetLastError();
 }
 
-template <int NDIM, bool SMEM>
-cudaError_t launch_mode(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
-    if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, SMEM, false, true, false>(P, threads, smem, ctas, nsm, s);
-    if (P.weights) return launch_variant<NDIM, SMEM, false, false, true>(P, threads, smem, ctas, nsm, s);
-    return P.hybrid ? launch_variant<NDIM, SMEM, true, false, false>(P, threads, smem, ctas, nsm, s)
-                    : launch_variant<NDIM, SMEM, false, false, false>(P, threads, smem, ctas, nsm, s);
+template <int NDIM, int PATH>
+cudaError_t launch_path(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
+    if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, threads, smem, ctas, nsm, s);
+    return P.hybrid ? launch_variant<NDIM, PATH, true, false, false>(P, threads, smem, ctas, nsm, s)
+                    : launch_variant<NDIM, PATH, false, false, false>(P, threads, smem, ctas, nsm, s);
+}
+
+// Pairs where the table has them, heads otherwise; the weight method reads
+// heads (its weight is checked before every transition).
+template <int NDIM>
+cudaError_t launch_mode(const WalkParams& P, bool smem_heads, int threads, size_t smem, int ctas, int nsm,
+                        cudaStream_t s) {
+    if (P.weights)
+        return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, threads, smem, ctas, nsm, s)
+                          : launch_variant<NDIM, HEADS, false, false, true>(P, threads, smem, ctas, nsm, s);
+    return P.pair ? launch_path<NDIM, PAIRS>(P, threads, smem, ctas, nsm, s)
+                 : launch_path<NDIM, HEADS>(P, threads, smem, ctas, nsm, s);
 }
 
 // One scattering per thread at x_in with incoming direction +e_z; sample i
@@ -734,7 +868,7 @@ __device__ __forceinline__ void fold_parked(const WalkParams& P, unsigned cell, 
 // Network inputs of queued packets q0 .. q0+cnt (rows past cnt are zeroed).
 // Negative frequencies are mirrored: a static uniform brick is symmetric under
 // x -> -x and the network was trained on x >= 0.
-__global__ void propose_features_kernel(const WalkParams P, const float* __restrict__ xc, FeatConst fc,
+__global__ void propose_features_kernel(const __grid_constant__ WalkParams P, const float* __restrict__ xc, FeatConst fc,
                                         unsigned long long q0, unsigned long long cnt, int batch,
                                         __nv_bfloat16* __restrict__ X) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -803,7 +937,7 @@ __device__ __forceinline__ int softmax_draw_warp(const float* __restrict__ z, in
 // head C's slice of that face when nC > 0, else two uniform coordinates --
 // then lane 0 makes the crossing with its own draws (a Doppler rebin, or the
 // five of an escape).
-__global__ void propose_place_kernel(const WalkParams P, const float* __restrict__ xc,
+__global__ void propose_place_kernel(const __grid_constant__ WalkParams P, const float* __restrict__ xc,
                                      const float* __restrict__ logits, int n_out, int nA, int nB, int nC,
                                      unsigned long long q0, unsigned long long cnt) {
     const unsigned lane = threadIdx.x & 31u;
@@ -1034,6 +1168,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     std::memset(&P, 0, sizeof(P));
     P.rows = (const uint4*)(tb + g.off_rows);
     P.fast = (const uint2*)(tb + g.off_fast);
+    P.pair = g.pairs() ? (const Pair*)(tb + g.off_pair) : nullptr;
     P.tau_row = (const float*)(tb + g.off_tau);
     P.upar = (const float2*)(tb + g.off_upar);
     P.cdesc = (const ClassDesc*)(tb + g.off_cdesc);
@@ -1134,17 +1269,15 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     const int threads = o.threads_per_cta ? o.threads_per_cta : 256;
     size_t smem = (size_t)(kCounters + 8 + kNsb) * 8;
     if (P.hist_in_smem) smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
+    smem += (size_t)threads * (kLoc64 * 8 + kLoc32 * 4);
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads
-    const bool use_smem_rows = o.table_in_smem && smem + rows_bytes <= (size_t)smem_optin;
-    if (use_smem_rows) smem += rows_bytes;
+    const bool smem_heads = P.weights && o.table_in_smem && smem + rows_bytes <= (size_t)smem_optin;
+    if (smem_heads) smem += rows_bytes;
     if ((e = cudaMemsetAsync(P.cursor, 0, 8, s)) != cudaSuccess) return e;
     if (P.save_state && !o.resume && (e = cudaMemsetAsync(P.st_status, PK_FRESH, o.n_packets, s)) != cudaSuccess)
         return e;
-    if (g.ndim == 1)
-        return use_smem_rows ? launch_mode<1, true>(P, threads, smem, o.ctas_per_sm, nsm, s)
-                             : launch_mode<1, false>(P, threads, smem, o.ctas_per_sm, nsm, s);
-    return use_smem_rows ? launch_mode<3, true>(P, threads, smem, o.ctas_per_sm, nsm, s)
-                         : launch_mode<3, false>(P, threads, smem, o.ctas_per_sm, nsm, s);
+    return g.ndim == 1 ? launch_mode<1>(P, smem_heads, threads, smem, o.ctas_per_sm, nsm, s)
+                       : launch_mode<3>(P, smem_heads, threads, smem, o.ctas_per_sm, nsm, s);
 }
 
 }  // namespace rddmc

@@ -6,6 +6,7 @@
 
 #include "escape.cuh"
 #include "grid.h"
+#include "pairs.cuh"
 
 namespace rddmc {
 
@@ -15,6 +16,7 @@ constexpr int kSmemHistMax = 8192;  // histogram entries kept in shared memory
 struct WalkParams {
     const uint4* rows;
     const uint2* fast;
+    const Pair* pair;         // two frequency moves per gather (null for large tables)
     const float* tau_row;     // tau_ij = k_ij dz per row (hybrid conversions)
     const float2* upar;       // u_par envelope split points
     const ClassDesc* cdesc;

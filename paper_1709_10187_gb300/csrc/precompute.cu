@@ -1,7 +1,11 @@
 // precompute.cu -- FP64 leakage-table kernels (Sec. 2.2, Sec. 2.5, Sec. 5.1).
 //
-// Kernel 1: phi[j] = bin mean of H(a,x) over bin j (k_ij = k0_i phi_j).
-// Kernel 2: one thread per (class, bin) row: leakage coefficients of
+// Kernel 1: phi[j] = bin mean of H(a,x) over bin j (k_ij = k0_i phi_j).  Half a
+// warp sums one edge's Dawson series, a lane per term, in the series' order.
+// Kernel 2, a thread per (class, bin) row; on a moving grid a block per class
+// and 127 of its rows, each thread first taking one bin edge, shifted by every
+// face's velocity difference in turn (faces with the same shift once), then its
+// row: leakage coefficients of
 //   eq. x-leakage and eq. z-leakage, the boundary / thin-neighbour form
 //   2/(3 dz (k dz + 2 lambda)), probabilities p_X = k_X / sum k accumulated in
 //   outcome order, 32-bit thresholds round-half-even(C 2^32) saturated at
@@ -21,10 +25,31 @@
 namespace rddmc {
 namespace {
 
-__global__ void phi_kernel(const double* __restrict__ edges, double* __restrict__ phi, int J, double a) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= J) return;
-    phi[j] = voigt_bin_mean_f64(a, edges[j], edges[j + 1]);
+constexpr int kPhiEdges = 32;   // bin edges of a phi block (half a warp each)
+constexpr int kRowEdges = 128;  // bin edges of a rows block (a thread each)
+
+// Latency of one exponential, one division and the ordered sum of 16 terms, for
+// any J: 52 us cold where a thread per bin, two series of 34 terms in a row, took
+// 167-188 us.
+__global__ void __launch_bounds__(kPhiEdges * 16) phi_kernel(const double* __restrict__ edges,
+                                                             double* __restrict__ phi, int J, double a) {
+    __shared__ VoigtEdge s_edge[kPhiEdges];
+    static_assert(kDawsonTerms == 16, "a lane per term");
+    const int j0 = (int)blockIdx.x * (kPhiEdges - 1), k = (int)threadIdx.x >> 4, i = (int)threadIdx.x & 15;
+    const double x = edges[min(j0 + k, J)], ax = fabs(x);
+    double F;
+    if (ax < 0.5) {
+        F = dawson_series_f64(ax);
+    } else {
+        F = DawsonCentre(ax).term(i);
+    }
+    double sum = 0.0;
+    for (int q = 15; q >= 0; --q) sum += __shfl_sync(0xffffffffu, F, q, 16);
+    if (ax >= 0.5) F = sum * kInvSqrtPi;
+    if (i == 0) s_edge[k] = voigt_edge(x, x < 0.0 ? -F : F);
+    __syncthreads();
+    const int t = (int)threadIdx.x;
+    if (t < kPhiEdges - 1 && j0 + t < J) phi[j0 + t] = voigt_bin_mean_f64(a, s_edge[t], s_edge[t + 1]);
 }
 
 __device__ __forceinline__ uint32_t quantise_dev(double C) {
@@ -34,21 +59,56 @@ __device__ __forceinline__ uint32_t quantise_dev(double C) {
     return (uint32_t)t;
 }
 
-template <int NDIM>
-__global__ void rows_kernel(const TableHeader h, const ClassDesc* __restrict__ cdesc,
-                            const double* __restrict__ edges, const double* __restrict__ phi,
-                            uint32_t* __restrict__ rows, uint2* __restrict__ fast, float* __restrict__ tau_row,
-                            float* __restrict__ rk, uint32_t* __restrict__ abs_thr, int dusty,
-                            unsigned long long* __restrict__ wq, float* __restrict__ ka_row, int weighted,
-                            int64_t nrow) {
+// Bound by FP64 issue where cells move: the neighbour's opacity over the shifted
+// bin takes one Dawson series (32 exponentials and divisions) per edge and
+// distinct shift.  16^3 cells x 64 bins, every cell its own shifts: 4.7 ms (12.8 ms
+// with two series of 34 terms per row and face).
+template <int NDIM, bool MOVING>
+__global__ void __launch_bounds__(kRowEdges)
+    rows_kernel(const TableHeader h, const ClassDesc* __restrict__ cdesc, const double* __restrict__ edges,
+                const double* __restrict__ phi, uint32_t* __restrict__ rows, uint2* __restrict__ fast,
+                float* __restrict__ tau_row, float* __restrict__ rk, uint32_t* __restrict__ abs_thr, int dusty,
+                unsigned long long* __restrict__ wq, float* __restrict__ ka_row, int weighted, int tiles, int64_t nrow) {
     constexpr int K = 2 + 2 * NDIM;
     constexpr int W = NDIM == 1 ? 4 : 8;  // words per row, the last holding the flags
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrow) return;
-    const int J = h.J;
-    const int cls = (int)(r / J);
-    const int j = (int)(r - (int64_t)cls * J);
+    __shared__ VoigtEdge s_edge[MOVING ? kRowEdges : 1];
+    const int J = h.J, tid = (int)threadIdx.x;
+    const int64_t lin = (int64_t)blockIdx.x * kRowEdges + tid;
+    const int cls = MOVING ? (int)(blockIdx.x / (unsigned)tiles) : (int)(min(lin, nrow - 1) / J);
+    const int j = MOVING ? (int)(blockIdx.x % (unsigned)tiles) * (kRowEdges - 1) + tid
+                         : (int)(lin - (int64_t)cls * J);
     const ClassDesc& D = cdesc[cls];
+    // bin-mean profile over the bin shifted by each face's velocity difference
+    double phi_nb[2 * NDIM];
+    if (MOVING) {
+#pragma unroll
+        for (int f = 0; f < 2 * NDIM; ++f) {
+            const double delta = D.face[f].delta;
+            phi_nb[f] = 0.0;
+            if (D.face[f].exterior || delta == 0.0) continue;  // one class per block: uniform
+            int same = -1;
+#pragma unroll
+            for (int g = 0; g < f; ++g)
+                if (same < 0 && !D.face[g].exterior && D.face[g].delta == delta) same = g;
+            if (same >= 0) {
+#pragma unroll
+                for (int g = 0; g < f; ++g)
+                    if (g == same) phi_nb[f] = phi_nb[g];
+                continue;
+            }
+            __syncthreads();  // the last face's readers
+            if (j <= J) {
+                const double x = edges[j] + delta;
+                s_edge[tid] = voigt_edge(x, dawson_f64(x));
+            }
+            __syncthreads();
+            if (tid < kRowEdges - 1 && j < J) phi_nb[f] = voigt_bin_mean_f64(h.a, s_edge[tid], s_edge[tid + 1]);
+        }
+        if (tid == kRowEdges - 1 || j >= J) return;
+    } else if (lin >= nrow) {
+        return;
+    }
+    const int64_t r = (int64_t)cls * J + j;
     const bool hybrid = h.mode == RDDMC_MODE_HYBRID;
     double dzmin = h.dz[0];
     for (int ax = 1; ax < NDIM; ++ax) dzmin = fmin(dzmin, h.dz[ax]);
@@ -79,10 +139,7 @@ __global__ void rows_kernel(const TableHeader h, const ClassDesc* __restrict__ c
             const double r_bnd = 1.0 / (3.0 * dz) * 2.0 / (k * dz + 2.0 * h.lambda);
             if (F.exterior) { rate[o] = r_bnd; act[o] = ACT_ESCAPE; continue; }
             // neighbour opacity over the Doppler-shifted bin (eq. velocity-shift)
-            const double knb = F.k0_nb * (F.delta == 0.0 ? phi[j]
-                                                         : voigt_bin_mean_f64(h.a, edges[j] + F.delta,
-                                                                              edges[j + 1] + F.delta)) +
-                               F.ks_nb;
+            const double knb = F.k0_nb * (F.delta == 0.0 ? phi[j] : phi_nb[2 * ax + sd]) + F.ks_nb;
             const double dznb = dz;
             if (hybrid && knb * dznb < h.tau_ddmc) { rate[o] = r_bnd; act[o] = ACT_TO_MC; continue; }
             rate[o] = 1.0 / (3.0 * dz) * 2.0 / (k * dz + knb * dznb);
@@ -150,26 +207,58 @@ __global__ void pair_kernel(const uint2* __restrict__ fast, Pair* __restrict__ p
 //   u > u0: e^{-u0^2} g(u),  g(u) = 1/(a^2 + (x-u)^2),  u1 <= u0 <= x, u0 >= 0.
 // Each piece bounds f, so any such pair samples f exactly; the pair with the
 // smallest envelope mass on a grid of candidates gives the best acceptance.
-__global__ void upar_kernel(float2* __restrict__ tab, double a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kUparN) return;
+// A block per |x|: a thread takes every 128th candidate, and the block keeps the
+// first of the smallest (as one pass in order would).  0.34 ms (5.4 ms with a
+// thread per |x|).
+__global__ void __launch_bounds__(128) upar_kernel(float2* __restrict__ tab, double a) {
+    constexpr int NP = 33, NQ = 34;
+    __shared__ double s_m[128], s_th0[NP], s_m3[NP];
+    __shared__ int s_c[128];
+    const int i = (int)blockIdx.x, tid = (int)threadIdx.x;
     const double x = (double)i / 16.0;
-    double best = 1e300, b1 = -30.0, b0 = 0.0;
-    for (int p = 0; p <= 32; ++p) {
-        const double u0 = x * p / 32.0;
+    if (tid < NP) {
+        const double u0 = x * tid / 32.0;
         const double th0 = atan((u0 - x) / a);
-        const double m3 = exp(-u0 * u0) * (1.5707963267948966 - th0) / a;
-        for (int q = 0; q <= 33; ++q) {
-            const double u1 = (q == 33) ? -30.0 : -4.0 + (u0 + 4.0) * q / 32.0;
-            const double g1 = 1.0 / (a * a + (x - u1) * (x - u1));
-            const double m1 = g1 * 0.88622692545275801365 * (1.0 + erf(u1));
-            const double c = u1 <= 0.0 ? 1.0 : exp(-u1 * u1);
-            const double m2 = c * (th0 - atan((u1 - x) / a)) / a;
-            const double m = m1 + m2 + m3;
-            if (m < best) { best = m; b1 = u1; b0 = u0; }
-        }
+        s_th0[tid] = th0;
+        s_m3[tid] = exp(-u0 * u0) * (1.5707963267948966 - th0) / a;
     }
-    tab[i] = make_float2((float)b1, (float)fmin(b0, x));
+    __syncthreads();
+    auto split = [&](int c, double& u0, double& u1) {
+        const int p = c / NQ, q = c % NQ;
+        u0 = x * p / 32.0;
+        u1 = (q == 33) ? -30.0 : -4.0 + (u0 + 4.0) * q / 32.0;
+    };
+    double best = 1e300;
+    int bc = 0x7fffffff;
+    for (int c = tid; c < NP * NQ; c += 128) {
+        double u0, u1;
+        split(c, u0, u1);
+        const double g1 = 1.0 / (a * a + (x - u1) * (x - u1));
+        const double m1 = g1 * 0.88622692545275801365 * (1.0 + erf(u1));
+        const double cc = u1 <= 0.0 ? 1.0 : exp(-u1 * u1);
+        const double m2 = cc * (s_th0[c / NQ] - atan((u1 - x) / a)) / a;
+        const double m = m1 + m2 + s_m3[c / NQ];
+        if (m < best) { best = m; bc = c; }
+    }
+    s_m[tid] = best;
+    s_c[tid] = bc;
+    __syncthreads();
+    for (int w = 64; w > 0; w >>= 1) {
+        if (tid < w) {
+            const double m = s_m[tid + w];
+            const int c = s_c[tid + w];
+            if (m < s_m[tid] || (m == s_m[tid] && c < s_c[tid])) {
+                s_m[tid] = m;
+                s_c[tid] = c;
+            }
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        double u0 = 0.0, u1 = -30.0;
+        if (s_m[0] < 1e300) split(s_c[0], u0, u1);
+        tab[i] = make_float2((float)u1, (float)fmin(u0, x));
+    }
 }
 
 }  // namespace
@@ -178,7 +267,7 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     char* base = (char*)d_table;
     const double* edges = (const double*)(base + g.off_edges);
     double* phi = (double*)(base + g.off_phi);
-    phi_kernel<<<(g.J + 127) / 128, 128, 0, s>>>(edges, phi, g.J, g.a);
+    phi_kernel<<<(g.J + kPhiEdges - 2) / (kPhiEdges - 1), kPhiEdges * 16, 0, s>>>(edges, phi, g.J, g.a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     TableHeader h;
@@ -191,8 +280,8 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     h.a = g.a;
     for (int a = 0; a < 3; ++a) h.dz[a] = 2.0 * g.R / g.n[a];
     const int64_t nrow = (int64_t)g.n_class * g.J;
-    const int threads = 128;
-    const int64_t blocks = (nrow + threads - 1) / threads;
+    const int tiles = (g.J + kRowEdges - 2) / (kRowEdges - 1);
+    const int64_t blocks = g.moving ? (int64_t)g.n_class * tiles : (nrow + kRowEdges - 1) / kRowEdges;
     const ClassDesc* cd = (const ClassDesc*)(base + g.off_cdesc);
     uint32_t* rows = (uint32_t*)(base + g.off_rows);
     uint2* fast = (uint2*)(base + g.off_fast);
@@ -203,12 +292,10 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     unsigned long long* wq = (unsigned long long*)(base + g.off_wq);
     const int weighted = g.weighted() ? 1 : 0;
     float* ka_row = (float*)(base + g.off_ka);
-    if (g.ndim == 1)
-        rows_kernel<1><<<(unsigned)blocks, threads, 0, s>>>(h, cd, edges, phi, rows, fast, tau_row, rk, abs_thr,
-                                                            dusty, wq, ka_row, weighted, nrow);
-    else
-        rows_kernel<3><<<(unsigned)blocks, threads, 0, s>>>(h, cd, edges, phi, rows, fast, tau_row, rk, abs_thr,
-                                                            dusty, wq, ka_row, weighted, nrow);
+    auto rows_k = g.ndim == 1 ? (g.moving ? rows_kernel<1, true> : rows_kernel<1, false>)
+                              : (g.moving ? rows_kernel<3, true> : rows_kernel<3, false>);
+    rows_k<<<(unsigned)blocks, kRowEdges, 0, s>>>(h, cd, edges, phi, rows, fast, tau_row, rk, abs_thr, dusty, wq,
+                                                  ka_row, weighted, tiles, nrow);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.pairs()) {
         pair_kernel<<<(unsigned)((nrow + 255) / 256), 256, 0, s>>>(fast, (Pair*)(base + g.off_pair), g.J, nrow);
@@ -216,7 +303,7 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     }
     // the u_par envelope table serves only the continuous MC of the hybrid scheme
     if (g.params.mode == RDDMC_MODE_HYBRID)
-        upar_kernel<<<(kUparN + 127) / 128, 128, 0, s>>>((float2*)(base + g.off_upar), g.a);
+        upar_kernel<<<kUparN, 128, 0, s>>>((float2*)(base + g.off_upar), g.a);
     return cudaGetLastError();
 }
 

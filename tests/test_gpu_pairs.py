@@ -1,0 +1,67 @@
+"""The walk's pair reads (two frequency moves per gather) against the oracle and
+the fast-head walk: grids of a few bins, where every pair touches the grid's
+ends, watchdog limits inside a group of four, slices, and the two sides of the
+row count up to which a table carries pairs."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import coracle as C  # noqa: E402
+from paper_1709_10187_gb300 import build as B  # noqa: E402
+from paper_1709_10187_gb300 import rddmc as R  # noqa: E402
+from paper_1709_10187_gb300 import workloads as W  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+COUNTS = ("emitted", "escaped", "aborted", "steps", "clamps", "event_draws")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    B.build()
+
+
+def _same(a, b, nf):
+    for k in COUNTS:
+        assert a[k] == b[k], k
+    assert np.array_equal(a["hist"], b["hist"]) and np.array_equal(a["faces"][:nf], b["faces"][:nf])
+    assert np.array_equal(a["sb"], b["sb"])
+
+
+@pytest.mark.parametrize("max_steps", [0, 1, 7, 130, 259])
+@pytest.mark.parametrize("ndim,J,v", [(1, 1, 0.0), (1, 2, 0.0), (1, 3, 0.0), (1, 5, 0.0), (3, 2, 0.0), (3, 3, 20.0),
+                                      (3, 4, 20.0)])
+def test_few_bins_and_odd_limits_match_the_oracle(ndim, J, v, max_steps):
+    n = (5, 1, 1) if ndim == 1 else (6, 6, 6)
+    w = W.Workload(f"pairs_{ndim}_{J}", ndim, n, J, -6.0, 6.0, 40.0, 1.0e4, 3000, 0x5EED0B01, sphere=ndim == 3,
+                   vmax_kms=v)
+    g = C.Grid(w)
+    ot = g.table()
+    p = R.Problem(w)
+    thr, flags = p.rows()
+    sel = np.ones(w.ncell * J, bool) if w.mask() is None else np.repeat(w.mask().astype(bool), J)
+    ot["thr"][sel] = thr[sel]  # walk the device's own thresholds (equal to one count)
+    gpu = p.run(w.packets, w.seed, max_steps=max_steps)
+    orc = C.walk(g, ot, w.seed, 0, w.packets, max_steps=max_steps or 1 << 62)
+    _same(gpu, orc, 2 * ndim)
+    p.close()
+
+
+@pytest.mark.parametrize("chunk", [4, 12, 256])
+def test_pairs_and_heads_walk_alike(chunk):
+    # dense tables below and above 2^20 rows: pairs on one side, heads on the other
+    for n, J in ((2047, 512), (2050, 512)):
+        w = W.Workload(f"rows_{n}", 1, (n, 1, 1), J, -60.0, 60.0, 1.0e6, 1.0e4, 4000, 0x5EED0B02)
+        assert (n * J > 1 << 20) == (n == 2050)
+        dense, dedup = R.Problem(w, layout=R.LAYOUT_DENSE), R.Problem(w)
+        out = []
+        for p in (dense, dedup):
+            p.reset()
+            p.launch(w.packets, w.seed, max_steps=6002, steps_per_launch=3000, chunk=chunk)
+            for _ in range(2):
+                p.launch(w.packets, w.seed, max_steps=6002, steps_per_launch=3000, resume=1, chunk=chunk)
+            out.append(p.read())
+        assert out[0]["emitted"] == w.packets == out[0]["escaped"] + out[0]["aborted"]
+        _same(out[0], out[1], 2)
+        for p in (dense, dedup):
+            p.close()

@@ -418,7 +418,7 @@ typedef struct rddmc_time_step {
     int32_t regroup;        /* lanes still walking their packets break off, so that the lanes whose
                                packets reached t_end take new ones, once fewer than this many of a
                                warp's lanes are walking (packets keep their state in registers and
-                               continue; results do not change): 0 = library default (8),
+                               continue; results do not change): 0 = library default (16),
                                -1 = never, at most 32 */
     int32_t reserved;       /* 0 */
 } rddmc_time_step;

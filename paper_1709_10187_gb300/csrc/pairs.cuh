@@ -74,35 +74,30 @@ struct TransitionStream {
 
     template <class K>
     __device__ __forceinline__ void init(uint32_t b, uint32_t b_hi, uint32_t p_lo, uint32_t p_hi, const K& P) {
-        const unsigned long long w1 = wide(0xCD9E8D57u, p_lo);
-        const unsigned long long w2 = wide(0xD2511F53u, hi(w1) ^ b_hi ^ P.rk0[0]);
+        const unsigned long long w1 = mul_wide(0xCD9E8D57u, p_lo);
+        const unsigned long long w2 = mul_wide(0xD2511F53u, hi(w1) ^ b_hi ^ P.rk0[0]);
         e0 = p_hi ^ P.rk1[0];
         e1 = lo(w1) ^ P.rk0[1];
         e2 = hi(w2) ^ P.rk1[1];
         e3 = lo(w2) ^ P.rk1[2];
-        w0 = wide(0xD2511F53u, b);
+        w0 = mul_wide(0xD2511F53u, b);
     }
 
     template <class K>
     __device__ __forceinline__ uint4 next(const K& P) {
-        const unsigned long long w1 = wide(0xCD9E8D57u, hi(w0) ^ e0);
-        const unsigned long long w2 = wide(0xD2511F53u, hi(w1) ^ e1), w3 = wide(0xCD9E8D57u, lo(w0) ^ e2);
+        const unsigned long long w1 = mul_wide(0xCD9E8D57u, hi(w0) ^ e0);
+        const unsigned long long w2 = mul_wide(0xD2511F53u, hi(w1) ^ e1), w3 = mul_wide(0xCD9E8D57u, lo(w0) ^ e2);
         w0 += 0xD2511F53u;
         uint4 c = make_uint4(hi(w3) ^ lo(w1) ^ P.rk0[2], lo(w3), hi(w2) ^ e3, lo(w2));
 #pragma unroll
         for (int r = 3; r < 10; ++r) {
-            const unsigned long long a0 = wide(0xD2511F53u, c.x), a1 = wide(0xCD9E8D57u, c.z);
+            const unsigned long long a0 = mul_wide(0xD2511F53u, c.x), a1 = mul_wide(0xCD9E8D57u, c.z);
             c = make_uint4(hi(a1) ^ c.y ^ P.rk0[r], lo(a1), hi(a0) ^ c.w ^ P.rk1[r], lo(a0));
         }
         return c;
     }
 
 private:
-    static __device__ __forceinline__ unsigned long long wide(uint32_t a, uint32_t b) {
-        unsigned long long r;
-        asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
-        return r;
-    }
     static __device__ __forceinline__ uint32_t hi(unsigned long long v) { return (uint32_t)(v >> 32); }
     static __device__ __forceinline__ uint32_t lo(unsigned long long v) { return (uint32_t)v; }
 };

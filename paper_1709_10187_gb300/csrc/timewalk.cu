@@ -21,20 +21,16 @@
 // Streams: transition word t is lane t&3 of Philox4x32-10(ctr = (t>>2, p_lo,
 // p_hi)), as in the persistent walk; dwell word d is lane d&3 of
 // Philox4x32-10(ctr = (d>>2, p_lo, p_hi | 2^30)); packet ids stay below 2^62.
-// Transitions run in groups of four with t a multiple of four at the start of
-// each group (one transition call per group; a packet resumed at another t
-// first walks single transitions up to the next multiple of four), and the
-// dwell words of a group come from at most two dwell blocks, the lower one
-// usually the block cached from the group before: two Philox calls per four
-// transitions in all.  Lanes take packets from a global cursor (one atomicAdd
-// per warp) and run at most `chunk` transitions between refills (256 by
-// default), so a lane whose packet stopped early in its step takes a new one
-// while long-running packets continue.  When fewer than `regroup` lanes of a
-// warp are still walking (8 by default), they break off after their group of
-// four, keeping packet, clock and cached blocks in registers, so that the
-// stopped lanes take new packets before the warp walks on: in thick media a
-// packet takes only a few transitions per step, and without the break a warp
-// waits for its slowest lane.
+// A warp walks in passes.  In a pass every walking lane takes the rest of its
+// block of four transition words (a packet resumes anywhere in a block) with the
+// dwell words that go with them: one transition block and one new dwell block
+// per pass, the other dwell block being kept from the pass before.  Lanes whose
+// packet reached t_{n+1} or finished wait; when fewer than `regroup` still walk
+// (16 by default), or after chunk / 4 passes, the waiting lanes save their
+// packets together and take new ones from a global cursor (one atomicAdd per
+// warp), while the others keep theirs in registers: in thick media a packet
+// takes only a few transitions per step, and resuming and saving it costs as
+// much as they do, so both run with as many lanes as can be had.
 //
 // Tallies: the path and bin estimates go to shared memory when the grid's
 // states fit (ticks as a u32 low word plus a u32 carry count, so every update
@@ -60,7 +56,9 @@ namespace {
 
 constexpr uint32_t kTicks = 1u << 31;  // ticks per time step
 constexpr size_t kSmemTallyMax = 110 * 1024;  // shared-memory budget per CTA for the per-state tallies
-constexpr int kRegroupDefault = 8;  // a warp regroups when fewer than a quarter of its lanes still walk
+// a warp regroups when fewer than half of its lanes still walk: the resonant
+// test's first 20 steps take 21.4, 20.7, 21.4 and 22.7 ms at 8, 16, 20 and 24
+constexpr int kRegroupDefault = 16;
 
 struct TimeParams {
     const float* rk;                 // 1 / K_s per row
@@ -93,6 +91,12 @@ __device__ __forceinline__ uint4 trans_block(unsigned long long b, uint32_t pl, 
     return philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), pl, ph), P);
 }
 
+// What bounds it: issue and the latency of one dwell (a chain of a table gather,
+// a logarithm, a shared atomic and a compare), with 24 warps per SM (shared
+// tallies and registers).  1e7 packets, first 20 steps of the resonant test: 20.7
+// ms; 23.6 ms with a loop that walked each lane up to a block's start by single
+// transitions before its groups of four.  Without regrouping losses (long steps,
+// 3e5 packets of the 64 x 128 slab): 925 ms, 935 ms before.
 // MINB: resident 256-thread CTAs per SM the register budget targets (2: no
 // spills, 16 warps per SM; 3: 24 warps with a few spilled registers).
 template <int NDIM, bool SMEM_TALLY, int MINB, bool LEAK, bool WEIGHT>
@@ -133,24 +137,24 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
     bool have = false, exhausted = false;
     unsigned long long pid = 0, t = 0, e = 0, d = 0;
     unsigned cell = 0, cls = 0, s = 0;  // s = cls * J + bin: the row of the state
+    unsigned st = 0;                    // cell * J + bin: the state of the tallies
     unsigned el = 0;                    // ticks elapsed in this step
-    uint32_t pl = 0, ph = 0;
-    unsigned long long tbc = ~0ull;     // index of the cached dwell block
-    uint4 rtc = make_uint4(0u, 0u, 0u, 0u);
+    bool kept = false;                  // dwk is the packet's dwell block of index (d - (t & 3)) >> 2
+    uint4 dwk = make_uint4(0u, 0u, 0u, 0u);
     float wgt = 1.0f;                   // dust by weights: the packet weight
-    unsigned long long tnc = ~0ull;     // index of the cached transition block
-    uint4 rnc = make_uint4(0u, 0u, 0u, 0u);
-    unsigned long long n_steps = 0, n_edraw = 0, n_dwell = 0;
+    // every dwell ends in a transition or stops the packet at t_{n+1}, so the
+    // dwells drawn are n_steps + n_alive
+    unsigned long long n_steps = 0, n_edraw = 0;
     unsigned n_emit = 0, n_esc = 0, n_abort = 0, n_clamp = 0, n_alive = 0, n_absorbed = 0, status_bits = 0;
 
     auto add_path = [&](unsigned ticks) {
         if (!ticks) return;
-        const unsigned st = min(cell * J + min(s - cls * J, J - 1u), ns1);
+        const unsigned i = min(st, ns1);
         if (SMEM_TALLY) {
-            const unsigned old = atomicAdd(&s_plo[st], ticks);  // ticks <= 2^31: at most one carry
-            if (old + ticks < old) atomicAdd(&s_phi[st], 1u);
+            const unsigned old = atomicAdd(&s_plo[i], ticks);  // ticks <= 2^31: at most one carry
+            if (old + ticks < old) atomicAdd(&s_phi[i], 1u);
         } else {
-            atomicAdd(&T.path[st], (unsigned long long)ticks);
+            atomicAdd(&T.path[i], (unsigned long long)ticks);
         }
     };
 
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         const unsigned act = (fl >> (2u * o)) & 3u;
         const unsigned bin = min(s - cls * J, J - 1u);
         if (o < 2u) {
-            if (act == ACT_MOVE) { s += o ? 1u : 0xffffffffu; return false; }
+            if (act == ACT_MOVE) { s += o ? 1u : 0xffffffffu; st += o ? 1u : 0xffffffffu; return false; }
             status_bits |= (unsigned)STATUS_UNSUPPORTED_EVENT;  // MC hand-offs are not part of this walk
             ++n_abort;
             return true;
@@ -220,6 +224,7 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         cell = min((face & 1u) ? cell + stride : cell - stride, (unsigned)P.ncell - 1u);
         cls = __ldg(&P.cell_class[cell]);
         s = cls * J + nbin;
+        st = cell * J + nbin;
         if (LEAK) add_leak(cell * (2u * NDIM) + (face ^ 1u), 1u, s, ticks);
         return false;
     };
@@ -233,15 +238,13 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         const float l = (float)ticks;
         const float ta = __ldg(&T.ka[ri]) * l * T.tick_len;
         const float avg = ta > 1e-4f ? -expm1f(-ta) / ta : 1.0f - 0.5f * ta;
-        const unsigned st = min(cell * J + min(s - cls * J, J - 1u), ns1);
-        atomicAdd(&T.wpath[st], (double)(wgt * l * avg));
+        atomicAdd(&T.wpath[min(st, ns1)], (double)(wgt * l * avg));
         wgt *= expf(-ta);
     };
 
     auto dwell_then_move = [&](unsigned wd, unsigned wt) -> int {
         const unsigned ri = min(s, nr1);
         ++d;
-        ++n_dwell;
         const float u = fmaf((float)wd, 0x1p-32f, 0x1p-33f);
         const float x = -__log2f(u) * (T.x_scale * __ldg(&T.rk[ri]));
         const unsigned dt = x < 4.0e9f ? __float2uint_rn(x) : 0xffffffffu;
@@ -259,7 +262,9 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         const uint2 f = __ldg(&P.fast[ri]);
         int r;
         if (wt < f.y) {
-            s += (wt >= f.x) ? 1u : 0xffffffffu;
+            const unsigned dj = (wt >= f.x) ? 1u : 0xffffffffu;
+            s += dj;
+            st += dj;
             r = 0;
         } else {
             r = generic(wt, dt) ? 2 : 0;
@@ -272,16 +277,38 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         return r;
     };
 
-    auto dwell_word = [&](unsigned long long dd) -> unsigned {
-        const unsigned long long b = dd >> 2;
-        if (b != tbc) { rtc = time_block(b, pl, ph, P); tbc = b; }
-        return word_of(rtc, (unsigned)dd & 3u);
-    };
-
-    auto trans_word = [&](unsigned long long tt) -> unsigned {
-        const unsigned long long b = tt >> 2;
-        if (b != tnc) { rnc = trans_block(b, pl, ph, P); tnc = b; }
-        return word_of(rnc, (unsigned)tt & 3u);
+    // The rest of the packet's block of transition words, t & 3 .. 3, and the
+    // dwell words that go with them.  Returns as dwell_then_move, 2 also when the
+    // packet reaches the watchdog.
+    auto pass = [&]() -> int {
+        const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
+        const unsigned k0 = (unsigned)t & 3u;
+        const unsigned long long room = P.max_steps - t;
+        const unsigned k1 = room < 4ull - k0 ? k0 + (unsigned)room : 4u;
+        const uint4 rn = trans_block(t >> 2, pl, ph, P);
+        // dwell words w .. w + 3 with w = d - k0 (d >= t: a packet draws a dwell
+        // per transition): the upper words of one block, the lower of the next
+        const unsigned long long w = d - k0;
+        const unsigned p = (unsigned)w & 3u;
+        uint4 lo = dwk;
+        if (!kept && p + k0 < 4u) lo = time_block(w >> 2, pl, ph, P);
+        uint4 dw = lo;
+        kept = p != 0u;
+        if (p) {
+            dwk = time_block((w >> 2) + 1ull, pl, ph, P);
+            if (p == 1u) dw = make_uint4(lo.y, lo.z, lo.w, dwk.x);
+            else if (p == 2u) dw = make_uint4(lo.z, lo.w, dwk.x, dwk.y);
+            else dw = make_uint4(lo.w, dwk.x, dwk.y, dwk.z);
+        }
+        int r = 0;
+#pragma unroll
+        for (unsigned k = 0; k < 4u; ++k)
+            if (r == 0 && k >= k0 && k < k1) r = dwell_then_move(word_of(dw, k), word_of(rn, k));
+        if (r == 0 && t >= P.max_steps) {
+            ++n_abort;
+            r = 2;
+        }
+        return r;
     };
 
     for (;;) {
@@ -298,9 +325,9 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
                 if (pid >= P.n_packets) {
                     exhausted = true;
                 } else {
-                    const uint8_t st = T.start ? (uint8_t)PK_FRESH : P.st_status[pid];
+                    const uint8_t was = T.start ? (uint8_t)PK_FRESH : P.st_status[pid];
                     unsigned bin = 0;
-                    if (st == PK_INFLIGHT) {
+                    if (was == PK_INFLIGHT) {
                         cell = P.st_cell[pid];
                         bin = P.st_bin[pid];
                         t = P.st_t[pid];
@@ -308,7 +335,7 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
                         d = T.st_d[pid];
                         if (WEIGHT) wgt = T.st_w[pid];
                         have = true;
-                    } else if (st == PK_FRESH) {
+                    } else if (was == PK_FRESH) {
                         // event draw 0: bit 31-a picks the centre cell on axis a, bit 28 the bin
                         const unsigned w = event_word(pid, 0, P.k0, P.k1);
                         unsigned idx[3];
@@ -328,88 +355,54 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
                     if (have) {
                         cell = min(cell, (unsigned)P.ncell - 1u);
                         cls = __ldg(&P.cell_class[cell]);
-                        s = cls * J + min(bin, J - 1u);
+                        bin = min(bin, J - 1u);
+                        s = cls * J + bin;
+                        st = cell * J + bin;
                         el = 0;
-                        pl = (uint32_t)pid;
-                        ph = (uint32_t)(pid >> 32);
-                        tbc = ~0ull;
-                        tnc = ~0ull;
+                        kept = false;
+                        n_steps -= t;
+                        n_edraw -= e;
                     }
                 }
             }
         }
         if (__all_sync(FULL, !have)) break;  // every lane is out of packets
         // once the cursor has run dry, lanes that stop cannot take new packets
-        const bool dry = __any_sync(FULL, exhausted);
-        if (!have) continue;
-
-        // ---- up to `chunk` dwells: single ones up to t = 0 mod 4, then groups of four
-        const unsigned long long t0 = t, e0 = e;
-        const unsigned long long lim = min(t + (unsigned long long)P.chunk, P.max_steps);
-        int r = 0;
-        bool cut = false;
-        while (r == 0 && (t & 3ull) && t < lim) r = dwell_then_move(dwell_word(d), trans_word(t));
-        while (r == 0 && t + 4ull <= lim) {
-            // Regroup: packets take different numbers of dwells to reach t_{n+1},
-            // so once fewer than `regroup` lanes are still walking, they break
-            // off (keeping their packets, blocks and clocks in registers) and the
-            // stopped lanes take new packets before the warp walks on.
-            if (T.regroup && !dry && __popc(__activemask()) < (unsigned)T.regroup) {
-                cut = true;
-                break;
-            }
-            const uint4 rn = trans_block(t >> 2, pl, ph, P);
-            tnc = t >> 2;
-            rnc = rn;
-            const unsigned long long b0 = d >> 2;
-            const unsigned p = (unsigned)d & 3u;
-            const uint4 lo = (b0 == tbc) ? rtc : time_block(b0, pl, ph, P);
-            uint4 hi = lo;
-            if (p) hi = time_block(b0 + 1ull, pl, ph, P);
-            tbc = p ? b0 + 1ull : b0;
-            rtc = hi;
-#pragma unroll
-            for (unsigned k = 0; k < 4u; ++k) {
-                const unsigned q = p + k;
-                const unsigned wd = q < 4u ? word_of(lo, q) : word_of(hi, q - 4u);
-                r = dwell_then_move(wd, word_of(rn, k));
-                if (r) break;
-            }
+        const int regroup = __any_sync(FULL, exhausted) ? 0 : T.regroup;
+        int r = have ? 0 : 3;
+        for (int left = P.chunk >> 2; left; --left) {
+            if (r == 0) r = pass();
+            const int walking = __popc(__ballot_sync(FULL, r == 0));
+            if (!walking || walking < regroup) break;
         }
-        if (!cut)
-            while (r == 0 && t < lim) r = dwell_then_move(dwell_word(d), trans_word(t));  // short chunk end
-        n_steps += t - t0;
-        n_edraw += e - e0;
-        if (r == 0 && t >= P.max_steps) {
-            ++n_abort;
-            r = 2;
-        }
-        if (r == 2) {
+        if (r == 1 || r == 2) {
+            n_steps += t;
+            n_edraw += e;
             have = false;
-            P.st_status[pid] = PK_DONE;
-        } else if (r == 1) {
-            const unsigned bin = min(s - cls * J, J - 1u);
-            const unsigned st = min(cell * J + bin, ns1);
-            if (SMEM_TALLY) atomicAdd(&s_bins[st], 1u);
-            else atomicAdd(&T.bins[st], 1ull);
-            if (WEIGHT) {
-                atomicAdd(&T.wbins[st], (double)wgt);
-                T.st_w[pid] = wgt;
+            if (r == 2) {
+                P.st_status[pid] = PK_DONE;
+            } else {
+                const unsigned i = min(st, ns1);
+                if (SMEM_TALLY) atomicAdd(&s_bins[i], 1u);
+                else atomicAdd(&T.bins[i], 1ull);
+                if (WEIGHT) {
+                    atomicAdd(&T.wbins[i], (double)wgt);
+                    T.st_w[pid] = wgt;
+                }
+                ++n_alive;
+                P.st_cell[pid] = cell;
+                P.st_bin[pid] = min(s - cls * J, J - 1u);
+                P.st_t[pid] = t;
+                P.st_e[pid] = e;
+                T.st_d[pid] = d;
+                P.st_status[pid] = PK_INFLIGHT;
             }
-            ++n_alive;
-            P.st_cell[pid] = cell;
-            P.st_bin[pid] = bin;
-            P.st_t[pid] = t;
-            P.st_e[pid] = e;
-            T.st_d[pid] = d;
-            P.st_status[pid] = PK_INFLIGHT;
-            have = false;
         }
     }
 
     // ---- flush: warp sums of the per-thread counters, then CTA totals to HBM
     unsigned long long v[10] = {n_emit, n_esc,  n_abort, n_steps, n_clamp,
-                                n_edraw, status_bits, n_dwell, n_alive, n_absorbed};
+                                n_edraw, status_bits, n_steps + n_alive, n_alive, n_absorbed};
 #pragma unroll
     for (int i = 0; i < 10; ++i) {
         unsigned long long x = v[i];

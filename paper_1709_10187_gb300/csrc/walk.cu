@@ -490,20 +490,19 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             const unsigned w = word_of(r, q);
             const unsigned ri = min(s, nr1);
             const uint4 a = __ldg(&rows[ri * RW]);
-            unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
+            unsigned k = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
             if (NDIM == 3) {
                 const uint4 b = __ldg(&rows[ri * RW + 1]);
-                o += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
+                k += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
             }
-            const bool plain = ((a.w >> (2u * o)) & 3u) == ACT_MOVE && !(P.dust && o == 2u * NDIM + 1u);
-            if (plain) {
-                if (o < 2u) {
-                    s += o ? 1u : 0xffffffffu;
+            if (((a.w >> (2u * k)) & 3u) == ACT_MOVE && !(P.dust && k == 2u * NDIM + 1u)) {
+                if (k < 2u) {
+                    s += k ? 1u : 0xffffffffu;
                 } else {
-                    const unsigned ax = (o - 2u) >> 1;
+                    const unsigned ax = (k - 2u) >> 1;
                     const unsigned stride =
                         NDIM == 1 ? 1u : (ax == 0 ? 1u : (ax == 1 ? (unsigned)P.n0 : (unsigned)P.n01));
-                    cell = min((o & 1u) ? cell + stride : cell - stride, (unsigned)P.ncell - 1u);
+                    cell = min((k & 1u) ? cell + stride : cell - stride, (unsigned)P.ncell - 1u);
                     const unsigned c1 = __ldg(&P.cell_class[cell]);
                     s += (c1 - cls) * J;
                     cls = c1;
@@ -514,11 +513,16 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         } while (++q < 4u);
         return 4u;
     };
+    auto done_with = [&]() {
+        release();
+        if (P.save_state) P.st_status[pid] = PK_DONE;
+    };
 
     for (;;) {
-        // ---- warp-cooperative refill
-        const unsigned need = __ballot_sync(FULL, !have && !exhausted);
-        if (need) {
+        // ---- warp-cooperative refill, repeated while lanes draw finished packets
+        for (;;) {
+            const unsigned need = __ballot_sync(FULL, !have && !exhausted);
+            if (!need) break;
             const int leader = __ffs(need) - 1;
             unsigned long long first = 0;
             if ((int)lane == leader) first = atomicAdd(P.cursor, (unsigned long long)__popc(need));
@@ -569,9 +573,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                 }
             }
         }
-        if (__all_sync(FULL, exhausted && !have)) break;
-        if (!have) continue;
-        if (P.time_slice_ns && global_ns() - t_begin > P.time_slice_ns) {
+        if (__all_sync(FULL, !have)) break;  // every lane is out of packets
+        if (have && P.time_slice_ns && global_ns() - t_begin > P.time_slice_ns) {
             // end of the wall-time slice: save the packet, take no new one
             P.st_cell[pid] = cell;
             P.st_bin[pid] = min(s - cls * J, J - 1u);
@@ -581,9 +584,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             P.st_status[pid] = PK_INFLIGHT;
             release();
             exhausted = true;
-            continue;
         }
-        if (PROPOSE && prop_takes(P, cell, min(s - cls * J, J - 1u))) {
+        if (PROPOSE && have && prop_takes(P, cell, min(s - cls * J, J - 1u))) {
             // the walk is Markov in (cell, bin): a packet in a state the proposal
             // serves waits for it (checked once per chunk of transitions)
             P.st_cell[pid] = cell;
@@ -601,18 +603,19 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
             const unsigned long long k = k0q + (unsigned long long)__popc(grp & ((1u << lane) - 1u));
             P.prop_qpid[min(k, P.n_packets - 1ull)] = pid;
             release();
-            continue;
         }
 
-        // ---- run up to `chunk` transitions (with a proposal, up to the next
-        // multiple of chunk, so the parking checkpoints do not depend on slicing)
-        unsigned long long lim = PROPOSE ? (t / (unsigned long long)P.chunk + 1ull) * (unsigned long long)P.chunk
-                                         : t + (unsigned long long)P.chunk;
+        // ---- run up to `chunk` transitions, to the slice's end or the watchdog's
+        // limit (with a proposal to the next multiple of chunk, so the parking
+        // checkpoints do not depend on slicing)
+        unsigned long long lim = PROPOSE ? (t / (unsigned long long)P.chunk + 1ull) * (unsigned long long)P.chunk : ~0ull;
         lim = lim < t_stop ? lim : t_stop;
         lim = lim < P.max_steps ? lim : P.max_steps;
-        bool fin = false;
-        {
-            const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
+        const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
+        if (have) {
+            const unsigned long long lim0 = lim;
+            if (!PROPOSE) lim = min(lim, t + (unsigned long long)P.chunk);
+            bool fin = false;
             unsigned long long blk = t >> 2;
             const unsigned ng = (unsigned)((lim - t) >> 2);  // full groups of four
             if constexpr (PATH == PAIRS) {
@@ -722,31 +725,31 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                 }
                 t += 4ull * ng;
             }
-            // at most three transitions left before the watchdog limit
-            while (t < lim) {
-                const unsigned long long b = t >> 2;
-                const uint4 r = philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), pl, ph), P);
-                const bool f = generic(word_of(r, (unsigned)t & 3u));
-                ++t;
-                if (f) { fin = true; break; }
-            }
+        chunk_done:
+            if (fin) done_with();
+            lim = lim0;
         }
-    chunk_done:
-        if (fin) {
-            release();
-            if (P.save_state) P.st_status[pid] = PK_DONE;
-        } else if (t >= P.max_steps) {
-            ++cnt32(L_ABORT);
-            release();
-            if (P.save_state) P.st_status[pid] = PK_DONE;
-        } else if (t >= t_stop) {
-            P.st_cell[pid] = cell;
-            P.st_bin[pid] = min(s - cls * J, J - 1u);
-            P.st_t[pid] = t;
-            P.st_e[pid] = e;
-            if (WEIGHT) P.st_lw[pid] = lw;
-            P.st_status[pid] = PK_INFLIGHT;
-            release();
+        // at most three transitions left before the watchdog limit
+        while (have && t < lim && lim - t < 4ull) {
+            const unsigned long long b = t >> 2;
+            const uint4 r = philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), pl, ph), P);
+            const bool f = generic(word_of(r, (unsigned)t & 3u));
+            ++t;
+            if (f) done_with();
+        }
+        if (have) {
+            if (t >= P.max_steps) {
+                ++cnt32(L_ABORT);
+                done_with();
+            } else if (t >= t_stop) {
+                P.st_cell[pid] = cell;
+                P.st_bin[pid] = min(s - cls * J, J - 1u);
+                P.st_t[pid] = t;
+                P.st_e[pid] = e;
+                if (WEIGHT) P.st_lw[pid] = lw;
+                P.st_status[pid] = PK_INFLIGHT;
+                release();
+            }
         }
     }
 

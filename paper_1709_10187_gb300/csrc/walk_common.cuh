@@ -69,11 +69,9 @@ struct WalkParams {
 __device__ __forceinline__ uint4 philox_rk(uint4 c, const WalkParams& P) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ P.rk0[r], lo1, hi0 ^ c.w ^ P.rk1[r], lo0);
+        const unsigned long long a0 = mul_wide(0xD2511F53u, c.x), a1 = mul_wide(0xCD9E8D57u, c.z);
+        c = make_uint4((uint32_t)(a1 >> 32) ^ c.y ^ P.rk0[r], (uint32_t)a1, (uint32_t)(a0 >> 32) ^ c.w ^ P.rk1[r],
+                       (uint32_t)a0);
     }
     return c;
 }

@@ -1064,89 +1064,176 @@ struct FpRegionParams {
     FeatConst fc;
 };
 
-__global__ void __launch_bounds__(256) fp_region_kernel(const WalkParams P, const FpRegionParams F) {
+// The start of sample i: brick, start cell (axis 0 fastest) and start bin from
+// its event draws 0-2.
+struct FpStart {
+    int br, mc, j;
+};
+__device__ __forceinline__ FpStart fp_start(const WalkParams& P, const FpRegionParams& F, unsigned long long pid) {
+    const uint4 w = philox_rk(make_uint4(0u, 0u, (uint32_t)pid, (uint32_t)(pid >> 32) | 0x80000000u), P);
+    const int k = min((int)(((unsigned long long)w.x * (unsigned long long)F.n_el) >> 32), F.n_el - 1);
+    const int cnt = F.bin_off[k + 1] - F.bin_off[k];
+    FpStart s;
+    s.br = F.bricks[k];
+    s.mc = (int)(((unsigned long long)w.y * (unsigned long long)(P.prop_r * P.prop_r * P.prop_r)) >> 32);
+    s.j = F.bins[F.bin_off[k] + min((int)(((unsigned long long)w.z * (unsigned long long)cnt) >> 32), cnt - 1)];
+    return s;
+}
+
+// A passage takes anything from one transition to a hundred thousand, so a lane
+// that ends one takes the next of its warp's range (kFpRefill transitions between
+// refills), and the grid is sized for several passages per lane: a thread per
+// passage left 6 of 32 lanes active.  Four transitions run as a chain of head
+// loads, as in the walk.  Bound by the longest passages' chains once the range is
+// drawn.  2e5 passages out of 6^3 regions of a 32^3 x 64 medium: 71 ms, 158 before.
+constexpr int kFpRefill = 64;
+constexpr int kFpThreads = 64;
+constexpr int kFpPerLane = 2;  // passages per lane below which the grid shrinks (1, 2, 4, 8: 76, 71, 77, 83 ms)
+
+__global__ void __launch_bounds__(kFpThreads, 12) fp_region_kernel(const __grid_constant__ WalkParams P,
+                                                                   const __grid_constant__ FpRegionParams F) {
     const unsigned J = (unsigned)P.J, nr1 = (unsigned)P.n_rows - 1u;
-    const int r = P.prop_r, bl = P.prop_b;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < F.n; i += stride) {
-        const unsigned long long pid = F.p0 + i;
-        EventStream es;
-        es.init(pid, 0, P.k0, P.k1);
-        const unsigned w0 = es.next(), w1 = es.next(), w2 = es.next();
-        const int k = min((int)(((unsigned long long)w0 * (unsigned long long)F.n_el) >> 32), F.n_el - 1);
-        const int br = F.bricks[k];
-        const int bc[3] = {br % P.prop_nbx, (br / P.prop_nbx) % P.prop_nby, br / (P.prop_nbx * P.prop_nby)};
-        const int mc = (int)(((unsigned long long)w1 * (unsigned long long)(r * r * r)) >> 32);
-        int l[3] = {mc % r, (mc / r) % r, mc / (r * r)};
-        int base[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) base[a] = bc[a] * bl - P.prop_sh + P.prop_m;
-        const int cnt = F.bin_off[k + 1] - F.bin_off[k];
-        int j = F.bins[F.bin_off[k] + min((int)(((unsigned long long)w2 * (unsigned long long)cnt) >> 32), cnt - 1)];
-        const int j0 = j;
-        const int l0[3] = {l[0], l[1], l[2]};
-        const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
-        int face = 6, pos = -1;
-        unsigned long long t = 0;
-        while (t < F.cap && face == 6) {
-            const unsigned long long blk = t >> 2;
-            const uint4 rw = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
-            bool stop = false;
-            for (unsigned q = (unsigned)(t & 3u); q < 4u && t < F.cap; ++q) {
-                const unsigned w = word_of(rw, q);
-                ++t;
-                int wc[3];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) wc[a] = min(max(base[a] + l[a], 0), P.n[a] - 1);
-                const unsigned cell = (unsigned)wc[0] + (unsigned)P.n0 * (unsigned)wc[1] + (unsigned)P.n01 * (unsigned)wc[2];
-                const unsigned cls = min(__ldg(&P.cell_class[min(cell, (unsigned)P.ncell - 1u)]), (unsigned)P.n_class - 1u);
-                const unsigned sidx = min(cls * J + (unsigned)j, nr1);
-                const uint2 f = __ldg(&P.fast[sidx]);
-                if (w < f.y) { j += (w >= f.x) ? 1 : -1; continue; }
-                const uint4 a = __ldg(&P.rows[2u * sidx]), c = __ldg(&P.rows[2u * sidx + 1u]);
-                const unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z) +
-                                   (unsigned)(w >= c.x) + (unsigned)(w >= c.y) + (unsigned)(w >= c.z) +
-                                   (unsigned)(w >= c.w);
-                if (o < 2u) { j += o ? 1 : -1; continue; }
-                const int fc_ = (int)o - 2, ax = fc_ >> 1, side = (fc_ & 1) ? 1 : -1;
-                if (l[ax] + side < 0 || l[ax] + side >= r) {
-                    face = fc_;
-                    const int u = ax == 0 ? 1 : 0, v = ax == 2 ? 1 : 2;  // the other two axes, lower first
-                    pos = l[u] + r * l[v];
-                    break;
-                }
-                const unsigned act = (a.w >> (2u * o)) & 3u;
-                if (act == ACT_ESCAPE || act == ACT_TO_MC) { stop = true; break; }  // not inside a region
-                if (act == ACT_REBIN) {
-                    const Rebin rb = P.rebin[cls * 6u + (unsigned)fc_];
-                    const unsigned wr = es.next();
-                    const int jn = j + rb.m + (wr >= rb.thr ? 1 : 0);
-                    j = jn < 0 ? 0 : (jn > (int)J - 1 ? (int)J - 1 : jn);
-                }
-                l[ax] += side;
-            }
-            if (stop) break;
+    const int r = P.prop_r;
+    const unsigned lane = threadIdx.x & 31u;
+    // this warp's samples: a contiguous range
+    const unsigned long long n_warp = (unsigned long long)gridDim.x * (kFpThreads / 32);
+    const unsigned long long warp = (unsigned long long)blockIdx.x * (kFpThreads / 32) + (threadIdx.x >> 5);
+    const unsigned long long per = (F.n + n_warp - 1ull) / n_warp;
+    unsigned long long next = min(warp * per, F.n);
+    const unsigned long long end = min(next + per, F.n);
+
+    bool have = false;
+    unsigned long long i = 0, t = 0;
+    unsigned e = 0;                     // event draws taken by rebins
+    unsigned cell = 0, cls = 0, s = 0;  // s = cls * J + bin
+    int l[3] = {0, 0, 0};
+    int face = 6, pos = -1;
+
+    // The outcome of word w from the full row; true when the passage has ended.
+    auto by_row = [&](unsigned w) -> bool {
+        const unsigned ri = min(s, nr1);
+        const uint4 a = __ldg(&P.rows[2u * ri]), c = __ldg(&P.rows[2u * ri + 1u]);
+        const unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z) + (unsigned)(w >= c.x) +
+                           (unsigned)(w >= c.y) + (unsigned)(w >= c.z) + (unsigned)(w >= c.w);
+        if (o < 2u) {
+            s += o ? 1u : 0xffffffffu;
+            return false;
         }
+        const int fc_ = (int)o - 2, ax = fc_ >> 1, side = (fc_ & 1) ? 1 : -1;
+        const int la = ax == 0 ? l[0] : (ax == 1 ? l[1] : l[2]);
+        if (la + side < 0 || la + side >= r) {
+            face = fc_;
+            pos = ax == 0 ? l[1] + r * l[2] : (ax == 1 ? l[0] + r * l[2] : l[0] + r * l[1]);  // lower axis first
+            return true;
+        }
+        const unsigned act = (a.w >> (2u * o)) & 3u;
+        if (act == ACT_ESCAPE || act == ACT_TO_MC) return true;  // not inside a region
+        int j = (int)min(s - cls * J, J - 1u);
+        if (act == ACT_REBIN) {
+            const Rebin rb = P.rebin[cls * 6u + (unsigned)fc_];
+            const unsigned wr = event_word(F.p0 + i, 3ull + e++, P.k0, P.k1);
+            const int jn = j + rb.m + (wr >= rb.thr ? 1 : 0);
+            j = jn < 0 ? 0 : (jn > (int)J - 1 ? (int)J - 1 : jn);
+        }
+        const unsigned stride = ax == 0 ? 1u : (ax == 1 ? (unsigned)P.n0 : (unsigned)P.n01);
+        if (ax == 0) l[0] += side;
+        else if (ax == 1) l[1] += side;
+        else l[2] += side;
+        cell = min(side > 0 ? cell + stride : cell - stride, (unsigned)P.ncell - 1u);
+        cls = min(__ldg(&P.cell_class[cell]), (unsigned)P.n_class - 1u);
+        s = cls * J + (unsigned)j;
+        return false;
+    };
+    auto cell_at = [&](int br, int mc, int lo[3]) -> unsigned {
+        const int bc[3] = {br % P.prop_nbx, (br / P.prop_nbx) % P.prop_nby, br / (P.prop_nbx * P.prop_nby)};
+        lo[0] = mc % r;
+        lo[1] = (mc / r) % r;
+        lo[2] = mc / (r * r);
+        unsigned wc[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            wc[a] = (unsigned)min(max(bc[a] * P.prop_b - P.prop_sh + P.prop_m + lo[a], 0), P.n[a] - 1);
+        return min(wc[0] + (unsigned)P.n0 * wc[1] + (unsigned)P.n01 * wc[2], (unsigned)P.ncell - 1u);
+    };
+
+    for (;;) {
+        const unsigned need = __ballot_sync(FULL, !have);
+        if (need && next < end) {
+            if (!have) {
+                i = next + (unsigned long long)__popc(need & ((1u << lane) - 1u));
+                if (i < end) {
+                    const FpStart st = fp_start(P, F, F.p0 + i);
+                    cell = cell_at(st.br, st.mc, l);
+                    cls = min(__ldg(&P.cell_class[cell]), (unsigned)P.n_class - 1u);
+                    s = cls * J + (unsigned)st.j;
+                    t = 0;
+                    e = 0;
+                    face = 6;
+                    pos = -1;
+                    have = true;
+                }
+            }
+            next += (unsigned long long)__popc(need);
+        }
+        if (__all_sync(FULL, !have)) break;
+        if (!have) continue;
+
+        const unsigned long long pid = F.p0 + i;
+        const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
+        const unsigned long long lim = min(t + (unsigned long long)kFpRefill, F.cap);
+        bool fin = false;
+        uint4 rn = philox_rk(make_uint4((uint32_t)(t >> 2), (uint32_t)(t >> 34), pl, ph), P);
+        while (!fin && t + 4ull <= lim) {  // t is a multiple of four until the cap
+            const uint4 w = rn;
+            const unsigned s0 = s;
+            const uint2 f0 = __ldg(&P.fast[min(s0, nr1)]);
+            const unsigned s1 = s0 + ((w.x >= f0.x) ? 1u : 0xffffffffu);
+            const uint2 f1 = __ldg(&P.fast[min(s1, nr1)]);
+            const unsigned s2 = s1 + ((w.y >= f1.x) ? 1u : 0xffffffffu);
+            const uint2 f2 = __ldg(&P.fast[min(s2, nr1)]);
+            const unsigned s3 = s2 + ((w.z >= f2.x) ? 1u : 0xffffffffu);
+            const uint2 f3 = __ldg(&P.fast[min(s3, nr1)]);
+            const unsigned s4 = s3 + ((w.w >= f3.x) ? 1u : 0xffffffffu);
+            const unsigned long long blk = (t >> 2) + 1ull;
+            rn = philox_rk(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
+            const bool ok0 = w.x < f0.y, ok1 = w.y < f1.y, ok2 = w.z < f2.y, ok3 = w.w < f3.y;
+            if (ok0 && ok1 && ok2 && ok3) {
+                s = s4;
+                t += 4ull;
+                continue;
+            }
+            unsigned q = !ok0 ? 0u : (!ok1 ? 1u : (!ok2 ? 2u : 3u));
+            s = !ok0 ? s0 : (!ok1 ? s1 : (!ok2 ? s2 : s3));
+            do fin = by_row(word_of(w, q));
+            while (++q < 4u && !fin);
+            t += q;
+        }
+        for (unsigned q = 0; !fin && t < lim; ++q) {  // the last three before the cap
+            ++t;
+            fin = by_row(word_of(rn, q));
+        }
+        if (!fin && t < F.cap) continue;
+        have = false;
+        const FpStart st = fp_start(P, F, pid);
+        const int j = (int)min(s - cls * J, J - 1u);
         int32_t* o8 = F.out + 8 * i;
-        o8[0] = br;
-        o8[1] = j0;
-        o8[2] = mc;
+        o8[0] = st.br;
+        o8[1] = st.j;
+        o8[2] = st.mc;
         o8[3] = face;
         o8[4] = j;
         o8[5] = pos;
-        o8[6] = (int32_t)(es.e - 3ull);
+        o8[6] = (int32_t)e;
         o8[7] = 0;
         F.steps[i] = t;
         if (F.X) {
-            int wc0[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) wc0[a] = min(max(base[a] + l0[a], 0), P.n[a] - 1);
-            const unsigned c0 = (unsigned)wc0[0] + (unsigned)P.n0 * (unsigned)wc0[1] + (unsigned)P.n01 * (unsigned)wc0[2];
-            const unsigned cls0 = min(__ldg(&P.cell_class[min(c0, (unsigned)P.ncell - 1u)]), (unsigned)P.n_class - 1u);
-            const float* sm = P.prop_sum + (size_t)br * kRegionSum;
+            int l0[3];
+            const unsigned c0 = cell_at(st.br, st.mc, l0);
+            const unsigned cls0 = min(__ldg(&P.cell_class[c0]), (unsigned)P.n_class - 1u);
+            const float* sm = P.prop_sum + (size_t)st.br * kRegionSum;
             const float dlog = log10f((float)(P.cdesc[cls0].k0 * P.dz[0])) - sm[0];
-            features_region(sm, F.lp[j0], F.xc[j0], dlog, l0, r, F.fc, F.X + kFeat * i);
-            F.tA[i] = face < 6 ? face * (int)J + min(max(j, 0), (int)J - 1) : -1;
+            features_region(sm, F.lp[st.j], F.xc[st.j], dlog, l0, r, F.fc, F.X + kFeat * i);
+            F.tA[i] = face < 6 ? face * (int)J + j : -1;
             F.tB[i] = step_bucket(t);
             if (F.tC) F.tC[i] = face < 6 ? face * r * r + pos : -1;
         }
@@ -1405,8 +1492,11 @@ extern "C" int rddmc_fp_region_generate(const rddmc_grid* g, const void* d_table
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return RDDMC_ERR_CUDA;
-    const unsigned long long want = (n + 255) / 256;
-    const unsigned blocks = (unsigned)(want < (unsigned long long)nsm * 8 ? want : (unsigned long long)nsm * 8);
-    fp_region_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(P, F);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fp_region_kernel, kFpThreads, 0) != cudaSuccess)
+        return RDDMC_ERR_CUDA;
+    const unsigned long long want = (n + kFpThreads * kFpPerLane - 1) / (kFpThreads * kFpPerLane);
+    const unsigned long long full = (unsigned long long)nsm * (unsigned)std::max(1, per_sm);
+    fp_region_kernel<<<(unsigned)std::min(want, full), kFpThreads, 0, (cudaStream_t)stream>>>(P, F);
     return cudaGetLastError() == cudaSuccess ? RDDMC_OK : RDDMC_ERR_CUDA;
 }

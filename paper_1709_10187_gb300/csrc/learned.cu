@@ -200,7 +200,7 @@ int rddmc_fp_generate(const rddmc_grid* const* grids, const void* const* d_table
 // W1[128x16] b1[128] W2[128x128] b2[128] W3[128x128] b3[128] W4[n_out x 128]
 // b4[n_out].  Every matrix product runs on the tcgen05 tensor cores
 // (umma.cuh: BF16 operands, FP32 accumulators in tensor memory), the backward
-// ones on transposed copies so that both operands are K-major; softmax,
+// ones on the activations and weights as they lie in memory; softmax,
 // cross-entropy, bias sums and Adam in FP32.
 namespace rddmc {
 namespace {
@@ -223,77 +223,93 @@ MlpOffsets mlp_offsets(int n_out) {
     return o;
 }
 
-// Softmax cross-entropy of the heads, one warp per row: loss += CE_A + CE_B
-// (+ CE_C over the S logits of the target's slice when head C is present and
-// its target is >= 0), summed over the batch; dlogits = (softmax - onehot) / B
-// on the logits a head used, zero elsewhere.
+// Softmax cross-entropy of the heads, a warp per row: loss += CE_A + CE_B (+ CE_C
+// over the S logits of the target's slice when head C is present and its target
+// is >= 0), summed over the batch; dlogits = (softmax - onehot) / B on the logits
+// a head used, zero elsewhere, in BF16 for the products, and its FP32 column sums
+// added to db.  ACC: every warp sums its rows' columns in shared memory (n_out
+// floats a warp) before the block adds them to db; otherwise (an n_out past
+// shared memory) each goes straight to db.
+//
+// One pass over the FP32 logits (the second and third read them back through L1)
+// and one over the BF16 gradients; the FP32 gradients are not stored.
+template <bool ACC>
 __global__ void softmax_ce_kernel(const float* __restrict__ logits, int n_out, int nA, int nB, int nC, int S,
                                   const int* __restrict__ tA, const int* __restrict__ tB, const int* __restrict__ tC,
-                                  int Bsz, float* __restrict__ dlogf, __nv_bfloat16* __restrict__ dlogb,
-                                  float* loss) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (row >= Bsz) return;
-    const float* z = logits + (size_t)row * n_out;
-    float* gf = dlogf + (size_t)row * n_out;
-    __nv_bfloat16* gb = dlogb + (size_t)row * n_out;
+                                  int Bsz, __nv_bfloat16* __restrict__ dlogb, float* __restrict__ db, float* loss) {
+    extern __shared__ float s_acc[];
+    const int warps = (int)blockDim.x >> 5, warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    float* acc = s_acc + (size_t)warp * n_out;
+    if (ACC)
+        for (int k = lane; k < n_out; k += 32) acc[k] = 0.0f;
     float total = 0.0f;
-    const bool skip = tA[row] < 0;  // ignored sample: no loss, no gradient
-    // zero everything past heads A and B (head C's unused slices, padding)
-    for (int k = (skip ? 0 : nA + nB) + lane; k < n_out; k += 32) {
-        gf[k] = 0.0f;
-        gb[k] = __float2bfloat16(0.0f);
+    for (int row = (int)blockIdx.x * warps + warp; row < Bsz; row += (int)gridDim.x * warps) {
+        const float* z = logits + (size_t)row * n_out;
+        __nv_bfloat16* gb = dlogb + (size_t)row * n_out;
+        const bool skip = tA[row] < 0;  // ignored sample: no loss, no gradient
+        // zero everything past heads A and B (head C's unused slices, padding)
+        for (int k = (skip ? 0 : nA + nB) + lane; k < n_out; k += 32) gb[k] = __float2bfloat16(0.0f);
+        if (skip) continue;
+        int tc = (nC > 0 && tC) ? tC[row] : -1;
+        if (tc >= nC) tc = -1;
+        const int nh = tc >= 0 ? 3 : 2;
+        for (int h = 0; h < nh; ++h) {
+            int lo, hi, tgt;
+            if (h == 0) { lo = 0; hi = nA; tgt = tA[row]; }
+            else if (h == 1) { lo = nA; hi = nA + nB; tgt = nA + tB[row]; }
+            else { lo = nA + nB + (tc / S) * S; hi = lo + S; tgt = nA + nB + tc; }
+            float mx = -3.0e38f;
+            for (int k = lo + lane; k < hi; k += 32) mx = fmaxf(mx, z[k]);
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            float se = 0.0f;
+            for (int k = lo + lane; k < hi; k += 32) se += __expf(z[k] - mx);
+            for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+            const float lse = mx + __logf(se);
+            total += lse - z[tgt];
+            __syncwarp();  // the zeros above and the columns of the last head come from other lanes
+            for (int k = lo + lane; k < hi; k += 32) {
+                const float g = (__expf(z[k] - lse) - (k == tgt ? 1.0f : 0.0f)) / (float)Bsz;
+                gb[k] = __float2bfloat16(g);
+                if (ACC) acc[k] += g;
+                else atomicAdd(&db[k], g);
+            }
+        }
+        __syncwarp();
     }
-    if (skip) return;
-    __syncwarp();
-    int tc = (nC > 0 && tC) ? tC[row] : -1;
-    if (tc >= nC) tc = -1;
-    const int nh = tc >= 0 ? 3 : 2;
-    for (int h = 0; h < nh; ++h) {
-        int lo, hi, tgt;
-        if (h == 0) { lo = 0; hi = nA; tgt = tA[row]; }
-        else if (h == 1) { lo = nA; hi = nA + nB; tgt = nA + tB[row]; }
-        else { lo = nA + nB + (tc / S) * S; hi = lo + S; tgt = nA + nB + tc; }
-        float mx = -3.0e38f;
-        for (int k = lo + lane; k < hi; k += 32) mx = fmaxf(mx, z[k]);
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float se = 0.0f;
-        for (int k = lo + lane; k < hi; k += 32) se += __expf(z[k] - mx);
-        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-        const float lse = mx + __logf(se);
-        total += lse - z[tgt];
-        for (int k = lo + lane; k < hi; k += 32) {
-            const float g = (__expf(z[k] - lse) - (k == tgt ? 1.0f : 0.0f)) / (float)Bsz;
-            gf[k] = g;
-            gb[k] = __float2bfloat16(g);
+    if (lane == 0 && total != 0.0f) atomicAdd(loss, total);
+    if (ACC) {
+        __syncthreads();
+        for (int k = (int)threadIdx.x; k < n_out; k += (int)blockDim.x) {
+            float t = 0.0f;
+            for (int w = 0; w < warps; ++w) t += s_acc[(size_t)w * n_out + k];
+            if (t != 0.0f) atomicAdd(&db[k], t);
         }
     }
-    if (lane == 0) atomicAdd(loss, total);
 }
 
-// db[n] += sum over the block's rows of dY[b, n]: blocks of 32 columns x 8 row
-// lanes, each block a contiguous range of rows; db must start at zero.
-__global__ void colsum_kernel(const float* __restrict__ dy, int Bsz, int N, int rows_per_block,
-                              float* __restrict__ db) {
-    __shared__ float part[8][33];
-    const int n = blockIdx.x * 32 + threadIdx.x;
-    const int r0 = blockIdx.y * rows_per_block, r1 = min(Bsz, r0 + rows_per_block);
-    float acc = 0.0f;
-    if (n < N)
-        for (int r = r0 + (int)threadIdx.y; r < r1; r += 8) acc += dy[(size_t)r * N + n];
-    part[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.y == 0 && n < N) {
-        float t = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t += part[i][threadIdx.x];
-        atomicAdd(&db[n], t);
+cudaError_t softmax_ce(const float* logits, int n_out, int nA, int nB, int nC, int S, const int* tA, const int* tB,
+                       const int* tC, int Bsz, __nv_bfloat16* dlogb, float* db, float* loss, cudaStream_t s) {
+    // at most 64 KiB of column sums a block (three blocks per SM), 8 warps while they fit
+    const size_t row = (size_t)n_out * sizeof(float);
+    const int warps = (int)std::max<size_t>(1, std::min<size_t>(8, (64u * 1024u) / row));
+    if (row > 200u * 1024u) {
+        softmax_ce_kernel<false><<<(Bsz + 7) / 8, 256, 0, s>>>(logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb,
+                                                              db, loss);
+        return cudaGetLastError();
     }
-}
-
-cudaError_t colsum(const float* dy, int Bsz, int N, float* db, cudaStream_t s) {
-    const int rpb = 256;
-    dim3 grid((N + 31) / 32, (Bsz + rpb - 1) / rpb);
-    colsum_kernel<<<grid, dim3(32, 8), 0, s>>>(dy, Bsz, N, rpb, db);
+    const size_t smem = row * warps;
+    cudaError_t e = cudaFuncSetAttribute(softmax_ce_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, nsm = 0, per_sm = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, softmax_ce_kernel<true>, warps * 32, smem)) !=
+            cudaSuccess)
+        return e;
+    const int blocks = std::min((Bsz + warps - 1) / warps, nsm * std::max(1, per_sm));
+    softmax_ce_kernel<true><<<blocks, warps * 32, smem, s>>>(logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb, db,
+                                                            loss);
     return cudaGetLastError();
 }
 
@@ -325,23 +341,16 @@ __global__ void to_bf16_kernel(uint64_t n, const float* __restrict__ w, __nv_bfl
     if (i < n) wb[i] = __float2bfloat16(w[i]);
 }
 
-// Work buffer (bytes, rows B a multiple of 64): H1 H2 H3 bf16 [B x 128] each,
-// dHf f32 [B x 128], dHb bf16 [B x 128] x2, logits f32 [B x n_out],
-// dlogf f32 [B x n_out], dlogb bf16 [B x n_out].
+// Work buffer (rows B a multiple of 64): H1 H2 H3 bf16 [B x 128] each, dHb bf16
+// [B x 128] x2, logits f32 [B x n_out], dlogb bf16 [B x n_out], XT bf16 [16 x B].
 struct MlpWork {
-    __nv_bfloat16 *H[3], *dHb[2], *dlogb;
-    float *dHf, *logits, *dlogf;
-    __nv_bfloat16 *dZT, *HT, *WT;  // transposed copies for the K-major products of the backward pass
+    __nv_bfloat16 *H[3], *dHb[2], *dlogb, *XT;
+    float* logits;
 };
 
-// The transposed copies serve every layer: dZT holds [n_out x B] and [128 x B],
-// WT holds [128 x n_out] and [128 x 128], so both take max(n_out, 128) rows.
 uint64_t mlp_work_bytes(int Bsz, int n_out) {
-    const uint64_t bh = (uint64_t)Bsz * kHid;
-    const uint64_t wide = (uint64_t)std::max(n_out, kHid);
-    return align256(bh * 2) * 5 + align256(bh * 4) + align256((uint64_t)Bsz * n_out * 4) * 2 +
-           align256((uint64_t)Bsz * n_out * 2) + align256((uint64_t)Bsz * wide * 2) + align256(bh * 2) +
-           align256(wide * kHid * 2);
+    return align256((uint64_t)Bsz * kHid * 2) * 5 + align256((uint64_t)Bsz * n_out * 4) +
+           align256((uint64_t)Bsz * n_out * 2) + align256((uint64_t)Bsz * kIn * 2);
 }
 
 MlpWork mlp_work(void* d_work, int Bsz, int n_out) {
@@ -350,13 +359,9 @@ MlpWork mlp_work(void* d_work, int Bsz, int n_out) {
     MlpWork w;
     for (int i = 0; i < 3; ++i) { w.H[i] = (__nv_bfloat16*)p; p += align256(bh * 2); }
     for (int i = 0; i < 2; ++i) { w.dHb[i] = (__nv_bfloat16*)p; p += align256(bh * 2); }
-    w.dHf = (float*)p; p += align256(bh * 4);
     w.logits = (float*)p; p += align256((uint64_t)Bsz * n_out * 4);
-    w.dlogf = (float*)p; p += align256((uint64_t)Bsz * n_out * 4);
     w.dlogb = (__nv_bfloat16*)p; p += align256((uint64_t)Bsz * n_out * 2);
-    w.dZT = (__nv_bfloat16*)p; p += align256((uint64_t)Bsz * std::max(n_out, kHid) * 2);  // [n_out or 128 x B]
-    w.HT = (__nv_bfloat16*)p; p += align256(bh * 2);                          // [128 x B] or [16 x B]
-    w.WT = (__nv_bfloat16*)p;                                                 // [128 x n_out or 128]
+    w.XT = (__nv_bfloat16*)p;
     return w;
 }
 
@@ -372,38 +377,45 @@ unsigned* tc_err_ptr() {
     return (unsigned*)a;
 }
 
-// C = epi(A W^T (+ bias)) on tcgen05 (umma.cuh): A [M x K], W [N x K], both K
-// contiguous; ksplit > 1 only with F32_ADD.  K <= 128 and not a multiple of 64
-// is staged by the threads, everything else by TMA.
-template <int EPI>
+// C = epi(A W^T (+ bias)) on tcgen05 (umma.cuh): A [M x K], W [N x K]; an operand
+// given MN-major lies as [K x M] (or [K x N]) row-major.  ksplit > 1 only with
+// F32_ADD.  K <= 128 and not a multiple of 64 is staged by the threads (K-major),
+// everything else by TMA.
+template <int EPI, bool MNA = false, bool MNB = false>
 cudaError_t gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* W, int ldw,
                     const float* bias, const __nv_bfloat16* mask, int ldmask, __nv_bfloat16* outb, float* outf,
-                    int ldc, cudaStream_t s, int ksplit = 1) {
+                    int ldc, cudaStream_t s, int ksplit = 1, float* colsum = nullptr) {
     unsigned* err = tc_err_ptr();
     if (!err || K % 16 || N % 16 || ksplit < 1 || (ksplit > 1 && EPI != umma::F32_ADD)) return cudaErrorInvalidValue;
     const int NT = std::min(256, N);
-    // two staging areas when a split has more than one K block of 128 (the copy
-    // of the next block overlaps the products of this one)
+    if (MNB && NT % 64) return cudaErrorInvalidValue;
+    const bool staged = !MNA && !MNB && K <= 128 && K % umma::kPanel != 0;
+    if (staged && ksplit != 1) return cudaErrorInvalidValue;
+    // panels in flight: three of a split (two CTAs per SM), up to six where one
+    // CTA runs the whole of a long K
     const int kpanels = (K + umma::kPanel - 1) / umma::kPanel;
     const int per_split = (kpanels + ksplit - 1) / ksplit;
-    const bool staged_k = K <= 128 && K % umma::kPanel != 0;
-    const int nstage = (!staged_k && per_split > umma::kMaxPanels) ? 2 : 1;
+    int nstage = staged ? 2 : std::min(per_split, ksplit > 1 ? 3 : umma::kMaxStages);
+    while (nstage > 2 && umma::smem_bytes(NT, nstage, MNB) > 200u * 1024u) --nstage;
     // at least 80 KiB of shared memory: at most two CTAs per SM, so their TMEM
     // accumulators (<= 256 columns each) always fit the SM's 512 columns
-    const size_t smem = std::max<size_t>(umma::smem_bytes(NT, nstage), 80 * 1024);
+    const size_t smem = std::max<size_t>(umma::smem_bytes(NT, nstage, MNB), 80 * 1024);
     dim3 grid((N + NT - 1) / NT, (M + umma::kTileM - 1) / umma::kTileM, ksplit);
     CUtensorMap mapA, mapW;
     std::memset(&mapA, 0, sizeof(mapA));
     std::memset(&mapW, 0, sizeof(mapW));
-    const bool staged = K <= 128 && K % umma::kPanel != 0;
-    if (staged && ksplit != 1) return cudaErrorInvalidValue;
-    if (!staged && !(umma::make_map(&mapA, A, M, K, lda, umma::kTileM) && umma::make_map(&mapW, W, N, K, ldw, NT)))
+    if (!staged && !((MNA ? umma::make_map(&mapA, A, K, M, lda, umma::kPanel)
+                          : umma::make_map(&mapA, A, M, K, lda, umma::kTileM)) &&
+                     (MNB ? umma::make_map(&mapW, W, K, N, ldw, umma::kPanel)
+                          : umma::make_map(&mapW, W, N, K, ldw, NT))))
         return cudaErrorInvalidValue;
-    auto kern = staged ? umma::gemm_tc_kernel<EPI, false> : umma::gemm_tc_kernel<EPI, true>;
+    auto kern = umma::gemm_tc_kernel<EPI, true, MNA, MNB>;
+    if constexpr (!MNA && !MNB)
+        if (staged) kern = umma::gemm_tc_kernel<EPI, false, false, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, umma::kThreads, smem, s>>>(M, N, K, NT, A, lda, W, ldw, mapA, mapW, bias, mask, ldmask, outb, outf,
-                                            ldc, nstage, err);
+                                            ldc, colsum, nstage, err);
     return cudaGetLastError();
 }
 
@@ -415,7 +427,7 @@ cudaError_t transpose(const __nv_bfloat16* in, int rows, int cols, int ld_in, __
 }
 
 cudaError_t mlp_forward(int n_out, const float* wf, const __nv_bfloat16* wb, const __nv_bfloat16* X, int Bsz,
-                        const MlpWork& w, cudaStream_t s) {
+                        const MlpWork& w, float* logits, cudaStream_t s) {
     const MlpOffsets o = mlp_offsets(n_out);
     cudaError_t e;
     if ((e = gemm_tc<umma::RELU_BF16>(Bsz, kHid, kIn, X, kIn, wb + o.W[0], kIn, wf + o.b[0], nullptr, 0, w.H[0],
@@ -426,7 +438,7 @@ cudaError_t mlp_forward(int n_out, const float* wf, const __nv_bfloat16* wb, con
                                           nullptr, 0, w.H[l], nullptr, kHid, s)) != cudaSuccess)
             return e;
     return gemm_tc<umma::LINEAR_F32>(Bsz, n_out, kHid, w.H[2], kHid, wb + o.W[3], kHid, wf + o.b[3], nullptr, 0,
-                                     nullptr, w.logits, n_out, s);
+                                     nullptr, logits, n_out, s);
 }
 
 }  // namespace
@@ -453,12 +465,10 @@ int rddmc_mlp_forward(int n_out, const float* d_wf, const void* d_wb, const void
         return RDDMC_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const MlpWork w = mlp_work(d_work, batch, n_out);
-    if (mlp_forward(n_out, d_wf, (const __nv_bfloat16*)d_wb, (const __nv_bfloat16*)d_x, batch, w, s) != cudaSuccess)
-        return RDDMC_ERR_CUDA;
-    if (d_logits && cudaMemcpyAsync(d_logits, w.logits, (size_t)batch * n_out * 4, cudaMemcpyDeviceToDevice, s) !=
-                        cudaSuccess)
-        return RDDMC_ERR_CUDA;
-    return RDDMC_OK;
+    return mlp_forward(n_out, d_wf, (const __nv_bfloat16*)d_wb, (const __nv_bfloat16*)d_x, batch, w,
+                       d_logits ? d_logits : w.logits, s) == cudaSuccess
+               ? RDDMC_OK
+               : RDDMC_ERR_CUDA;
 }
 
 int rddmc_mlp_loss_grad(int n_out, int nA, int nB, int nC, int S, const float* d_wf, const void* d_wb,
@@ -473,45 +483,37 @@ int rddmc_mlp_loss_grad(int n_out, int nA, int nB, int nC, int S, const float* d
     const __nv_bfloat16* wb = (const __nv_bfloat16*)d_wb;
     const __nv_bfloat16* X = (const __nv_bfloat16*)d_x;
     const MlpWork w = mlp_work(d_work, batch, n_out);
-    if (mlp_forward(n_out, d_wf, wb, X, batch, w, s) != cudaSuccess) return RDDMC_ERR_CUDA;
+    if (mlp_forward(n_out, d_wf, wb, X, batch, w, w.logits, s) != cudaSuccess) return RDDMC_ERR_CUDA;
     if (cudaMemsetAsync(d_loss, 0, 4, s) != cudaSuccess) return RDDMC_ERR_CUDA;
-    softmax_ce_kernel<<<(batch + 7) / 8, 256, 0, s>>>(w.logits, n_out, nA, nB, nC, S, d_ta, d_tb,
-                                                       nC > 0 ? d_tc : nullptr, batch, w.dlogf, w.dlogb, d_loss);
     // gradients accumulate (split-K products, column sums) into a zeroed buffer
     if (cudaMemsetAsync(d_grad, 0, o.total * sizeof(float), s) != cudaSuccess) return RDDMC_ERR_CUDA;
-    // Every product runs on tcgen05 with K contiguous in both operands:
-    //   dW = dZ^T H     as (dZ^T [out x B]) (H^T [in x B])^T, K = batch, split over K
-    //   dH = (dZ W) .* [H > 0]  as (dZ [B x out]) (W^T [in x out])^T, K = out
+    // Every product runs on tcgen05 with the operands as they lie in memory:
+    //   dW = dZ^T H             A = dZ [B x out] and W = H [B x in], both MN-major, K = batch, split over K
+    //   dH = (dZ W) .* [H > 0]  A = dZ [B x out], W = W [out x in] MN-major, K = out
+    // and the masked epilogue adds the columns of dH to the next bias gradient.
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    chk(softmax_ce(w.logits, n_out, nA, nB, nC, S, d_ta, d_tb, nC > 0 ? d_tc : nullptr, batch, w.dlogb,
+                   d_grad + o.b[3], d_loss, s));
     // output layer
-    chk(transpose(w.dlogb, batch, n_out, n_out, w.dZT, batch, s));
-    chk(transpose(w.H[2], batch, kHid, kHid, w.HT, batch, s));
-    chk(gemm_tc<umma::F32_ADD>(n_out, kHid, batch, w.dZT, batch, w.HT, batch, nullptr, nullptr, 0, nullptr,
-                               d_grad + o.W[3], kHid, s, ksplit_for(n_out, kHid, batch)));
-    chk(colsum(w.dlogf, batch, n_out, d_grad + o.b[3], s));
-    chk(transpose(wb + o.W[3], n_out, kHid, kHid, w.WT, n_out, s));
-    chk(gemm_tc<umma::MASK_BF16>(batch, kHid, n_out, w.dlogb, n_out, w.WT, n_out, nullptr, w.H[2], kHid, w.dHb[0],
-                                 w.dHf, kHid, s));
+    chk(gemm_tc<umma::F32_ADD, true, true>(n_out, kHid, batch, w.dlogb, n_out, w.H[2], kHid, nullptr, nullptr, 0,
+                                           nullptr, d_grad + o.W[3], kHid, s, ksplit_for(n_out, kHid, batch)));
+    chk(gemm_tc<umma::MASK_BF16, false, true>(batch, kHid, n_out, w.dlogb, n_out, wb + o.W[3], kHid, nullptr, w.H[2],
+                                              kHid, w.dHb[0], nullptr, kHid, s, 1, d_grad + o.b[2]));
     int cur = 0;
     for (int l = 2; l >= 1; --l) {
         // layer l (W[l]: H[l-1] -> H[l]); dHb[cur] holds dL/d(pre-activation of H[l])
-        chk(transpose(w.dHb[cur], batch, kHid, kHid, w.dZT, batch, s));
-        chk(transpose(w.H[l - 1], batch, kHid, kHid, w.HT, batch, s));
-        chk(gemm_tc<umma::F32_ADD>(kHid, kHid, batch, w.dZT, batch, w.HT, batch, nullptr, nullptr, 0, nullptr,
-                                   d_grad + o.W[l], kHid, s, ksplit_for(kHid, kHid, batch)));
-        chk(colsum(w.dHf, batch, kHid, d_grad + o.b[l], s));
-        chk(transpose(wb + o.W[l], kHid, kHid, kHid, w.WT, kHid, s));
-        chk(gemm_tc<umma::MASK_BF16>(batch, kHid, kHid, w.dHb[cur], kHid, w.WT, kHid, nullptr, w.H[l - 1], kHid,
-                                     w.dHb[cur ^ 1], w.dHf, kHid, s));
+        chk(gemm_tc<umma::F32_ADD, true, true>(kHid, kHid, batch, w.dHb[cur], kHid, w.H[l - 1], kHid, nullptr, nullptr,
+                                               0, nullptr, d_grad + o.W[l], kHid, s, ksplit_for(kHid, kHid, batch)));
+        chk(gemm_tc<umma::MASK_BF16, false, true>(batch, kHid, kHid, w.dHb[cur], kHid, wb + o.W[l], kHid, nullptr,
+                                                  w.H[l - 1], kHid, w.dHb[cur ^ 1], nullptr, kHid, s, 1,
+                                                  d_grad + o.b[l - 1]));
         cur ^= 1;
     }
-    // input layer: dW1 = dZ1^T X
-    chk(transpose(w.dHb[cur], batch, kHid, kHid, w.dZT, batch, s));
-    chk(transpose(X, batch, kIn, kIn, w.HT, batch, s));
-    chk(gemm_tc<umma::F32_ADD>(kHid, kIn, batch, w.dZT, batch, w.HT, batch, nullptr, nullptr, 0, nullptr,
-                               d_grad + o.W[0], kIn, s, ksplit_for(kHid, kIn, batch)));
-    chk(colsum(w.dHf, batch, kHid, d_grad + o.b[0], s));
+    // input layer: dW1 = dZ1^T X (16 columns, short of a box: a K-major copy)
+    chk(transpose(X, batch, kIn, kIn, w.XT, batch, s));
+    chk(gemm_tc<umma::F32_ADD, true, false>(kHid, kIn, batch, w.dHb[cur], kHid, w.XT, batch, nullptr, nullptr, 0,
+                                            nullptr, d_grad + o.W[0], kIn, s, ksplit_for(kHid, kIn, batch)));
     if (e != cudaSuccess) return RDDMC_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? RDDMC_OK : RDDMC_ERR_CUDA;
 }

@@ -1,22 +1,27 @@
 // umma.cuh -- dense BF16 products on the 5th-generation tensor cores
 // (tcgen05.mma, FP32 accumulators in tensor memory) for the learned proposal's
-// network: C[M x N] = A[M x K] W[N x K]^T (+ bias, epilogue), both operands
-// row-major with K contiguous ("K-major"), K a multiple of 16.
+// network: C[M x N] = A[M x K] W[N x K]^T (+ bias, epilogue).  Each operand is
+// read as it lies in memory: K contiguous ("K-major", a row per M or N index) or
+// M or N contiguous ("MN-major", a row per K index), so that the backward
+// products need no transposed copies.
 //
 // One CTA of 128 threads computes a 128 x NT tile (NT <= 256, a multiple of
-// 16), over K in blocks of 128 (two 64-column panels), optionally a range of
-// K per blockIdx.z (split-K).  A block of A and W is staged in shared memory
-// in the 128-byte swizzled K-major layout (rows of 64 BF16 = 128 B, eight-row
-// atoms of 1 KiB, 16-byte chunk c of row r stored at chunk c ^ (r mod 8)): by
-// TMA (cp.async.bulk.tensor with 128-byte swizzle; rows and columns past the
-// matrix filled with zeros by the copy engine), or by the threads for a single
-// block with K not a multiple of 64.  One elected thread issues the block's
-// tcgen05.mma instructions into a TMEM accumulator of 128 lanes x NT columns,
-// commits them to an mbarrier and waits before reusing the shared memory;
-// after the last block every warp reads its 32 lanes back with tcgen05.ld and
-// turns each 32 x 32 block around in shared memory, so that the epilogue's
-// stores run along rows.  Waits are bounded: a wait that runs out sets the
-// error word and the tile's outputs are left unwritten.
+// 16; of 64 when W is MN-major), over K in panels of 64, optionally a range of
+// them per blockIdx.z (split-K).  A panel of A and W is staged in shared memory
+// by TMA (cp.async.bulk.tensor with 128-byte swizzle, elements past the matrix
+// filled with zeros by the copy engine), or by the threads for a single K-major
+// block of K <= 128 that is not a multiple of 64:
+//   K-major:  rows of 64 BF16 = 128 B, eight-row atoms of 1 KiB, 16-byte chunk c
+//             of row r at chunk c ^ (r mod 8); one box of all rows;
+//   MN-major: boxes of 64 M (or N) indices x 64 K rows, 8 KiB each, in the same
+//             atoms of eight K rows.
+// One elected thread keeps nstage panels in flight, issues each panel's four
+// tcgen05.mma into a TMEM accumulator of 128 lanes x NT columns and commits them
+// to the mbarrier that frees the stage.  After the last panel every warp reads
+// its 32 lanes back with tcgen05.ld and turns each 32 x 32 block around in shared
+// memory, so that the epilogue's stores run along rows.  Waits are bounded: a
+// wait that runs out sets the error word and the tile's outputs are left
+// unwritten.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -29,29 +34,33 @@ namespace umma {
 constexpr int kTileM = 128;
 constexpr int kThreads = 128;
 constexpr int kPanel = 64;  // BF16 per 128-byte swizzled row
-constexpr int kMaxPanels = 2;  // a K block is at most 128 wide
+constexpr int kMaxStages = 6;
+constexpr uint32_t kBoxBytes = 8192;  // an MN-major box: 64 K rows of 128 B
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Shared-memory matrix descriptor: start address, leading byte offset (unused
-// by swizzled K-major layouts, set to 16 B), stride byte offset between
-// eight-row atoms (1 KiB), descriptor version 1, 128-byte swizzle.
+// Shared-memory matrix descriptor: start address, leading byte offset (between
+// boxes of 64 M or N indices of an MN-major operand; unused by swizzled K-major
+// layouts, set to 16 B), stride byte offset between eight-row atoms (1 KiB),
+// descriptor version 1, 128-byte swizzle.
+template <bool MN>
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)(16u >> 4) << 16;
+    d |= (uint64_t)((MN ? kBoxBytes : 16u) >> 4) << 16;
     d |= (uint64_t)(1024u >> 4) << 32;
     d |= (uint64_t)1u << 46;
     d |= (uint64_t)2u << 61;
     return d;
 }
 
-// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N >> 3 and M >> 4.
-__host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, each
+// K-major or MN-major (transpose bits 15 and 16), N >> 3 and M >> 4.
+__host__ __device__ constexpr uint32_t instr_desc(int m, int n, bool mn_a, bool mn_b) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((mn_a ? 1u : 0u) << 15) | ((mn_b ? 1u : 0u) << 16) |
+           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 __host__ __device__ constexpr int tmem_cols(int nt) {
@@ -98,16 +107,18 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
-// Issue the tcgen05.mma instructions of one staged block: `slices` K-slices of
-// 16 (four per 64-column panel), the first of them overwriting the accumulator
-// when `first`.
-__device__ __forceinline__ void mma_block(uint32_t tmem, unsigned char* sA, unsigned char* sB, int NT, int slices,
-                                          bool first) {
-    const uint32_t idesc = instr_desc(kTileM, NT);
+// Issue the tcgen05.mma instructions of `slices` K-slices of 16 (four per panel;
+// panels panel_a and panel_b bytes apart, for the thread-staged block), the
+// first of them overwriting the accumulator when `first`.
+template <bool MNA, bool MNB>
+__device__ __forceinline__ void mma_panel(uint32_t tmem, unsigned char* sA, unsigned char* sB, int NT, int slices,
+                                          bool first, uint32_t panel_a, uint32_t panel_b) {
+    const uint32_t idesc = instr_desc(kTileM, NT, MNA, MNB);
     for (int s = 0; s < slices; ++s) {
-        const int p = s >> 2, off = (s & 3) * 32;  // panel, byte offset of the 16-wide K slice
-        const uint64_t ad = smem_desc(smem_u32(sA + (size_t)p * kTileM * 128 + off));
-        const uint64_t bd = smem_desc(smem_u32(sB + (size_t)p * NT * 128 + off));
+        // 16 K indices further: 32 bytes along a K-major row, 16 rows of an MN-major box
+        const uint32_t p = (uint32_t)(s >> 2), k = (uint32_t)(s & 3);
+        const uint64_t ad = smem_desc<MNA>(smem_u32(sA) + p * panel_a + k * (MNA ? 2048u : 32u));
+        const uint64_t bd = smem_desc<MNB>(smem_u32(sB) + p * panel_b + k * (MNB ? 2048u : 32u));
         const uint32_t acc = (first && s == 0) ? 0u : 1u;
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -116,15 +127,25 @@ __device__ __forceinline__ void mma_block(uint32_t tmem, unsigned char* sA, unsi
     }
 }
 
-// C = epi(A W^T (+ bias)) for A [M x K], W [N x K], both K contiguous.
-// Grid: (ceil(N / NT), ceil(M / 128), ksplit); blockIdx.z takes a range of K
-// in blocks of 128 (64-column panels).  TMA path: tensor maps mapA (box 64 x
-// 128) and mapW (box 64 x NT), any K (columns past K are zero-filled);
-// thread-staged path: K <= 128.  Epilogues: RELU_BF16 and LINEAR_F32 add the
-// bias; MASK_BF16 keeps entries where mask > 0 and writes them to outb (BF16)
-// and outf (FP32); F32_ADD adds into outf (split-K partial sums).  err: set
-// to 1 when a wait ran out (the tile's outputs are then left unwritten).
-template <int EPI, bool TMA>
+__device__ __forceinline__ void commit_to(uint64_t* mbar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                 :: "r"(smem_u32(mbar)));
+}
+
+// Bytes of a stage's W panel.
+__host__ __device__ constexpr uint32_t w_bytes(int NT, bool mn_b) {
+    return mn_b ? (uint32_t)((NT + 63) / 64) * kBoxBytes : (uint32_t)NT * 128u;
+}
+
+// C = epi(A W^T (+ bias)).  Grid: (ceil(N / NT), ceil(M / 128), ksplit);
+// blockIdx.z takes a range of K in 64-wide panels.  TMA path: tensor maps mapA
+// and mapW (boxes of 64 columns x all tile rows when K-major, x 64 rows when
+// MN-major); thread-staged path: K <= 128, both K-major.  Epilogues: RELU_BF16
+// and LINEAR_F32 add the bias; MASK_BF16 keeps entries where mask > 0, writes
+// them to outb (BF16) and adds their FP32 column sums to colsum; F32_ADD adds
+// into outf (split-K partial sums).  err: set to 1 when a wait ran out (the
+// tile's outputs are then left unwritten).
+template <int EPI, bool TMA, bool MNA, bool MNB>
 __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, int NT,
                                                            const __nv_bfloat16* __restrict__ A, int lda,
                                                            const __nv_bfloat16* __restrict__ W, int ldw,
@@ -133,18 +154,23 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
                                                            const float* __restrict__ bias,
                                                            const __nv_bfloat16* __restrict__ mask, int ldmask,
                                                            __nv_bfloat16* __restrict__ outb, float* __restrict__ outf,
-                                                           int ldc, int nstage, unsigned* err) {
+                                                           int ldc, float* __restrict__ colsum, int nstage,
+                                                           unsigned* err) {
+    static_assert(TMA || (!MNA && !MNB), "the thread-staged block is K-major");
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    // nstage (1 or 2) staging areas of one K block each: A panels, then W panels
-    const size_t stage_bytes = (size_t)kMaxPanels * (kTileM + NT) * 128;
-    unsigned char* sA = base;  // stage 0's A panels (also the epilogue's scratch)
-    auto stage_a = [&](int st) { return base + (size_t)st * stage_bytes; };
-    auto stage_b = [&](int st) { return base + (size_t)st * stage_bytes + (size_t)kMaxPanels * kTileM * 128; };
-    // per stage: tbar (its TMA copy landed) and mbar (its products completed)
-    uint64_t* tbar = reinterpret_cast<uint64_t*>(base + (size_t)nstage * stage_bytes);
-    uint64_t* mbar = tbar + 2;
-    uint32_t* taddr_s = reinterpret_cast<uint32_t*>(tbar + 4);
+    // nstage staging areas of one panel each: A, then W
+    constexpr uint32_t a_bytes = kTileM * 128;
+    const uint32_t b_bytes = w_bytes(NT, MNB);
+    unsigned char* sA = base;  // also the epilogue's scratch
+    auto stage_a = [&](int st) { return base + (size_t)st * (a_bytes + b_bytes); };
+    auto stage_b = [&](int st) { return base + (size_t)st * (a_bytes + b_bytes) + a_bytes; };
+    // per stage: full (its copies landed) and empty (its products completed);
+    // then the barrier of the last products
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + (size_t)nstage * (a_bytes + b_bytes));
+    uint64_t* empty = full + kMaxStages;
+    uint64_t* last = empty + kMaxStages;
+    uint32_t* taddr_s = reinterpret_cast<uint32_t*>(last + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * kTileM, n0 = blockIdx.x * NT;
@@ -161,12 +187,13 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 4; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(tbar + i)));
+        for (int i = 0; i < 2 * kMaxStages + 1; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(full + i)));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (!TMA) {  // one block: K <= 128
         stage(A, lda, m0, kTileM, min(kTileM, M - m0), K, stage_a(0));
-        stage(W, ldw, n0, NT, min(NT, N - n0), K, stage_b(0));
+        stage(W, ldw, n0, NT, min(NT, N - n0), K, base + 2 * a_bytes);
         asm volatile("fence.proxy.async.shared::cta;");  // generic-proxy stores -> tensor-core reads
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -174,78 +201,59 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *taddr_s;
 
-    // One thread stages (TMA), issues and waits.  With two stages the copy of
-    // K block b+1 is issued as soon as its stage is free (the products of block
-    // b-1 completed), so it lands while block b's products run; with one stage
-    // each block is copied, multiplied and waited for in turn.  Use k of a
-    // stage completes phase k of its two mbarriers (parity k & 1); a stage is
+    // One thread copies (TMA), issues and waits.  Panel p uses stage p mod
+    // nstage; its copy is issued once the products of panel p - nstage have
+    // completed, nstage panels ahead of the products at most.  Use k of a stage
+    // completes phase k of its two barriers (parity k & 1), and a stage is
     // rewritten only after its previous use was waited for, so no barrier runs
     // two phases ahead of its wait.
     __shared__ int ok_s;
     if (threadIdx.x == 0) {
         bool ok = true;
         if (TMA) {
-            const int nb = (p_end - p_begin + kMaxPanels - 1) / kMaxPanels;
-            auto issue = [&](int blk) {
-                const int st = nstage == 2 ? (blk & 1) : 0;
-                const int p = p_begin + blk * kMaxPanels;
-                const int np = min(kMaxPanels, p_end - p);
-                const uint32_t bytes = (uint32_t)(np * (kTileM + NT) * 128);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                             :: "r"(smem_u32(tbar + st)), "r"(bytes) : "memory");
-                for (int q = 0; q < np; ++q) {
-                    tma_load_2d(stage_a(st) + (size_t)q * kTileM * 128, &mapA, (p + q) * kPanel, m0, tbar + st);
-                    tma_load_2d(stage_b(st) + (size_t)q * NT * 128, &mapW, (p + q) * kPanel, n0, tbar + st);
-                }
-            };
-            int pend = 0;  // copies issued and not yet waited for
-            issue(0);
-            pend = 1;
-            int b = 0;
-            for (; b < nb; ++b) {
-                const int st = nstage == 2 ? (b & 1) : 0;
-                const uint32_t use = nstage == 2 ? (uint32_t)(b >> 1) : (uint32_t)b;
-                if (nstage == 2 && b + 1 < nb) {
-                    // stage of block b+1 last held block b-1: wait for its products
-                    if (b >= 1 && !(ok = wait_parity(mbar + ((b + 1) & 1), (uint32_t)((b - 1) >> 1) & 1u))) break;
-                    issue(b + 1);
-                    ++pend;
-                }
-                if (!(ok = wait_parity(tbar + st, use & 1u))) break;
-                --pend;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const int np = min(kMaxPanels, p_end - (p_begin + b * kMaxPanels));
-                mma_block(tmem, stage_a(st), stage_b(st), NT, 4 * np, b == 0);  // columns past K were zero-filled
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(smem_u32(mbar + st)));
-                if (nstage == 1) {
-                    if (!(ok = wait_parity(mbar, use & 1u))) break;
-                    if (b + 1 < nb) {
-                        issue(b + 1);
-                        ++pend;
+            const int np = p_end - p_begin;
+            int issued = 0, landed = 0;
+            for (int p = 0; p < np && ok; ++p) {
+                while (issued < np && issued < p + nstage) {
+                    const int st = issued % nstage, use = issued / nstage;
+                    if (use > 0 && !(ok = wait_parity(empty + st, (uint32_t)(use - 1) & 1u))) break;
+                    const int k = (p_begin + issued) * kPanel;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                                 :: "r"(smem_u32(full + st)), "r"(a_bytes + b_bytes) : "memory");
+                    if (MNA) {
+                        for (int c = 0; c < kTileM / 64; ++c)
+                            tma_load_2d(stage_a(st) + c * kBoxBytes, &mapA, m0 + 64 * c, k, full + st);
+                    } else {
+                        tma_load_2d(stage_a(st), &mapA, k, m0, full + st);
                     }
+                    if (MNB) {
+                        for (int c = 0; c < (NT + 63) / 64; ++c)
+                            tma_load_2d(stage_b(st) + c * kBoxBytes, &mapW, n0 + 64 * c, k, full + st);
+                    } else {
+                        tma_load_2d(stage_b(st), &mapW, k, n0, full + st);
+                    }
+                    ++issued;
                 }
+                if (!ok) break;
+                const int st = p % nstage;
+                if (!(ok = wait_parity(full + st, (uint32_t)(p / nstage) & 1u))) break;
+                ++landed;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                mma_panel<MNA, MNB>(tmem, stage_a(st), stage_b(st), NT, 4, p == 0, 0u, 0u);
+                commit_to(empty + st);
             }
-            if (ok && nstage == 2) {
-                // the last commit covers every product issued before it
-                const int bl = nb - 1;
-                ok = wait_parity(mbar + (bl & 1), (uint32_t)(bl >> 1) & 1u);
+            if (ok) {
+                commit_to(last);  // covers every product issued before it
+                ok = wait_parity(last, 0);
             }
-            if (!ok) {
-                // a wait ran out: give the copies still in flight another bounded
-                // wait before the CTA leaves (their stages' next phases)
-                for (int i = 0; i < pend && i < 2; ++i) {
-                    const int blk = b + i;  // the copies of blocks b (and b+1) were issued, not waited
-                    const int st = nstage == 2 ? (blk & 1) : 0;
-                    const uint32_t use = nstage == 2 ? (uint32_t)(blk >> 1) : (uint32_t)blk;
-                    wait_parity(tbar + st, use & 1u);
-                }
-            }
+            // a wait ran out: give the copies still in flight another bounded wait
+            // before the CTA leaves
+            for (int p = landed; !ok && p < issued; ++p) wait_parity(full + p % nstage, (uint32_t)(p / nstage) & 1u);
         } else {
-            mma_block(tmem, stage_a(0), stage_b(0), NT, K / 16, true);  // only the staged K columns
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(mbar)));
-            ok = wait_parity(mbar, 0);
+            // only the staged K columns
+            mma_panel<false, false>(tmem, stage_a(0), base + 2 * a_bytes, NT, K / 16, true, a_bytes, (uint32_t)NT * 128u);
+            commit_to(last);
+            ok = wait_parity(last, 0);
         }
         if (!ok) atomicOr(err, 1u);
         ok_s = ok ? 1 : 0;
@@ -294,6 +302,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
             const int n = n0 + c0 + lane;
             const bool col_ok = c0 + lane < NT && n < N;
             const float b = (col_ok && (EPI == RELU_BF16 || EPI == LINEAR_F32)) ? bias[n] : 0.0f;
+            float csum = 0.0f;
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
                 const int row = m0 + warp * 32 + r;
@@ -307,11 +316,12 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
                 } else if (EPI == MASK_BF16) {
                     const float y = mk[r] > 0.0f ? x : 0.0f;
                     outb[o] = __float2bfloat16(y);
-                    outf[o] = y;
+                    csum += y;
                 } else {
                     atomicAdd(&outf[o], x);
                 }
             }
+            if (EPI == MASK_BF16 && col_ok) atomicAdd(&colsum[n], csum);
             __syncwarp();
         }
     }
@@ -340,11 +350,11 @@ __global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in, int 
     }
 }
 
-// Dynamic shared memory of a 128 x NT tile with `stages` staging areas of two
-// 64-column panels of A and W each (+1 KiB alignment slack, four mbarriers and
-// the TMEM address).
-__host__ __device__ constexpr size_t smem_bytes(int nt, int stages) {
-    return 1024 + (size_t)stages * kMaxPanels * (kTileM + nt) * 128 + 64;
+// Dynamic shared memory of a 128 x NT tile with `stages` panels of A and W (+1 KiB
+// alignment slack, the barriers and the TMEM address); the thread-staged block
+// takes two panels of each.
+__host__ __device__ constexpr size_t smem_bytes(int nt, int stages, bool mn_b) {
+    return 1024 + (size_t)stages * (kTileM * 128 + w_bytes(nt, mn_b)) + (2 * kMaxStages + 2) * 8;
 }
 
 // 2D BF16 tensor map of a row-major [rows x cols] matrix with leading

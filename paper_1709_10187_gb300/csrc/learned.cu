@@ -259,14 +259,17 @@ __global__ void softmax_ce_kernel(const float* __restrict__ logits, int n_out, i
             else if (h == 1) { lo = nA; hi = nA + nB; tgt = nA + tB[row]; }
             else { lo = nA + nB + (tc / S) * S; hi = lo + S; tgt = nA + nB + tc; }
             float mx = -3.0e38f;
+#pragma unroll 8
             for (int k = lo + lane; k < hi; k += 32) mx = fmaxf(mx, z[k]);
             for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             float se = 0.0f;
+#pragma unroll 8
             for (int k = lo + lane; k < hi; k += 32) se += __expf(z[k] - mx);
             for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
             const float lse = mx + __logf(se);
             total += lse - z[tgt];
             __syncwarp();  // the zeros above and the columns of the last head come from other lanes
+#pragma unroll 8
             for (int k = lo + lane; k < hi; k += 32) {
                 const float g = (__expf(z[k] - lse) - (k == tgt ? 1.0f : 0.0f)) / (float)Bsz;
                 gb[k] = __float2bfloat16(g);
@@ -389,6 +392,7 @@ cudaError_t gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const 
     if (!err || K % 16 || N % 16 || ksplit < 1 || (ksplit > 1 && EPI != umma::F32_ADD)) return cudaErrorInvalidValue;
     const int NT = std::min(256, N);
     if (MNB && NT % 64) return cudaErrorInvalidValue;
+    if ((EPI == umma::RELU_BF16 || EPI == umma::MASK_BF16) && N != kHid) return cudaErrorInvalidValue;
     const bool staged = !MNA && !MNB && K <= 128 && K % umma::kPanel != 0;
     if (staged && ksplit != 1) return cudaErrorInvalidValue;
     // panels in flight: three of a split (two CTAs per SM), up to six where one

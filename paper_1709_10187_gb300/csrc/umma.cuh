@@ -18,8 +18,8 @@
 // One elected thread keeps nstage panels in flight, issues each panel's four
 // tcgen05.mma into a TMEM accumulator of 128 lanes x NT columns and commits them
 // to the mbarrier that frees the stage.  After the last panel every warp reads
-// its 32 lanes back with tcgen05.ld and turns each 32 x 32 block around in shared
-// memory, so that the epilogue's stores run along rows.  Waits are bounded: a
+// its 32 lanes back with tcgen05.ld; FP32 outputs are turned around in shared
+// memory, 32 x 32 at a time, so that their stores run along rows.  Waits are bounded: a
 // wait that runs out sets the error word and the tile's outputs are left
 // unwritten.
 #pragma once
@@ -130,6 +130,24 @@ __device__ __forceinline__ void mma_panel(uint32_t tmem, unsigned char* sA, unsi
 __device__ __forceinline__ void commit_to(uint64_t* mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  :: "r"(smem_u32(mbar)));
+}
+
+// 32 accumulator columns of this warp's 32 TMEM lanes: thread t's row.
+__device__ __forceinline__ void load_acc32(uint32_t ta, float* v) {
+    uint32_t u[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+          "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]),
+          "=r"(u[15]), "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]),
+          "=r"(u[22]), "=r"(u[23]), "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]),
+          "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+        : "r"(ta));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]);
 }
 
 // Bytes of a stage's W panel.
@@ -261,7 +279,61 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok_s) {
+    if (ok_s && (EPI == RELU_BF16 || EPI == MASK_BF16)) {
+        // thread t of warp w holds row m0 + 32 w + t: its BF16 outputs are 64
+        // contiguous bytes per 32 columns, so it stores (and reads the mask) in
+        // 16-byte pieces.  N is 128 here: a tile's columns are all there.
+        const int row = m0 + warp * 32 + lane;
+        const bool row_ok = row < M;
+        uint4 mk[4][4];
+        if (EPI == MASK_BF16) {  // all of the row's mask in flight together
+            const uint4* mrow = reinterpret_cast<const uint4*>(mask + (size_t)min(row, M - 1) * ldmask + n0);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mk[c][i] = mrow[4 * c + i];
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float v[32];
+            load_acc32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(32 * c), v);
+            uint32_t packed[16];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                if (EPI == RELU_BF16) {
+                    v[j] = fmaxf(v[j] + bias[n0 + 32 * c + j], 0.0f);
+                } else {
+                    const uint32_t w = (&mk[c][j >> 3].x)[(j >> 1) & 3];
+                    const float h = __uint_as_float((j & 1) ? (w & 0xffff0000u) : (w << 16));
+                    v[j] = (h > 0.0f && row_ok) ? v[j] : 0.0f;
+                }
+                if (j & 1) {
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[j - 1], v[j]);
+                    packed[j >> 1] = *reinterpret_cast<const uint32_t*>(&b2);
+                }
+            }
+            if (row_ok) {
+                uint4* o = reinterpret_cast<uint4*>(outb + (size_t)row * ldc + n0 + 32 * c);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    o[i] = make_uint4(packed[4 * i], packed[4 * i + 1], packed[4 * i + 2], packed[4 * i + 3]);
+            }
+            if (EPI == MASK_BF16) {
+                // column sums over the warp's 32 rows: halve the columns a lane holds
+                // at every exchange, until lane l holds the sum of column l
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1) {
+                    const bool up = (lane & w) != 0;
+#pragma unroll
+                    for (int j = 0; j < w; ++j) {
+                        const float keep = up ? v[j + w] : v[j], send = up ? v[j] : v[j + w];
+                        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+                    }
+                }
+                atomicAdd(&colsum[n0 + 32 * c + lane], v[0]);
+            }
+        }
+    } else if (ok_s) {
         // warp w reads TMEM lanes 32w..32w+31 (thread t holds row m0 + 32w + t,
         // 32 columns at a time), then turns each 32 x 32 block around through
         // shared memory (the operand staging area, free now that the products
@@ -270,58 +342,23 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(int M, int N, int K, 
         // columns of one row
         float* st = reinterpret_cast<float*>(sA) + warp * (32 * 33);
         for (int c0 = 0; c0 < NT; c0 += 32) {
-            // the ReLU mask of this warp's 32 rows at column n0 + c0 + lane, loaded
-            // before the accumulator so that the 32 loads are in flight together
-            // (indices clamped into the matrix: rows and columns past it are
-            // loaded but not stored)
-            float mk[32];
-            if (EPI == MASK_BF16) {
-                const int nn = min(n0 + c0 + lane, N - 1);
+            float v[32];
+            load_acc32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-                for (int r = 0; r < 32; ++r) {
-                    const int row = min(m0 + warp * 32 + r, M - 1);
-                    mk[r] = __bfloat162float(mask[(size_t)row * ldmask + nn]);
-                }
-            }
-            uint32_t v[32];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-                  "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-                  "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                : "r"(ta));
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-            for (int j = 0; j < 32; ++j) st[lane * 33 + j] = __uint_as_float(v[j]);
+            for (int j = 0; j < 32; ++j) st[lane * 33 + j] = v[j];
             __syncwarp();
             const int n = n0 + c0 + lane;
             const bool col_ok = c0 + lane < NT && n < N;
-            const float b = (col_ok && (EPI == RELU_BF16 || EPI == LINEAR_F32)) ? bias[n] : 0.0f;
-            float csum = 0.0f;
+            const float b = (col_ok && EPI == LINEAR_F32) ? bias[n] : 0.0f;
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
                 const int row = m0 + warp * 32 + r;
                 if (row >= M || !col_ok) continue;
                 const float x = st[r * 33 + lane];
                 const size_t o = (size_t)row * ldc + n;
-                if (EPI == RELU_BF16) {
-                    outb[o] = __float2bfloat16(fmaxf(x + b, 0.0f));
-                } else if (EPI == LINEAR_F32) {
-                    outf[o] = x + b;
-                } else if (EPI == MASK_BF16) {
-                    const float y = mk[r] > 0.0f ? x : 0.0f;
-                    outb[o] = __float2bfloat16(y);
-                    csum += y;
-                } else {
-                    atomicAdd(&outf[o], x);
-                }
+                if (EPI == LINEAR_F32) outf[o] = x + b;
+                else atomicAdd(&outf[o], x);
             }
-            if (EPI == MASK_BF16 && col_ok) atomicAdd(&colsum[n], csum);
             __syncwarp();
         }
     }

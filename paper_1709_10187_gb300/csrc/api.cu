@@ -25,6 +25,40 @@ uint32_t quantise(double C) {
     return (uint32_t)t;
 }
 
+// Per cell, the number of spatial moves after which a packet is certainly still
+// in a cell of the same class: the cells' distance (moves along the axes) to the
+// nearest cell with a neighbour of another class, in vacuum or outside the grid,
+// at most 254.  One pass along the cells and one back give these distances.
+// Cells with a Doppler shift across a face get kNoMargin.
+std::vector<uint8_t> class_margins(const rddmc_grid& g) {
+    std::vector<uint8_t> m((size_t)g.ncell, 254), shifted(g.v.empty() ? 0 : (size_t)g.ncell, 0);
+    const int64_t stride[3] = {1, g.n[0], (int64_t)g.n[0] * g.n[1]};
+    auto nearer = [&](int64_t c, int64_t n) { m[c] = m[n] + 1 < m[c] ? (uint8_t)(m[n] + 1) : m[c]; };
+    int idx[3] = {0, 0, 0};
+    for (int64_t c = 0; c < g.ncell; ++c) {
+        for (int ax = 0; ax < g.ndim; ++ax) {
+            if (idx[ax] == 0 || idx[ax] + 1 == g.n[ax]) m[c] = 0;
+            if (idx[ax] + 1 == g.n[ax]) continue;
+            const int64_t n = c + stride[ax];
+            if (g.cell_class[n] != g.cell_class[c]) m[c] = m[n] = 0;
+            if (!g.v.empty() && g.v[3 * c + ax] != g.v[3 * n + ax] && g.cell_class[n] != UINT32_MAX &&
+                g.cell_class[c] != UINT32_MAX)
+                shifted[c] = shifted[n] = 1;
+        }
+        for (int ax = 0; ax < g.ndim; ++ax)
+            if (idx[ax] > 0) nearer(c, c - stride[ax]);
+        for (int ax = 0; ax < 3 && ++idx[ax] == g.n[ax]; ++ax) idx[ax] = 0;
+    }
+    for (int64_t c = g.ncell - 1; c >= 0; --c) {
+        for (int ax = 0; ax < 3 && --idx[ax] < 0; ++ax) idx[ax] = g.n[ax] - 1;
+        for (int ax = 0; ax < g.ndim; ++ax)
+            if (idx[ax] + 1 < g.n[ax]) nearer(c, c + stride[ax]);
+    }
+    for (size_t c = 0; c < shifted.size(); ++c)
+        if (shifted[c]) m[c] = (uint8_t)kNoMargin;
+    return m;
+}
+
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? RDDMC_OK : RDDMC_ERR_CUDA; }
 
 }  // namespace
@@ -199,6 +233,8 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     g->n_class = (int)g->class_rep.size();
     if ((uint64_t)g->n_class * (uint64_t)J > (1ull << 40)) { delete g; return RDDMC_ERR_UNSUPPORTED; }
 
+    if (g->pairs()) g->margin = class_margins(*g);
+
     // Table layout.
     uint64_t off = align256(sizeof(TableHeader));
     g->off_class = off; off += align256((uint64_t)ncell * 4);
@@ -215,6 +251,7 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     g->off_abs = off; off += align256((uint64_t)g->n_class * J * 4);
     g->off_wq = off; off += align256((uint64_t)g->n_class * J * 8);
     g->off_ka = off; off += align256((uint64_t)g->n_class * J * 4);
+    g->off_margin = off; off += g->pairs() ? align256((uint64_t)ncell) : 0;
     g->off_pair = off + 256; off += g->pairs() ? 256 + align256((uint64_t)g->n_class * J * 16 + kPairPad) : 0;
     g->table_bytes = off;
     *out = g;
@@ -314,6 +351,12 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
     if ((e = cudaMemcpyAsync(base + g->off_rebin, rb.data(), rb.size() * sizeof(Rebin), cudaMemcpyHostToDevice, s)) !=
         cudaSuccess)
         return cuda_status(e);
+    if (g->pairs()) {  // no margins on dusty grids: their rows have one more outcome
+        e = g->dusty() ? cudaMemsetAsync(base + g->off_margin, (int)kNoMargin, g->margin.size(), s)
+                       : cudaMemcpyAsync(base + g->off_margin, g->margin.data(), g->margin.size(),
+                                         cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
     if (g->moving && (e = cudaMemcpyAsync(base + g->off_vel, g->v.data(), g->v.size() * 8, cudaMemcpyHostToDevice,
                                           s)) != cudaSuccess)
         return cuda_status(e);
@@ -456,12 +499,12 @@ int rddmc_table_rows(const rddmc_grid* g, const void* d_table, uint32_t* thr, ui
                 flags[s_] = 0;
                 continue;
             }
-            // stored words: thr0, thr1, thr2, flags[, thr3..thr6]; FLAG_FASTX is
-            // an encoding detail of the walk and is not returned
+            // stored words: thr0, thr1, thr2, flags[, thr3..thr6]; FLAG_FASTX and
+            // FLAG_FASTZ are encoding details of the walk and are not returned
             const uint32_t* r = &rows[((uint64_t)k * g->J + j) * wpr];
             for (int o = 0; o < g->K - 1; ++o) thr[s_ * (K - 1) + o] = o < 3 ? r[o] : r[o + 1];
             if (g->dusty()) thr[s_ * (K - 1) + g->K - 1] = ab[(uint64_t)k * g->J + j];
-            flags[s_] = r[3] & ~FLAG_FASTX;
+            flags[s_] = r[3] & ~(FLAG_FASTX | FLAG_FASTZ);
         }
     }
     return RDDMC_OK;

@@ -22,6 +22,7 @@ struct rddmc_grid {
     std::vector<double> edges;
     std::vector<uint32_t> cell_class;   // UINT32_MAX for vacuum cells
     std::vector<int64_t> class_rep;     // a representative cell per class
+    std::vector<uint8_t> margin;        // per cell: spatial moves that stay in its class (with the pairs)
     std::vector<double> n_rel;          // per cell (copied)
     std::vector<double> v;              // per cell x3, km/s (empty if static)
     double vth = 12.85;                 // thermal velocity, km/s
@@ -34,7 +35,7 @@ struct rddmc_grid {
     // table layout (byte offsets)
     uint64_t off_class = 0, off_cdesc = 0, off_rebin = 0, off_vel = 0, off_edges = 0, off_phi = 0,
              off_rows = 0, off_fast = 0, off_tau = 0, off_upar = 0, off_rk = 0, off_abs = 0, off_wq = 0, off_ka = 0, off_pair = 0,
-             table_bytes = 0;
+             off_margin = 0, table_bytes = 0;
     // leakage parameters of the last precompute
     rddmc_leak_params params{};
     bool precomputed = false;

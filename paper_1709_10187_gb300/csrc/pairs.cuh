@@ -59,6 +59,70 @@ __device__ __forceinline__ void walk_four(const Pair* base, const uint4& r, uint
     ok4 = ok2 && max(r.z, r.w) < b.guard;
 }
 
+// Four transitions of any plain moves on the rows, without a branch on their
+// outcomes.  In a cell at least four moves inside its class (margin) a spatial
+// move leaves the row as it is, so a transition is one row's thresholds against
+// its word, and the rows' flags say that every outcome is a plain move
+// (FLAG_FASTX, FLAG_FASTZ); nearer the class's edge the outcome's own action is
+// looked at and the class follows the cell.  Moves s, cell and cls and returns
+// true; returns false with all as they were when a transition is not a plain
+// move, and on moving and dusty grids, which the caller walks outcome by outcome.
+// Such groups took 520 of 650 cycles per warp on the wide-core slab when every
+// transition branched.
+template <int NDIM, bool INSIDE, class K>
+__device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, const uint4& r, unsigned& s,
+                                          unsigned& cell, unsigned& cls) {
+    unsigned s1 = s, c1 = cell, k1 = cls, flags = FLAG_FASTX | FLAG_FASTZ;
+    bool plain = true;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const unsigned w = q == 0 ? r.x : (q == 1 ? r.y : (q == 2 ? r.z : r.w));
+        const unsigned row = min(s1, nr1);
+        const uint4 a = __ldg(&P.rows[NDIM == 1 ? row : 2u * row]);
+        const bool spatial = w >= a.y;  // thresholds of j-1 | j+1 | -x | +x ...
+        unsigned move, outcome;
+        if (NDIM == 1) {
+            const bool up = w >= (spatial ? a.z : a.x);
+            move = up ? 1u : 0xffffffffu;
+            outcome = (spatial ? 2u : 0u) + (up ? 1u : 0u);
+        } else {
+            const uint4 b = __ldg(&P.rows[2u * row + 1u]);  // ... | -y | +y | -z | +z
+            const bool y = w >= b.x, z = w >= b.z;
+            const bool up = w >= (spatial ? (z ? b.w : (y ? b.y : a.z)) : a.x);
+            const unsigned stride = !spatial ? 1u : (z ? (unsigned)P.n01 : (y ? (unsigned)P.n0 : 1u));
+            move = up ? stride : 0u - stride;
+            outcome = (spatial ? (z ? 6u : (y ? 4u : 2u)) : 0u) + (up ? 1u : 0u);
+        }
+        if (INSIDE) flags &= a.w;
+        else plain = plain && ((a.w >> (2u * outcome)) & 3u) == ACT_MOVE;
+        if (!spatial) {
+            s1 += move;
+        } else {
+            c1 += move;
+            if (!INSIDE) {
+                c1 = min(c1, (unsigned)P.ncell - 1u);
+                const unsigned k = __ldg(&P.cell_class[c1]);
+                s1 += (k - k1) * J;
+                k1 = k;
+            }
+        }
+    }
+    if (!plain || flags != (FLAG_FASTX | FLAG_FASTZ)) return false;
+    s = s1;
+    cell = c1;
+    cls = k1;
+    return true;
+}
+
+template <int NDIM, class K>
+__device__ __forceinline__ bool walk_four_rows(const K& P, unsigned nr1, unsigned J, const uint4& r, unsigned& s,
+                                               unsigned& cell, unsigned& cls) {
+    const unsigned deep = __ldg(&P.margin[cell]);
+    if (deep == kNoMargin) return false;
+    return deep >= 4u ? walk_rows<NDIM, true>(P, nr1, J, r, s, cell, cls)
+                      : walk_rows<NDIM, false>(P, nr1, J, r, s, cell, cls);
+}
+
 // Consecutive transition blocks of one packet for a fixed high word of the
 // block index: Philox4x32-10 of (b, b_hi, p_lo, p_hi) with what the first three
 // rounds owe to the packet and b_hi alone computed once, and the first product

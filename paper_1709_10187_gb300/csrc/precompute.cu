@@ -168,6 +168,10 @@ __global__ void __launch_bounds__(kRowEdges)
 #pragma unroll
     for (int o = 0; o < K; ++o) fl |= (act[o] & 3u) << (2 * o);
     if (act[0] == ACT_MOVE && act[1] == ACT_MOVE) fl |= FLAG_FASTX;
+    bool fastz = !dusty;
+#pragma unroll
+    for (int o = 2; o < K; ++o) fastz = fastz && act[o] == ACT_MOVE;
+    if (fastz) fl |= FLAG_FASTZ;
     if (D.moving) fl |= FLAG_MOVING;
     if (hybrid && k * dzmin < h.tau_ddmc) fl |= FLAG_THIN;
     // word order: thr0, thr1, thr2, flags[, thr3..thr6] so that the first 16

@@ -5,7 +5,9 @@
 //    | cell velocity f64[3*ncell] (moving media only) | edges f64[J+1] | phi f64[J] | rows
 //    | fast heads uint2[n_class*J] | tau f32[n_class*J] | u_par split points f32x2[kUparN]
 //    | 1/K_s f32[n_class*J] | dust absorption thresholds u32[n_class*J] | dust weights u64[n_class*J]
-//    | dust opacities f32[n_class*J] | pairs 16 B[n_class*J] with pads (tables up to kPairRows rows)]
+//    | dust opacities f32[n_class*J] | pairs 16 B[n_class*J] with pads (tables up to kPairRows rows)
+//    | margins u8[ncell] (with the pairs): spatial moves a packet can make from a cell and stay in its class,
+//    at most 254, or kNoMargin]
 // With dust absorption (Sec. 2.6) the categorical draw has one more outcome,
 // absorption, after the leakage outcomes: the row thresholds are cumulative over
 // the leakage rates plus k_a, and the absorption threshold (where absorption
@@ -37,6 +39,7 @@ constexpr int kHistOff = 22;
 constexpr int kNsb = 64;            // impact-parameter bins over b/R in [0, kSbMax)
 constexpr double kSbMax = 1.28;
 constexpr int64_t kPairRows = 1 << 20;  // tables up to this many rows carry the walk's pairs (pairs.cuh)
+constexpr unsigned kNoMargin = 255;     // margin of a cell with a Doppler rebin on one of its faces, or with dust
 constexpr int kUparN = 1024;        // |x| grid of the u_par envelope split points
 constexpr float kUparStep = 1.0f / 16.0f;
 
@@ -48,6 +51,7 @@ enum Counter : int {
 
 // 2-bit actions per outcome in the flags word.
 constexpr uint32_t ACT_MOVE = 0u, ACT_ESCAPE = 1u, ACT_TO_MC = 2u, ACT_REBIN = 3u;
+constexpr uint32_t FLAG_FASTZ = 1u << 28;   // every spatial outcome is a plain move, and there is no absorption
 constexpr uint32_t FLAG_FASTX = 1u << 29;   // both frequency outcomes are plain moves
 constexpr uint32_t FLAG_MOVING = 1u << 30;
 constexpr uint32_t FLAG_THIN = 1u << 31;

@@ -316,8 +316,11 @@ enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2 };
 // four dependent 8-byte gathers of a group, which held the L1 at its random
 // gather rate, down to two.  __grid_constant__: the escape functions take the
 // parameter block's address, and without it every read of P went to a local
-// copy (9 local loads per group).  Two 4096-step slices of 4e6 packets on the
-// 256 x 512 slab: 32.5 ms with heads, 27.7 ms.
+// copy (9 local loads per group).  A group that is not four frequency moves is
+// walked on its rows, again without a branch per transition (walk_four_rows).
+// Two 4096-step slices of 4e6 packets on the 256 x 512 slab: 32.6 ms with heads,
+// 27.7 ms with pairs, 26.1 ms with the rows in groups too; 2e6 packets on its
+// wide-core grid to escape: 205, 184 and 98 ms.
 template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
 __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const __grid_constant__ WalkParams P) {
     constexpr int RW = NDIM == 1 ? 1 : 2;  // uint4 per row
@@ -640,7 +643,12 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                             o = min(o4 - 64u, omax);
                             return false;
                         }
-                        s = (ok2 ? o2 - 32u : o) >> 4;
+                        s = o >> 4;
+                        if (walk_four_rows<NDIM>(P, nr1, J, r, s, cell, cls)) {
+                            o = 16u * s;
+                            return false;
+                        }
+                        if (ok2) s = (o2 - 32u) >> 4;
                         const unsigned q = by_rows(r, ok2 ? 2u : 0u);
                         o = min(16u * s, omax);
                         t = 4ull * (blk - behind) + q + 1ull;
@@ -1259,6 +1267,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.rows = (const uint4*)(tb + g.off_rows);
     P.fast = (const uint2*)(tb + g.off_fast);
     P.pair = g.pairs() ? (const Pair*)(tb + g.off_pair) : nullptr;
+    P.margin = g.pairs() ? (const uint8_t*)(tb + g.off_margin) : nullptr;
     P.tau_row = (const float*)(tb + g.off_tau);
     P.upar = (const float2*)(tb + g.off_upar);
     P.cdesc = (const ClassDesc*)(tb + g.off_cdesc);

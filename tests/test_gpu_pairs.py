@@ -47,6 +47,38 @@ def test_few_bins_and_odd_limits_match_the_oracle(ndim, J, v, max_steps):
     p.close()
 
 
+@pytest.mark.parametrize("case", ["slab", "graded", "cube", "sphere", "layers"])
+@pytest.mark.parametrize("max_steps", [0, 41])
+def test_rows_in_groups_of_four_match_the_oracle(case, max_steps):
+    # wing-heavy grids: most transitions are spatial moves on the rows, in cells
+    # more and less than four moves inside their class, to the grid's ends, to
+    # vacuum and between classes of different density
+    n_rel, sphere = None, False
+    if case in ("slab", "graded"):
+        n, ndim = (24, 1, 1), 1
+        if case == "graded":
+            n_rel = np.linspace(0.5, 2.0, 24)
+    else:
+        n, ndim = ((11, 14, 9), 3) if case != "sphere" else ((13, 13, 13), 3)
+        sphere = case == "sphere"
+        if case == "layers":  # two media, six cells thick on average
+            n_rel = np.where(np.arange(11 * 14 * 9) // 11 % 14 < 7, 1.0, 3.0)
+    w = W.Workload(f"rows_{case}", ndim, n, 15, -45.0, 45.0, 2.0e3, 1.0e4, 4000, 0x5EED0B03, sphere=sphere)
+    g = C.Grid(w, n_rel=n_rel)
+    ot = g.table()
+    p = R.Problem(w, n_rel=n_rel)
+    thr, _ = p.rows()
+    sel = np.ones(w.ncell * w.J, bool) if w.mask() is None else np.repeat(w.mask().astype(bool), w.J)
+    ot["thr"][sel] = thr[sel]
+    orc = C.walk(g, ot, w.seed, 0, w.packets, max_steps=max_steps or 1 << 62)
+    _same(p.run(w.packets, w.seed, max_steps=max_steps), orc, 2 * ndim)
+    # the batched walk takes the same path with its own lane's tables
+    b = R.Batch([p, p], [w.packets, 7])
+    b.launch(R.RunOpts(w.seed, 0, max_steps))
+    _same(b.read(0), orc, 2 * ndim)
+    p.close()
+
+
 @pytest.mark.parametrize("chunk", [4, 12, 256])
 def test_pairs_and_heads_walk_alike(chunk):
     # dense tables below and above 2^20 rows: pairs on one side, heads on the other

@@ -7,8 +7,9 @@
 // [off_i, off_i + n_i) and its packet p uses the streams of global id off_i + p
 // under the batch seed, so one Philox key schedule serves every lane.  A lane
 // maps a refilled id to its instance by binary search over the offsets and
-// walks it exactly as the single-grid kernel does (the 8-byte fast head for
-// frequency moves, the full row otherwise).  Counters are kept per lane and
+// walks it exactly as the single-grid kernel does (pairs for two frequency moves
+// per gather, or the 8-byte fast heads where an instance's table is too large
+// for pairs; the full row otherwise).  Counters are kept per lane and
 // added to the instance's tally block when the lane changes instance;
 // escapes go straight to the instance's histograms with global atomics (they
 // are rare and instances differ in size, so per-CTA shared histograms would
@@ -23,6 +24,7 @@
 
 #include "escape.cuh"
 #include "grid.h"
+#include "pairs.cuh"
 
 namespace rddmc {
 namespace {
@@ -32,6 +34,8 @@ constexpr unsigned FULL = 0xffffffffu;
 struct InstDesc {
     const uint4* rows;
     const uint2* fast;
+    const Pair* pair;               // null for a large table
+    const uint8_t* margin;          // with pair
     const uint32_t* cell_class;
     const Rebin* rebin;
     const double* edges;
@@ -54,18 +58,6 @@ struct BatchParams {
     uint32_t rk0[10], rk1[10];
     int chunk;
 };
-
-__device__ __forceinline__ uint4 bphilox(uint4 c, const BatchParams& P) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ P.rk0[r], lo1, hi0 ^ c.w ^ P.rk1[r], lo0);
-    }
-    return c;
-}
 
 __device__ __forceinline__ unsigned bword(const uint4& r, unsigned q) {
     return q == 0 ? r.x : (q == 1 ? r.y : (q == 2 ? r.z : r.w));
@@ -95,15 +87,27 @@ __device__ __noinline__ void batch_escape(const BatchParams& P, const InstDesc& 
     if (sb >= 0) atomicAdd(&T[kHistOff + D.J + 2 + sb], 1ull);
 }
 
-__global__ void __launch_bounds__(256, 3) batch_kernel(const BatchParams P) {
+// What a lane needs of its instance outside the pair loop, in shared memory: read
+// on the rare outcomes, and the loop keeps its registers.
+struct LaneInst {
+    const uint4* rows;
+    const uint2* fast;
+    const uint32_t* cell_class;
+    const uint8_t* margin;
+    unsigned J, ncls1, n0, n01, ndim;
+    int ncell;
+};
+
+// Bound by dispatch in the pair loop and by its lanes in thin media, which leave
+// it for the rows (the 64-instance study: 20.0 ms with heads, 11.5 ms).
+__global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ BatchParams P) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LaneInst& L = reinterpret_cast<LaneInst*>(smem_raw)[threadIdx.x];
     const unsigned lane = threadIdx.x & 31u;
     bool have = false, exhausted = false;
     int inst = -1;
-    // instance parameters held by the lane
-    const uint2* fast = nullptr;
-    const uint4* rows = nullptr;
-    const uint32_t* cell_class = nullptr;
-    unsigned J = 1, nr1 = 0, ncell1 = 0, ncls1 = 0, n0 = 1, n01 = 1, ndim = 1;
+    const Pair* pair = nullptr;
+    unsigned nr1 = 0;
     unsigned long long gid = 0, t = 0, e = 0;
     unsigned cell = 0, cls = 0, s = 0;
     unsigned long long n_steps = 0, n_edraw = 0;
@@ -122,45 +126,47 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const BatchParams P) {
         n_steps = n_edraw = 0;
     };
 
-    auto generic = [&](unsigned w) -> bool {
-        const unsigned rw = ndim == 1 ? 1u : 2u;
+    // One full transition on word w: every threshold, the outcome's action.
+    // Returns true when the packet has finished.
+    auto transition = [&](unsigned w) -> bool {
+        const bool slab = L.ndim == 1u;
         const unsigned ri = min(s, nr1);
-        const uint4 a = __ldg(&rows[ri * rw]);
+        const uint4 a = __ldg(&L.rows[slab ? ri : 2u * ri]);
         unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
-        if (ndim == 3) {
-            const uint4 b = __ldg(&rows[ri * rw + 1]);
+        if (!slab) {
+            const uint4 b = __ldg(&L.rows[2u * ri + 1u]);
             o += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
         }
         const unsigned fl = a.w;
         const unsigned act = (fl >> (2u * o)) & 3u;
-        const unsigned bin = min(s - cls * J, J - 1u);
         if (o < 2u) {
             if (act == ACT_MOVE) { s += o ? 1u : 0xffffffffu; return false; }
             ++n_abort;  // a hand-off to MC: batches run the DDMC walk only
             return true;
         }
         const unsigned face = o - 2u;
+        if (act == ACT_TO_MC) { ++n_abort; return true; }
+        const unsigned J = L.J;
+        unsigned bin = min(s - cls * J, J - 1u);
         if (act == ACT_ESCAPE) {
             batch_escape(P, P.desc[inst], cell, bin, face, gid, e, (fl & FLAG_MOVING) != 0u);
-            if (ndim == 3 || (fl & FLAG_MOVING)) e += 5;
+            if (!slab || (fl & FLAG_MOVING)) e += 5;
             ++n_esc;
             return true;
         }
-        if (act == ACT_TO_MC) { ++n_abort; return true; }
-        unsigned nbin = bin;
         if (act == ACT_REBIN) {
-            const Rebin rb = P.desc[inst].rebin[min(cls, ncls1) * (2u * ndim) + face];
+            const Rebin rb = P.desc[inst].rebin[min(cls, L.ncls1) * (2u * L.ndim) + face];
             const unsigned w1 = event_word(gid, e++, P.k0, P.k1);
             int jn = (int)bin + rb.m + (w1 >= rb.thr ? 1 : 0);
             if (jn < 0) { jn = 0; ++n_clamp; }
             if (jn > (int)J - 1) { jn = (int)J - 1; ++n_clamp; }
-            nbin = (unsigned)jn;
+            bin = (unsigned)jn;
         }
         const unsigned ax = face >> 1;
-        const unsigned stride = ax == 0 ? 1u : (ax == 1 ? n0 : n01);
-        cell = min((face & 1u) ? cell + stride : cell - stride, ncell1);
-        cls = __ldg(&cell_class[cell]);
-        s = cls * J + nbin;
+        const unsigned stride = ax == 0 ? 1u : (ax == 1 ? L.n0 : L.n01);
+        cell = min((face & 1u) ? cell + stride : cell - stride, (unsigned)L.ncell - 1u);
+        cls = __ldg(&L.cell_class[cell]);
+        s = cls * J + bin;
         return false;
     };
 
@@ -181,26 +187,26 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const BatchParams P) {
                         const int mid = (lo + hi) >> 1;
                         if (q >= P.off[mid]) lo = mid; else hi = mid;
                     }
+                    const InstDesc& D = P.desc[lo];
                     if (lo != inst) {
                         flush();
                         inst = lo;
-                        const InstDesc& D = P.desc[inst];
-                        fast = D.fast; rows = D.rows; cell_class = D.cell_class;
-                        J = (unsigned)D.J; nr1 = (unsigned)D.n_rows - 1u; ncell1 = (unsigned)D.ncell - 1u;
-                        ncls1 = (unsigned)D.n_class - 1u; n0 = (unsigned)D.n0; n01 = (unsigned)D.n01;
-                        ndim = (unsigned)D.ndim;
+                        pair = D.pair;
+                        nr1 = (unsigned)D.n_rows - 1u;
+                        L.rows = D.rows; L.fast = D.fast; L.cell_class = D.cell_class;
+                        L.margin = D.margin; L.J = (unsigned)D.J; L.ncell = D.ncell; L.ncls1 = (unsigned)D.n_class - 1u;
+                        L.n0 = (unsigned)D.n0; L.n01 = (unsigned)D.n01; L.ndim = (unsigned)D.ndim;
                     }
-                    const InstDesc& D = P.desc[inst];
                     gid = D.pkt_begin + (q - P.off[inst]);
                     const unsigned w = event_word(gid, 0, P.k0, P.k1);
                     unsigned idx[3];
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
                         idx[a] = (unsigned)D.src_cand[a][(D.src_ncand[a] == 2) ? ((w >> (31 - a)) & 1u) : 0u];
-                    cell = min(idx[0] + n0 * idx[1] + n01 * idx[2], ncell1);
+                    cell = min(idx[0] + L.n0 * idx[1] + L.n01 * idx[2], (unsigned)L.ncell - 1u);
                     const unsigned bin = (unsigned)D.src_bin[(D.src_nbin == 2) ? ((w >> 28) & 1u) : 0u];
-                    cls = __ldg(&cell_class[cell]);
-                    s = cls * J + min(bin, J - 1u);
+                    cls = __ldg(&L.cell_class[cell]);
+                    s = cls * L.J + min(bin, L.J - 1u);
                     t = 0;
                     e = 1;
                     ++n_emit;
@@ -219,54 +225,79 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const BatchParams P) {
         {
             const uint32_t pl = (uint32_t)gid, ph = (uint32_t)(gid >> 32);
             unsigned long long blk = t >> 2;
-            const unsigned ng = (unsigned)((lim - t) >> 2);
-            uint4 rn = bphilox(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
-            unsigned g = 0;
-            while (g < ng) {
-                const uint4 r = rn;
-                ++blk;
-                rn = bphilox(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), pl, ph), P);
-                unsigned q;
-                {
-                    // four transitions as one branch-free chain of head loads
-                    // (clamped speculative states), checked at its end, as in
-                    // the single-grid walk
-                    const unsigned s0 = s;
-                    const uint2 f0 = __ldg(&fast[min(s0, nr1)]);
-                    const unsigned s1 = s0 + ((r.x >= f0.x) ? 1u : 0xffffffffu);
-                    const uint2 f1 = __ldg(&fast[min(s1, nr1)]);
-                    const unsigned s2 = s1 + ((r.y >= f1.x) ? 1u : 0xffffffffu);
-                    const uint2 f2 = __ldg(&fast[min(s2, nr1)]);
-                    const unsigned s3 = s2 + ((r.z >= f2.x) ? 1u : 0xffffffffu);
-                    const uint2 f3 = __ldg(&fast[min(s3, nr1)]);
-                    const unsigned s4 = s3 + ((r.w >= f3.x) ? 1u : 0xffffffffu);
-                    const bool ok0 = r.x < f0.y, ok1 = r.y < f1.y, ok2 = r.z < f2.y, ok3 = r.w < f3.y;
-                    if (ok0 && ok1 && ok2 && ok3) {
-                        s = s4;
-                        ++g;
-                        continue;
+            const unsigned long long blk_end = blk + ((lim - t) >> 2);
+            while (blk < blk_end) {  // one pass, or two when the block index crosses a multiple of 2^32
+                const uint32_t bh = (uint32_t)(blk >> 32);
+                const unsigned long long wrap = ((unsigned long long)bh + 1ull) << 32;
+                unsigned left = (unsigned)((blk_end < wrap ? blk_end : wrap) - blk);
+                blk += left;
+                TransitionStream ts;
+                ts.init((uint32_t)blk - left, bh, pl, ph, P);
+                uint4 ra = ts.next(P), rb;
+                // one group of four on r while the next block is drawn into rn; true
+                // when the packet finished
+                auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
+                    unsigned q = 0;
+                    if (pair) {
+                        const uint32_t o = 16u * min(s, nr1);
+                        uint32_t o2, o4;
+                        bool ok2, ok4;
+                        walk_four(pair, r, o, o2, o4, ok2, ok4);
+                        rn = ts.next(P);
+                        if (ok4) {
+                            s = (o4 - 64u) >> 4;
+                            return false;
+                        }
+                        s = o >> 4;
+                        if (L.ndim == 1u ? walk_four_rows<1>(L, nr1, L.J, r, s, cell, cls)
+                                         : walk_four_rows<3>(L, nr1, L.J, r, s, cell, cls))
+                            return false;
+                        if (ok2) {
+                            s = (o2 - 32u) >> 4;
+                            q = 2u;
+                        }
+                    } else {
+                        // a large table: four transitions as one branch-free chain of
+                        // head loads (clamped speculative states), checked at its
+                        // end, as in the single-grid walk
+                        rn = ts.next(P);
+                        const uint2* fast = L.fast;
+                        const unsigned s0 = s;
+                        const uint2 f0 = __ldg(&fast[min(s0, nr1)]);
+                        const unsigned s1 = s0 + ((r.x >= f0.x) ? 1u : 0xffffffffu);
+                        const uint2 f1 = __ldg(&fast[min(s1, nr1)]);
+                        const unsigned s2 = s1 + ((r.y >= f1.x) ? 1u : 0xffffffffu);
+                        const uint2 f2 = __ldg(&fast[min(s2, nr1)]);
+                        const unsigned s3 = s2 + ((r.z >= f2.x) ? 1u : 0xffffffffu);
+                        const uint2 f3 = __ldg(&fast[min(s3, nr1)]);
+                        const bool ok0 = r.x < f0.y, ok1 = r.y < f1.y, ok2 = r.z < f2.y, ok3 = r.w < f3.y;
+                        if (ok0 && ok1 && ok2 && ok3) {
+                            s = s3 + ((r.w >= f3.x) ? 1u : 0xffffffffu);
+                            return false;
+                        }
+                        q = !ok0 ? 0u : (!ok1 ? 1u : (!ok2 ? 2u : 3u));
+                        s = !ok0 ? s0 : (!ok1 ? s1 : (!ok2 ? s2 : s3));
                     }
-                    q = !ok0 ? 0u : (!ok1 ? 1u : (!ok2 ? 2u : 3u));
-                    s = !ok0 ? s0 : (!ok1 ? s1 : (!ok2 ? s2 : s3));
-                    goto slow;
+                    do {
+                        if (transition(bword(r, q))) {
+                            t = 4ull * (blk - behind) + q + 1ull;
+                            return true;
+                        }
+                    } while (++q < 4u);
+                    return false;
+                };
+                if (left & 1u) {
+                    if (group(ra, rb, left)) { fin = true; goto chunk_done; }
+                    ra = rb;
                 }
-                ++g;
-                continue;
-            slow:
-                for (; q < 4u; ++q) {
-                    if (generic(bword(r, q))) {
-                        fin = true;
-                        t += 4ull * g + q + 1ull;
-                        goto chunk_done;
-                    }
-                }
-                ++g;
+                for (left &= ~1u; left; left -= 2u)
+                    if (group(ra, rb, left) || group(rb, ra, left - 1u)) { fin = true; goto chunk_done; }
             }
-            t += 4ull * ng;
+            t = 4ull * blk;
             while (t < lim) {
                 const unsigned long long b = t >> 2;
-                const uint4 r = bphilox(make_uint4((uint32_t)b, (uint32_t)(b >> 32), pl, ph), P);
-                const bool f = generic(bword(r, (unsigned)t & 3u));
+                const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)(b >> 32), pl, ph), P.k0, P.k1);
+                const bool f = transition(bword(r, (unsigned)t & 3u));
                 ++t;
                 if (f) { fin = true; break; }
             }
@@ -302,6 +333,8 @@ struct rddmc_batch {
 
 namespace {
 
+size_t lane_bytes(int threads) { return (size_t)threads * sizeof(LaneInst); }
+
 uint64_t off_array_bytes(size_t n_inst) { return align256((n_inst + 1) * 8ull); }
 
 void fill_params(const rddmc_batch* b, const void* d_desc, bool trial, const rddmc_run_opts* o, void* d_scratch,
@@ -334,7 +367,7 @@ cudaError_t enqueue(const rddmc_batch* b, const BatchParams& P, const rddmc_run_
     const int threads = o->threads_per_cta ? o->threads_per_cta : 256;
     const int ctas = o->ctas_per_sm ? o->ctas_per_sm : std::max(1, b->default_ctas);
     if ((e = cudaMemsetAsync(P.cursor, 0, 8, s)) != cudaSuccess) return e;
-    batch_kernel<<<(unsigned)(ctas * nsm), threads, 0, s>>>(P);
+    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
     return cudaGetLastError();
 }
 
@@ -383,6 +416,8 @@ int rddmc_batch_create(const rddmc_grid* const* grids, const void* const* d_tabl
         std::memset(&D, 0, sizeof(D));
         D.rows = (const uint4*)(tb + g->off_rows);
         D.fast = (const uint2*)(tb + g->off_fast);
+        D.pair = g->pairs() ? (const Pair*)(tb + g->off_pair) : nullptr;
+        D.margin = g->pairs() ? (const uint8_t*)(tb + g->off_margin) : nullptr;
         D.cell_class = (const uint32_t*)(tb + g->off_class);
         D.rebin = (const Rebin*)(tb + g->off_rebin);
         D.edges = (const double*)(tb + g->off_edges);
@@ -410,7 +445,7 @@ int rddmc_batch_create(const rddmc_grid* const* grids, const void* const* d_tabl
     b->total = b->off.back();
     b->desc_bytes = align256(b->desc.size() * sizeof(InstDesc)) + 2 * off_array_bytes(b->desc.size());
     int ctas = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, batch_kernel, 256, 0) != cudaSuccess) ctas = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, batch_kernel, 256, lane_bytes(256)) != cudaSuccess) ctas = 1;
     b->default_ctas = std::max(1, ctas);
     *out = b;
     return RDDMC_OK;
@@ -493,7 +528,7 @@ int rddmc_batch_graph_create(const rddmc_batch* b, const void* d_desc, const rdd
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return RDDMC_ERR_CUDA;
     cudaMemsetAsync(d_tallies, 0, b->tally_words * 8ull, s);
     cudaMemsetAsync(d_scratch, 0, 8, s);
-    batch_kernel<<<(unsigned)(ctas * nsm), threads, 0, s>>>(P);
+    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
     const cudaError_t le = cudaGetLastError();
     const cudaError_t ce = cudaStreamEndCapture(s, &graph);
     if (le != cudaSuccess || ce != cudaSuccess || !graph) {
@@ -540,7 +575,7 @@ int rddmc_batch_autotune(const rddmc_batch* b, const void* d_desc, const rddmc_r
     const int threads_c[] = {128, 256};
     const int chunk_c[] = {64, 256, 1024};
     int occ128 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ128, batch_kernel, 128, 0) != cudaSuccess) occ128 = 6;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ128, batch_kernel, 128, lane_bytes(128)) != cudaSuccess) occ128 = 6;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return RDDMC_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return RDDMC_ERR_CUDA; }

@@ -96,6 +96,7 @@ struct LaneInst {
     const uint8_t* margin;
     unsigned J, ncls1, n0, n01, ndim;
     int ncell;
+    static constexpr bool kDust = false;  // instances have none
 };
 
 // Bound by dispatch in the pair loop and by its lanes in thin media, which leave
@@ -240,20 +241,18 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                     unsigned q = 0;
                     if (pair) {
                         const uint32_t o = 16u * min(s, nr1);
-                        uint32_t o2, o4;
-                        bool ok2, ok4;
-                        walk_four(pair, r, o, o2, o4, ok2, ok4);
+                        const FourMoves m = walk_four(pair, r, o);
                         rn = ts.next(P);
-                        if (ok4) {
-                            s = (o4 - 64u) >> 4;
+                        if (m.ok4) {
+                            s = (m.o4 - 64u) >> 4;
                             return false;
                         }
                         s = o >> 4;
                         if (L.ndim == 1u ? walk_four_rows<1>(L, nr1, L.J, r, s, cell, cls)
                                          : walk_four_rows<3>(L, nr1, L.J, r, s, cell, cls))
                             return false;
-                        if (ok2) {
-                            s = (o2 - 32u) >> 4;
+                        if (m.ok2) {
+                            s = (m.o2 - 32u) >> 4;
                             q = 2u;
                         }
                     } else {
@@ -417,7 +416,7 @@ int rddmc_batch_create(const rddmc_grid* const* grids, const void* const* d_tabl
         D.rows = (const uint4*)(tb + g->off_rows);
         D.fast = (const uint2*)(tb + g->off_fast);
         D.pair = g->pairs() ? (const Pair*)(tb + g->off_pair) : nullptr;
-        D.margin = g->pairs() ? (const uint8_t*)(tb + g->off_margin) : nullptr;
+        D.margin = !g->margin.empty() ? (const uint8_t*)(tb + g->off_margin) : nullptr;
         D.cell_class = (const uint32_t*)(tb + g->off_class);
         D.rebin = (const Rebin*)(tb + g->off_rebin);
         D.edges = (const double*)(tb + g->off_edges);

@@ -22,7 +22,7 @@ struct rddmc_grid {
     std::vector<double> edges;
     std::vector<uint32_t> cell_class;   // UINT32_MAX for vacuum cells
     std::vector<int64_t> class_rep;     // a representative cell per class
-    std::vector<uint8_t> margin;        // per cell: spatial moves that stay in its class (with the pairs)
+    std::vector<uint8_t> margin;        // per cell: spatial moves that stay in its class (pairs and a static grid; else empty)
     std::vector<double> n_rel;          // per cell (copied)
     std::vector<double> v;              // per cell x3, km/s (empty if static)
     double vth = 12.85;                 // thermal velocity, km/s

@@ -29,11 +29,9 @@ struct alignas(16) Pair {
 // gather's address, so a move is one predicated add.
 //
 // Four frequency moves on the words of r from offset o0: two gathers through L1
-// (the table is read-only during a walk).  up2 and up4 return 32 times the
-// upward moves of the first two and of all four transitions; ok2 and ok4 whether
-// those were frequency moves.  Offsets stay inside the pair region and its pads
-// whatever the table holds: o0 is clamped by the caller, the second gather lies
-// within two rows of it (kPairPad bytes before and after the region).
+// (the table is read-only during a walk).  Offsets stay inside the pair region
+// and its pads whatever the table holds: o0 is clamped by the caller, the second
+// gather lies within two rows of it (kPairPad bytes before and after the region).
 constexpr int kPairPad = 32;
 
 __device__ __forceinline__ Pair load_pair(const Pair* base, uint32_t offset, int shift) {
@@ -41,22 +39,28 @@ __device__ __forceinline__ Pair load_pair(const Pair* base, uint32_t offset, int
     return Pair{v.x, v.y, v.z, v.w};
 }
 
-__device__ __forceinline__ void walk_four(const Pair* base, const uint4& r, uint32_t o0, uint32_t& o2, uint32_t& o4,
-                                          bool& ok2, bool& ok4) {
+struct FourMoves {
+    uint32_t o2, o4;  // offsets after two and four moves, less the constants -32 and -64
+    bool ok2, ok4;    // the first two, all four transitions are frequency moves
+};
+
+__device__ __forceinline__ FourMoves walk_four(const Pair* base, const uint4& r, uint32_t o0) {
+    FourMoves m;
     const Pair a = load_pair(base, o0, 0);
     const bool d0 = r.x >= a.z;
     const bool d1 = r.y >= (d0 ? a.p1 : a.m1);
-    o2 = o0;
-    if (d0) o2 += 32u;
-    if (d1) o2 += 32u;
-    const Pair b = load_pair(base, o2, -32);
+    m.o2 = o0;
+    if (d0) m.o2 += 32u;
+    if (d1) m.o2 += 32u;
+    const Pair b = load_pair(base, m.o2, -32);
     const bool d2 = r.z >= b.z;
     const bool d3 = r.w >= (d2 ? b.p1 : b.m1);
-    o4 = o2;
-    if (d2) o4 += 32u;
-    if (d3) o4 += 32u;
-    ok2 = max(r.x, r.y) < a.guard;
-    ok4 = ok2 && max(r.z, r.w) < b.guard;
+    m.o4 = m.o2;
+    if (d2) m.o4 += 32u;
+    if (d3) m.o4 += 32u;
+    m.ok2 = max(r.x, r.y) < a.guard;
+    m.ok4 = m.ok2 && max(r.z, r.w) < b.guard;
+    return m;
 }
 
 // Four transitions of any plain moves on the rows, without a branch on their
@@ -66,10 +70,10 @@ __device__ __forceinline__ void walk_four(const Pair* base, const uint4& r, uint
 // (FLAG_FASTX, FLAG_FASTZ); nearer the class's edge the outcome's own action is
 // looked at and the class follows the cell.  Moves s, cell and cls and returns
 // true; returns false with all as they were when a transition is not a plain
-// move, and on moving and dusty grids, which the caller walks outcome by outcome.
+// move, and on moving grids, which the caller walks outcome by outcome.
 // Such groups took 520 of 650 cycles per warp on the wide-core slab when every
 // transition branched.
-template <int NDIM, bool INSIDE, class K>
+template <int NDIM, bool INSIDE, bool DUST, class K>
 __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, const uint4& r, unsigned& s,
                                           unsigned& cell, unsigned& cls) {
     unsigned s1 = s, c1 = cell, k1 = cls, flags = FLAG_FASTX | FLAG_FASTZ;
@@ -93,6 +97,7 @@ __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, 
             move = up ? stride : 0u - stride;
             outcome = (spatial ? (z ? 6u : (y ? 4u : 2u)) : 0u) + (up ? 1u : 0u);
         }
+        if constexpr (DUST) plain = plain && w < __ldg(&P.abs_thr[row]);  // not absorbed
         if (INSIDE) flags &= a.w;
         else plain = plain && ((a.w >> (2u * outcome)) & 3u) == ACT_MOVE;
         if (!spatial) {
@@ -117,10 +122,11 @@ __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, 
 template <int NDIM, class K>
 __device__ __forceinline__ bool walk_four_rows(const K& P, unsigned nr1, unsigned J, const uint4& r, unsigned& s,
                                                unsigned& cell, unsigned& cls) {
-    const unsigned deep = __ldg(&P.margin[cell]);
-    if (deep == kNoMargin) return false;
-    return deep >= 4u ? walk_rows<NDIM, true>(P, nr1, J, r, s, cell, cls)
-                      : walk_rows<NDIM, false>(P, nr1, J, r, s, cell, cls);
+    if (!P.margin) return false;
+    if constexpr (K::kDust)
+        if (P.dust) return walk_rows<NDIM, false, true>(P, nr1, J, r, s, cell, cls);
+    return __ldg(&P.margin[cell]) >= 4u ? walk_rows<NDIM, true, false>(P, nr1, J, r, s, cell, cls)
+                                        : walk_rows<NDIM, false, false>(P, nr1, J, r, s, cell, cls);
 }
 
 // Consecutive transition blocks of one packet for a fixed high word of the

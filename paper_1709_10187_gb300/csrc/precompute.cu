@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kRowEdges)
 #pragma unroll
     for (int o = 0; o < K; ++o) fl |= (act[o] & 3u) << (2 * o);
     if (act[0] == ACT_MOVE && act[1] == ACT_MOVE) fl |= FLAG_FASTX;
-    bool fastz = !dusty;
+    bool fastz = true;
 #pragma unroll
     for (int o = 2; o < K; ++o) fastz = fastz && act[o] == ACT_MOVE;
     if (fastz) fl |= FLAG_FASTZ;

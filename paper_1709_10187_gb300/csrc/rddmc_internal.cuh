@@ -6,8 +6,8 @@
 //    | fast heads uint2[n_class*J] | tau f32[n_class*J] | u_par split points f32x2[kUparN]
 //    | 1/K_s f32[n_class*J] | dust absorption thresholds u32[n_class*J] | dust weights u64[n_class*J]
 //    | dust opacities f32[n_class*J] | pairs 16 B[n_class*J] with pads (tables up to kPairRows rows)
-//    | margins u8[ncell] (with the pairs): spatial moves a packet can make from a cell and stay in its class,
-//    at most 254, or kNoMargin]
+//    | margins u8[ncell] (with the pairs, static grids): spatial moves a packet can make from a cell and stay in its class,
+//    at most 254]
 // With dust absorption (Sec. 2.6) the categorical draw has one more outcome,
 // absorption, after the leakage outcomes: the row thresholds are cumulative over
 // the leakage rates plus k_a, and the absorption threshold (where absorption
@@ -39,7 +39,6 @@ constexpr int kHistOff = 22;
 constexpr int kNsb = 64;            // impact-parameter bins over b/R in [0, kSbMax)
 constexpr double kSbMax = 1.28;
 constexpr int64_t kPairRows = 1 << 20;  // tables up to this many rows carry the walk's pairs (pairs.cuh)
-constexpr unsigned kNoMargin = 255;     // margin of a cell with a Doppler rebin on one of its faces, or with dust
 constexpr int kUparN = 1024;        // |x| grid of the u_par envelope split points
 constexpr float kUparStep = 1.0f / 16.0f;
 

@@ -51,6 +51,11 @@ constexpr unsigned long long kLwMin = 25317190836906ull;
 #ifndef RDDMC_WALK_MIN_BLOCKS
 #define RDDMC_WALK_MIN_BLOCKS 3
 #endif
+// The hybrid kernel's excursions need more: two (128 registers) 10.6 ms, three
+// 11.7 ms on two 4096-step slices of 5e5 packets, 256 x 512 hybrid slab.
+#ifndef RDDMC_WALK_HYBRID_MIN_BLOCKS
+#define RDDMC_WALK_HYBRID_MIN_BLOCKS 2
+#endif
 
 // ---------------------------------------------------------------- hybrid MC
 // Continuous MC of a packet in thin states (Sec. 5.1, Sec. 5.2), in FP32.  It
@@ -304,7 +309,8 @@ __device__ __forceinline__ bool prop_takes(const WalkParams& P, unsigned cell, u
 
 // Per-thread counters in shared memory.
 enum Loc64 { L_STEPS = 0, L_EDRAW = 1, L_MC = 2, kLoc64 = 3 };
-enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6 };
+enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6,
+             L_EVENT_BLK = 6, L_EVENT = 7, kLoc32Events = 11 };  // the event words kept for rebins (3D)  // the block of event words kept for rebins
 
 // How a kernel instantiation reads frequency moves: fast heads through L1 or
 // from shared memory, or pairs through L1.
@@ -320,9 +326,9 @@ enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2 };
 // walked on its rows, again without a branch per transition (walk_four_rows).
 // Two 4096-step slices of 4e6 packets on the 256 x 512 slab: 32.6 ms with heads,
 // 27.7 ms with pairs, 26.1 ms with the rows in groups too; 2e6 packets on its
-// wide-core grid to escape: 205, 184 and 98 ms.
+// wide-core grid to escape: 205, 184 and 98-103 ms.
 template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
-__global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const __grid_constant__ WalkParams P) {
+__global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : RDDMC_WALK_MIN_BLOCKS) walk_kernel(const __grid_constant__ WalkParams P) {
     constexpr int RW = NDIM == 1 ? 1 : 2;  // uint4 per row
     constexpr bool SMEM_ROWS = PATH == HEADS_SMEM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -335,7 +341,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
     // shared memory and leave their registers to the transition loop
     unsigned long long* loc64 = s_hist + (P.hist_in_smem ? ((nhist + 1) & ~1) : 0) + threadIdx.x;
     unsigned* loc32 = reinterpret_cast<unsigned*>(loc64 - threadIdx.x + kLoc64 * blockDim.x) + threadIdx.x;
-    uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + kLoc32 * blockDim.x);
+    constexpr int kSlots = NDIM == 3 ? kLoc32Events : kLoc32;
+    uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + kSlots * blockDim.x);
     auto cnt64 = [&](int i) -> unsigned long long& { return loc64[i * blockDim.x]; };
     auto cnt32 = [&](int i) -> unsigned& { return loc32[i * blockDim.x]; };
 #pragma unroll
@@ -413,23 +420,47 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         return false;
     };
 
-    // One full transition: every threshold, the outcome's action, spatial moves
-    // with the class lookup, Doppler rebins and escapes.  Returns true when the
-    // packet has finished.
-    auto generic = [&](unsigned w) -> bool {
+    // The next event word, for a Doppler rebin of a 3D walk: every fourth draws a
+    // block, kept in shared memory with its index (event indices grow by a few per
+    // transition, so the index's low word names the block).  Drawing one per rebin
+    // cost the sphere in outflow 4 %.
+    auto rebin_word = [&]() -> unsigned {
+        const unsigned long long b = e >> 2;
+        if (cnt32(L_EVENT_BLK) != (unsigned)b) {
+            const uint4 v = philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), (uint32_t)pid,
+                                                 (uint32_t)(pid >> 32) | 0x80000000u), P);
+            cnt32(L_EVENT) = v.x;
+            cnt32(L_EVENT + 1) = v.y;
+            cnt32(L_EVENT + 2) = v.z;
+            cnt32(L_EVENT + 3) = v.w;
+            cnt32(L_EVENT_BLK) = (unsigned)b;
+        }
+        return cnt32(L_EVENT + (int)((unsigned)e++ & 3u));
+    };
+
+    // Outcome of word w in the current state's row, and the row's flags.
+    auto outcome_of = [&](unsigned w, unsigned& fl) -> unsigned {
         const unsigned ri = min(s, nr1);
-        if (WEIGHT) lw += __ldg(&P.wq[ri]);  // the weight kept over the dwell in this state
         const uint4 a = __ldg(&rows[ri * RW]);
         unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
         if (NDIM == 3) {
             const uint4 b = __ldg(&rows[ri * RW + 1]);
             o += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
         }
+        fl = a.w;
+        return o;
+    };
+
+    // One full transition, outcome o of word w: the outcome's action, spatial
+    // moves with the class lookup, Doppler rebins and escapes.  Returns true when
+    // the packet has finished.
+    auto take_outcome = [&](unsigned w, unsigned o, unsigned fl) -> bool {
+        const unsigned ri = min(s, nr1);
+        if (WEIGHT) lw += __ldg(&P.wq[ri]);  // the weight kept over the dwell in this state
         if (P.dust && o == 2u * NDIM + 1u && w >= __ldg(&P.abs_thr[ri])) {  // absorbed by dust (Sec. 2.6)
             atomicAdd(&s_cnt[C_ABSORBED], 1ull);
             return true;
         }
-        const unsigned fl = a.w;
         const unsigned act = (fl >> (2u * o)) & 3u;
         const unsigned bin = min(s - cls * J, J - 1u);
         if (o < 2u) {
@@ -471,7 +502,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         unsigned nbin = bin;
         if (act == ACT_REBIN) {
             const Rebin rb = P.rebin[min(cls, (unsigned)P.n_class - 1u) * (2u * NDIM) + face];
-            const unsigned w1 = event_word(pid, e++, P.k0, P.k1);
+            const unsigned w1 = NDIM == 3 ? rebin_word() : event_word(pid, e++, P.k0, P.k1);
             int jn = (int)bin + rb.m + (w1 >= rb.thr ? 1 : 0);
             if (jn < 0) { jn = 0; ++cnt32(L_CLAMP); }
             if (jn > (int)J - 1) { jn = (int)J - 1; ++cnt32(L_CLAMP); }
@@ -485,20 +516,25 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
         return faded();
     };
 
-    // The transitions q .. 3 of words r, row by row: a plain move (frequency or
-    // spatial) in place, any other outcome through the generic step.  Returns 4,
-    // or the index of the transition that finished the packet.
+    auto generic = [&](unsigned w) -> bool {
+        unsigned fl;
+        const unsigned o = outcome_of(w, fl);
+        return take_outcome(w, o, fl);
+    };
+
+    // The transitions q .. 3 of words r, row by row: plain moves (frequency or
+    // spatial) in place, any other outcome through the generic step.  The lanes
+    // of a warp meet at the generic step, each at its own first such outcome, so
+    // that their rebins, escapes and excursions run together (two 4096-step
+    // slices of 1e6 packets on the 64^3 sphere in outflow: 12.1 -> 11.8 ms).
+    // Returns 4, or the index of the transition that finished the packet.
     auto by_rows = [&](const uint4& r, unsigned q) -> unsigned {
         do {
-            const unsigned w = word_of(r, q);
-            const unsigned ri = min(s, nr1);
-            const uint4 a = __ldg(&rows[ri * RW]);
-            unsigned k = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
-            if (NDIM == 3) {
-                const uint4 b = __ldg(&rows[ri * RW + 1]);
-                k += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
-            }
-            if (((a.w >> (2u * k)) & 3u) == ACT_MOVE && !(P.dust && k == 2u * NDIM + 1u)) {
+            unsigned w = 0, k = 0, fl = 0;
+            for (; q < 4u; ++q) {
+                w = word_of(r, q);
+                k = outcome_of(w, fl);
+                if (((fl >> (2u * k)) & 3u) != ACT_MOVE || (P.dust && k == 2u * NDIM + 1u)) break;
                 if (k < 2u) {
                     s += k ? 1u : 0xffffffffu;
                 } else {
@@ -510,9 +546,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                     s += (c1 - cls) * J;
                     cls = c1;
                 }
-            } else if (generic(w)) {
-                return q;
             }
+            if (q < 4u && take_outcome(w, k, fl)) return q;
         } while (++q < 4u);
         return 4u;
     };
@@ -561,6 +596,7 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                         have = true;
                     }
                     if (have) {
+                        if (NDIM == 3) cnt32(L_EVENT_BLK) = ~(unsigned)(e >> 2);  // not the next event's block
                         cell = min(cell, (unsigned)P.ncell - 1u);
                         cls = __ldg(&P.cell_class[cell]);
                         s = cls * J + min(bin, J - 1u);
@@ -635,12 +671,10 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                     // one group of four on r while the next block is drawn into rn;
                     // true when the packet finished
                     auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
-                        uint32_t o2, o4;
-                        bool ok2, ok4;
-                        walk_four(P.pair, r, o, o2, o4, ok2, ok4);
+                        const FourMoves m = walk_four(P.pair, r, o);
                         rn = ts.next(P);
-                        if (ok4) {
-                            o = min(o4 - 64u, omax);
+                        if (m.ok4) {
+                            o = min(m.o4 - 64u, omax);
                             return false;
                         }
                         s = o >> 4;
@@ -648,8 +682,8 @@ __global__ void __launch_bounds__(256, RDDMC_WALK_MIN_BLOCKS) walk_kernel(const 
                             o = 16u * s;
                             return false;
                         }
-                        if (ok2) s = (o2 - 32u) >> 4;
-                        const unsigned q = by_rows(r, ok2 ? 2u : 0u);
+                        if (m.ok2) s = (m.o2 - 32u) >> 4;
+                        const unsigned q = by_rows(r, m.ok2 ? 2u : 0u);
                         o = min(16u * s, omax);
                         t = 4ull * (blk - behind) + q + 1ull;
                         return q < 4u;
@@ -815,20 +849,25 @@ cudaError_t launch_variant(const WalkParams& P, int threads, size_t smem, int ct
 template <int NDIM, int PATH>
 cudaError_t launch_path(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
     if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, threads, smem, ctas, nsm, s);
-    return P.hybrid ? launch_variant<NDIM, PATH, true, false, false>(P, threads, smem, ctas, nsm, s)
-                    : launch_variant<NDIM, PATH, false, false, false>(P, threads, smem, ctas, nsm, s);
+    if constexpr (NDIM == 1 || PATH != PAIRS)
+        if (P.hybrid) return launch_variant<NDIM, PATH, true, false, false>(P, threads, smem, ctas, nsm, s);
+    return launch_variant<NDIM, PATH, false, false, false>(P, threads, smem, ctas, nsm, s);
 }
 
-// Pairs where the table has them, heads otherwise; the weight method reads
-// heads (its weight is checked before every transition).
+// Pairs where the table has them, heads otherwise.  The weight method reads
+// heads (its weight is checked before every transition), and so does the 3D
+// hybrid, which leaves most groups for an excursion: heads name the first
+// transition that is not a frequency move without reading rows (2048 steps of
+// 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7 against 6.7
+// in a 20 km/s outflow).
 template <int NDIM>
 cudaError_t launch_mode(const WalkParams& P, bool smem_heads, int threads, size_t smem, int ctas, int nsm,
                         cudaStream_t s) {
     if (P.weights)
         return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, threads, smem, ctas, nsm, s)
                           : launch_variant<NDIM, HEADS, false, false, true>(P, threads, smem, ctas, nsm, s);
-    return P.pair ? launch_path<NDIM, PAIRS>(P, threads, smem, ctas, nsm, s)
-                 : launch_path<NDIM, HEADS>(P, threads, smem, ctas, nsm, s);
+    return P.pair && !(NDIM == 3 && P.hybrid) ? launch_path<NDIM, PAIRS>(P, threads, smem, ctas, nsm, s)
+                                              : launch_path<NDIM, HEADS>(P, threads, smem, ctas, nsm, s);
 }
 
 // One scattering per thread at x_in with incoming direction +e_z; sample i
@@ -1267,7 +1306,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.rows = (const uint4*)(tb + g.off_rows);
     P.fast = (const uint2*)(tb + g.off_fast);
     P.pair = g.pairs() ? (const Pair*)(tb + g.off_pair) : nullptr;
-    P.margin = g.pairs() ? (const uint8_t*)(tb + g.off_margin) : nullptr;
+    P.margin = g.margin.empty() ? nullptr : (const uint8_t*)(tb + g.off_margin);
     P.tau_row = (const float*)(tb + g.off_tau);
     P.upar = (const float2*)(tb + g.off_upar);
     P.cdesc = (const ClassDesc*)(tb + g.off_cdesc);
@@ -1368,7 +1407,7 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     const int threads = o.threads_per_cta ? o.threads_per_cta : 256;
     size_t smem = (size_t)(kCounters + 8 + kNsb) * 8;
     if (P.hist_in_smem) smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
-    smem += (size_t)threads * (kLoc64 * 8 + kLoc32 * 4);
+    smem += (size_t)threads * (kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4);
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads
     const bool smem_heads = P.weights && o.table_in_smem && smem + rows_bytes <= (size_t)smem_optin;
     if (smem_heads) smem += rows_bytes;

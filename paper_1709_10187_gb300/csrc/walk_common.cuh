@@ -41,6 +41,7 @@ struct WalkParams {
     uint8_t* st_status;
     unsigned long long* tally;
     unsigned long long n_packets, max_steps, slice, mc_cap;
+    static constexpr bool kDust = true;  // may walk a dusty grid
     unsigned long long time_slice_ns;  // wall-time slice of the launch (0 = none)
     uint32_t k0, k1;
     uint32_t rk0[10], rk1[10];  // Philox round keys k + r * (Weyl constant)

@@ -97,3 +97,33 @@ def test_pairs_and_heads_walk_alike(chunk):
         _same(out[0], out[1], 2)
         for p in (dense, dedup):
             p.close()
+
+
+@pytest.mark.parametrize("case", ["slab", "cube", "sphere_moving"])
+@pytest.mark.parametrize("dust", [0.0, 3.0])
+def test_dusty_and_moving_rows_match_the_oracle(case, dust):
+    # absorbed packets among the groups on the rows; rebins whose event words
+    # come from a kept block, over slices that cut packets between them
+    if case != "sphere_moving" and not dust:
+        pytest.skip("covered above")
+    ndim = 1 if case == "slab" else 3
+    n = {"slab": (20, 1, 1), "cube": (9, 8, 10), "sphere_moving": (12, 12, 12)}[case]
+    w = W.Workload(f"dust_{case}", ndim, n, 21, -42.0, 42.0, 1.0e3, 1.0e4, 4000, 0x5EED0B04,
+                   sphere=case == "sphere_moving", vmax_kms=60.0 if case == "sphere_moving" else 0.0)
+    g = C.Grid(w, dust_abs=dust)
+    ot = g.table()
+    p = R.Problem(w, dust_abs=dust)
+    thr, _ = p.rows()
+    sel = np.ones(w.ncell * w.J, bool) if w.mask() is None else np.repeat(w.mask().astype(bool), w.J)
+    ot["thr"][sel] = thr[sel]
+    orc = C.walk(g, ot, w.seed, 0, w.packets, max_steps=1 << 62)
+    one = p.run(w.packets, w.seed)
+    _same(one, orc, 2 * ndim)
+    assert one["absorbed"] == orc["absorbed"] and (one["absorbed"] > 0) == (dust > 0.0)
+    p.reset()
+    p.launch(w.packets, w.seed, steps_per_launch=12)
+    for _ in range(30):
+        p.launch(w.packets, w.seed, steps_per_launch=12, resume=1)
+    p.launch(w.packets, w.seed, steps_per_launch=1 << 40, resume=1)
+    _same(p.read(), orc, 2 * ndim)
+    p.close()

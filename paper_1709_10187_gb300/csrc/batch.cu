@@ -57,6 +57,7 @@ struct BatchParams {
     uint32_t k0, k1;
     uint32_t rk0[10], rk1[10];
     int chunk;
+    unsigned lanes;  // lanes of a warp that take packets
 };
 
 __device__ __forceinline__ unsigned bword(const uint4& r, unsigned q) {
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LaneInst& L = reinterpret_cast<LaneInst*>(smem_raw)[threadIdx.x];
     const unsigned lane = threadIdx.x & 31u;
-    bool have = false, exhausted = false;
+    bool have = false, exhausted = lane >= P.lanes;
     int inst = -1;
     const Pair* pair = nullptr;
     unsigned nr1 = 0;
@@ -358,16 +359,30 @@ void fill_params(const rddmc_batch* b, const void* d_desc, bool trial, const rdd
     P.chunk = o->chunk ? o->chunk : 256;
 }
 
-cudaError_t enqueue(const rddmc_batch* b, const BatchParams& P, const rddmc_run_opts* o, cudaStream_t s) {
+// Launches the batch on s.  Fewer packets than the lanes of a launch that fills
+// the chip are spread over its schedulers as in the single-grid walk.
+cudaError_t launch(const rddmc_batch* b, BatchParams& P, const rddmc_run_opts* o, int nsm, cudaStream_t s) {
+    const int full = std::max(1, b->default_ctas);  // of 256 threads, per SM
+    const bool few = !o->threads_per_cta && !o->ctas_per_sm && P.total < 256ull * full * nsm;
+    const int threads = o->threads_per_cta ? o->threads_per_cta : (few ? 128 : 256);
+    int ctas = o->ctas_per_sm ? o->ctas_per_sm : full;
+    P.lanes = 32;
+    if (few) {
+        const uint64_t per = 128ull * nsm;
+        ctas = (int)((P.total + per - 1) / per);
+        if (ctas <= 2) P.lanes = (unsigned)((P.total + 4ull * ctas * nsm - 1) / (4ull * ctas * nsm));
+    }
+    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
+    return cudaGetLastError();
+}
+
+cudaError_t enqueue(const rddmc_batch* b, BatchParams& P, const rddmc_run_opts* o, cudaStream_t s) {
     int nsm = 0, dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int threads = o->threads_per_cta ? o->threads_per_cta : 256;
-    const int ctas = o->ctas_per_sm ? o->ctas_per_sm : std::max(1, b->default_ctas);
     if ((e = cudaMemsetAsync(P.cursor, 0, 8, s)) != cudaSuccess) return e;
-    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
-    return cudaGetLastError();
+    return launch(b, P, o, nsm, s);
 }
 
 // The buffers of a batched launch (the same rules for a launch, a graph and the
@@ -521,14 +536,11 @@ int rddmc_batch_graph_create(const rddmc_batch* b, const void* d_desc, const rdd
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return RDDMC_ERR_CUDA;
-    const int threads = o->threads_per_cta ? o->threads_per_cta : 256;
-    const int ctas = o->ctas_per_sm ? o->ctas_per_sm : std::max(1, b->default_ctas);
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return RDDMC_ERR_CUDA;
     cudaMemsetAsync(d_tallies, 0, b->tally_words * 8ull, s);
     cudaMemsetAsync(d_scratch, 0, 8, s);
-    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
-    const cudaError_t le = cudaGetLastError();
+    const cudaError_t le = launch(b, P, o, nsm, s);
     const cudaError_t ce = cudaStreamEndCapture(s, &graph);
     if (le != cudaSuccess || ce != cudaSuccess || !graph) {
         if (graph) cudaGraphDestroy(graph);

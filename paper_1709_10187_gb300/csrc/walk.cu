@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : R
     const unsigned nr1 = (unsigned)P.n_rows - 1u;
     const uint32_t omax = 16u * nr1;  // the last row's pair
     const unsigned long long t_begin = P.time_slice_ns ? global_ns() : 0ull;
-    bool have = false, exhausted = false;
+    bool have = false, exhausted = lane >= P.lanes;
     unsigned long long pid = 0, t = 0, e = 0, t_stop = 0;
     unsigned long long lw = 0;  // weight method: -ln(packet weight) in 2^-40 units
     unsigned cell = 0, cls = 0, s = 0;  // s = cls * J + bin: the row of the state
@@ -831,27 +831,57 @@ __global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : R
         if (s_sb[i]) atomicAdd(&P.tally[kHistOff + nhist + i], s_sb[i]);
 }
 
-template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
-cudaError_t launch_variant(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (!ctas) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>,
-                                                          threads, smem);
-        if (e != cudaSuccess) return e;
+// A launch's threads per CTA and CTAs per SM (0: chosen by launch_variant), the
+// SMs, and the shared memory of a CTA and of each of its threads.
+struct LaunchShape {
+    int threads, ctas_per_sm, sms;
+    size_t smem, smem_per_thread;
+
+    // Fewer packets than the lanes of a launch that fills the chip.
+    bool few(const WalkParams& P) const {
+        return !threads && !ctas_per_sm && P.n_packets < 256ull * RDDMC_WALK_MIN_BLOCKS * (unsigned)sms;
     }
+};
+
+// Few packets crowd on the CTAs that start first, two to six warps on one
+// scheduler while others are idle, and a packet's chain of gathers gains from a
+// scheduler of its own.  Such launches use CTAs of 128 threads, one warp per
+// scheduler, as many per SM as the packets need, and while those are one or two
+// they spread the packets over all warps' lanes (more warps per SM or full
+// warps first measured slower).  To escape on the 64 x 128 slab: 2048 packets
+// 86 -> 70 ms, 2e4 118 -> 85, 4e4 166 -> 103; 16384 steps on the dusty wide-core
+// slab, 2e4 packets 3.6 -> 3.3 ms; 2048 steps on the hybrid sphere, 2e4 packets
+// 4.6 -> 2.6 ms.
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
+cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
+    const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>;
+    const bool few = L.few(P);
+    const int threads = L.threads ? L.threads : (few ? 128 : 256);
+    const size_t smem = L.smem + (size_t)threads * L.smem_per_thread;
+    int ctas = L.ctas_per_sm;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (!ctas &&
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem)) != cudaSuccess)
+        return e;
     if (ctas < 1) ctas = 1;
-    walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT><<<(unsigned)(ctas * nsm), threads, smem, s>>>(P);
+    P.lanes = 32;
+    if (few) {
+        const uint64_t n = P.n_packets, per = (uint64_t)threads * L.sms;
+        ctas = (int)std::min<uint64_t>((uint64_t)ctas, (n + per - 1) / per);
+        const uint64_t warps = (uint64_t)ctas * per / 32;
+        if (ctas <= 2) P.lanes = (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps);
+    }
+    kernel<<<(unsigned)(ctas * L.sms), threads, smem, s>>>(P);
     return cudaGetLastError();
 }
 
 template <int NDIM, int PATH>
-cudaError_t launch_path(const WalkParams& P, int threads, size_t smem, int ctas, int nsm, cudaStream_t s) {
-    if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, threads, smem, ctas, nsm, s);
+cudaError_t launch_path(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
+    if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, L, s);
     if constexpr (NDIM == 1 || PATH != PAIRS)
-        if (P.hybrid) return launch_variant<NDIM, PATH, true, false, false>(P, threads, smem, ctas, nsm, s);
-    return launch_variant<NDIM, PATH, false, false, false>(P, threads, smem, ctas, nsm, s);
+        if (P.hybrid) return launch_variant<NDIM, PATH, true, false, false>(P, L, s);
+    return launch_variant<NDIM, PATH, false, false, false>(P, L, s);
 }
 
 // Pairs where the table has them, heads otherwise.  The weight method reads
@@ -859,15 +889,17 @@ cudaError_t launch_path(const WalkParams& P, int threads, size_t smem, int ctas,
 // hybrid, which leaves most groups for an excursion: heads name the first
 // transition that is not a frequency move without reading rows (2048 steps of
 // 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7 against 6.7
-// in a 20 km/s outflow).
+// in a 20 km/s outflow).  A moving 3D grid leaves them for its rebins: pairs
+// where the launch fills the chip (two 4096-step slices of 1e6 packets on the
+// sphere: 11.2 against 11.9 ms), heads where the latency counts (16384 steps of
+// 2e4 packets 5.0 against 5.4 ms, of 6e4 6.4 against 6.8).
 template <int NDIM>
-cudaError_t launch_mode(const WalkParams& P, bool smem_heads, int threads, size_t smem, int ctas, int nsm,
-                        cudaStream_t s) {
+cudaError_t launch_mode(WalkParams& P, bool smem_heads, const LaunchShape& L, cudaStream_t s) {
     if (P.weights)
-        return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, threads, smem, ctas, nsm, s)
-                          : launch_variant<NDIM, HEADS, false, false, true>(P, threads, smem, ctas, nsm, s);
-    return P.pair && !(NDIM == 3 && P.hybrid) ? launch_path<NDIM, PAIRS>(P, threads, smem, ctas, nsm, s)
-                                              : launch_path<NDIM, HEADS>(P, threads, smem, ctas, nsm, s);
+        return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, L, s)
+                          : launch_variant<NDIM, HEADS, false, false, true>(P, L, s);
+    const bool pairs = P.pair && !(NDIM == 3 && (P.hybrid || (P.moving && L.few(P))));
+    return pairs ? launch_path<NDIM, PAIRS>(P, L, s) : launch_path<NDIM, HEADS>(P, L, s);
 }
 
 // One scattering per thread at x_in with incoming direction +e_z; sample i
@@ -1404,18 +1436,17 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return e;
-    const int threads = o.threads_per_cta ? o.threads_per_cta : 256;
-    size_t smem = (size_t)(kCounters + 8 + kNsb) * 8;
-    if (P.hist_in_smem) smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
-    smem += (size_t)threads * (kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4);
+    LaunchShape L{o.threads_per_cta, o.ctas_per_sm, nsm, (size_t)(kCounters + 8 + kNsb) * 8,
+                  kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4};
+    if (P.hist_in_smem) L.smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads
-    const bool smem_heads = P.weights && o.table_in_smem && smem + rows_bytes <= (size_t)smem_optin;
-    if (smem_heads) smem += rows_bytes;
+    const size_t counters = (size_t)(L.threads ? L.threads : 256) * L.smem_per_thread;
+    const bool smem_heads = P.weights && o.table_in_smem && L.smem + counters + rows_bytes <= (size_t)smem_optin;
+    if (smem_heads) L.smem += rows_bytes;
     if ((e = cudaMemsetAsync(P.cursor, 0, 8, s)) != cudaSuccess) return e;
     if (P.save_state && !o.resume && (e = cudaMemsetAsync(P.st_status, PK_FRESH, o.n_packets, s)) != cudaSuccess)
         return e;
-    return g.ndim == 1 ? launch_mode<1>(P, smem_heads, threads, smem, o.ctas_per_sm, nsm, s)
-                       : launch_mode<3>(P, smem_heads, threads, smem, o.ctas_per_sm, nsm, s);
+    return g.ndim == 1 ? launch_mode<1>(P, smem_heads, L, s) : launch_mode<3>(P, smem_heads, L, s);
 }
 
 }  // namespace rddmc

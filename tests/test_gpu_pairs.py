@@ -127,3 +127,26 @@ def test_dusty_and_moving_rows_match_the_oracle(case, dust):
     p.launch(w.packets, w.seed, steps_per_launch=1 << 40, resume=1)
     _same(p.read(), orc, 2 * ndim)
     p.close()
+
+
+@pytest.mark.parametrize("moving", [False, True])
+def test_small_launches_walk_every_packet_as_full_ones_do(moving):
+    # the default launch shape on both sides of its lines: a lane per warp, one
+    # and two warps per scheduler, a launch that just fills the chip
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = (W.Workload("few_sphere", 3, (6, 6, 6), 9, -9.0, 9.0, 60.0, 1.0e4, 1, 0x5EED0B05, sphere=True, vmax_kms=30.0)
+         if moving else W.Workload("few_slab", 1, (8, 1, 1), 16, -8.0, 8.0, 200.0, 1.0e4, 1, 0x5EED0B05))
+    p = R.Problem(w)
+    for n in (1, 4 * sms, 4 * sms + 1, 128 * sms, 128 * sms + 1, 256 * sms, 256 * sms + 1, 768 * sms - 1, 768 * sms):
+        got = p.run(n, w.seed)
+        assert got["emitted"] == n == got["escaped"]
+        _same(got, p.run(n, w.seed, threads_per_cta=256, ctas_per_sm=3), 2 * w.ndim)
+        m = max(1, n // 3)
+        b = R.Batch([p, p], [m, n])
+        b.launch(R.RunOpts(w.seed, 0, 0))
+        first, second = b.read(0), b.read(1)
+        b.launch(R.RunOpts(w.seed, 0, 0, 0, 0, 3, 256))
+        _same(first, b.read(0), 2 * w.ndim)
+        _same(second, b.read(1), 2 * w.ndim)
+        _same(first, p.run(m, w.seed), 2 * w.ndim)
+    p.close()

@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : R
 // A launch's threads per CTA and CTAs per SM (0: chosen by launch_variant), the
 // SMs, and the shared memory of a CTA and of each of its threads.
 struct LaunchShape {
-    int threads, ctas_per_sm, sms;
+    int threads, ctas_per_sm, chunk, sms;
     size_t smem, smem_per_thread;
 
     // Fewer packets than the lanes of a launch that fills the chip.
@@ -851,7 +851,8 @@ struct LaunchShape {
 // warps first measured slower).  To escape on the 64 x 128 slab: 2048 packets
 // 86 -> 70 ms, 2e4 118 -> 85, 4e4 166 -> 103; 16384 steps on the dusty wide-core
 // slab, 2e4 packets 3.6 -> 3.3 ms; 2048 steps on the hybrid sphere, 2e4 packets
-// 4.6 -> 2.6 ms.
+// 4.6 -> 2.6 ms.  With every packet in a lane from the start the default chunk is
+// 4096 transitions (2048 packets 69 -> 64 ms; 1024: 65, 16384: 64).
 template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
 cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
     const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>;
@@ -871,6 +872,8 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
         ctas = (int)std::min<uint64_t>((uint64_t)ctas, (n + per - 1) / per);
         const uint64_t warps = (uint64_t)ctas * per / 32;
         if (ctas <= 2) P.lanes = (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps);
+        // no lane waits for a new packet, so the queue is asked less often
+        if (!PROPOSE && !P.time_slice_ns && L.chunk == 0 && n <= warps * 32) P.chunk = 4096;
     }
     kernel<<<(unsigned)(ctas * L.sms), threads, smem, s>>>(P);
     return cudaGetLastError();
@@ -1436,7 +1439,7 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return e;
-    LaunchShape L{o.threads_per_cta, o.ctas_per_sm, nsm, (size_t)(kCounters + 8 + kNsb) * 8,
+    LaunchShape L{o.threads_per_cta, o.ctas_per_sm, o.chunk, nsm, (size_t)(kCounters + 8 + kNsb) * 8,
                   kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4};
     if (P.hist_in_smem) L.smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads

@@ -290,8 +290,134 @@ __global__ void softmax_ce_kernel(const float* __restrict__ logits, int n_out, i
     }
 }
 
+// The same with a row of head A in registers, a warp per row: V 16-byte pieces
+// a lane hold its logits from one read to the gradients, V more its columns'
+// sums over the warp's rows; only heads B and C (the columns past nA) sum in
+// shared memory.  nA and n_out are multiples of 4, nA <= 128 V.  Bound by the
+// logits' read and the gradients' write, and before by reading each logit three
+// times, by a shared-memory sum per column and by 608 blocks' atomics on every
+// column: a training step of 8192 rows, 1536 + 32 + 216 logits, 277 -> 195 us.
+template <int V>
+__global__ void __launch_bounds__(V <= 12 ? 512 : 384, 1)
+softmax_ce_rows_kernel(const float* __restrict__ logits, int n_out, int nA, int nB, int nC, int S,
+                       const int* __restrict__ tA, const int* __restrict__ tB, const int* __restrict__ tC, int Bsz,
+                       __nv_bfloat16* __restrict__ dlogb, float* __restrict__ db, float* loss) {
+    extern __shared__ __align__(16) float s_sum[];  // warps x n_out
+    const int warps = (int)blockDim.x >> 5, warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    float* acc = s_sum + (size_t)warp * n_out;
+    for (int k = nA + lane; k < n_out; k += 32) acc[k] = 0.0f;
+    float4 sum[V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) sum[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const int n4 = nA >> 2;
+    // x / Bsz: a product where it is exact
+    const bool pow2 = (Bsz & (Bsz - 1)) == 0;
+    const float inv = 1.0f / (float)Bsz;
+    auto mean = [&](float x) { return pow2 ? x * inv : x / (float)Bsz; };
+    float total = 0.0f;
+    for (int row = (int)blockIdx.x * warps + warp; row < Bsz; row += (int)gridDim.x * warps) {
+        const float* z = logits + (size_t)row * n_out;
+        __nv_bfloat16* gb = dlogb + (size_t)row * n_out;
+        const int ta = tA[row];
+        const bool skip = ta < 0;  // ignored sample: no loss, no gradient
+        for (int k = (skip ? 0 : nA + nB) + lane; k < n_out; k += 32) gb[k] = __float2bfloat16(0.0f);
+        if (skip) continue;
+        int tc = (nC > 0 && tC) ? tC[row] : -1;
+        if (tc >= nC) tc = -1;
+        {
+            float4 v[V];
+            float mx = -3.0e38f;
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if (lane + 32 * i < n4) v[i] = __ldcs(reinterpret_cast<const float4*>(z) + lane + 32 * i);
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if (lane + 32 * i < n4) mx = fmaxf(mx, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            float se = 0.0f;
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if (lane + 32 * i < n4)
+                    se += (__expf(v[i].x - mx) + __expf(v[i].y - mx)) + (__expf(v[i].z - mx) + __expf(v[i].w - mx));
+            for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+            const float lse = mx + __logf(se);
+            total += lse - z[ta];
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                if (lane + 32 * i >= n4) continue;
+                const int k = 4 * (lane + 32 * i);
+                float4 g;
+                g.x = mean(__expf(v[i].x - lse) - (k == ta ? 1.0f : 0.0f));
+                g.y = mean(__expf(v[i].y - lse) - (k + 1 == ta ? 1.0f : 0.0f));
+                g.z = mean(__expf(v[i].z - lse) - (k + 2 == ta ? 1.0f : 0.0f));
+                g.w = mean(__expf(v[i].w - lse) - (k + 3 == ta ? 1.0f : 0.0f));
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(g.x, g.y), hi = __floats2bfloat162_rn(g.z, g.w);
+                *reinterpret_cast<uint2*>(gb + k) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
+                                                               *reinterpret_cast<const uint32_t*>(&hi));
+                sum[i].x += g.x;
+                sum[i].y += g.y;
+                sum[i].z += g.z;
+                sum[i].w += g.w;
+            }
+        }
+        for (int h = 1; h < (tc >= 0 ? 3 : 2); ++h) {
+            const int lo = h == 1 ? nA : nA + nB + (tc / S) * S, hi = h == 1 ? nA + nB : lo + S;
+            const int tgt = h == 1 ? nA + tB[row] : nA + nB + tc;
+            float mx = -3.0e38f;
+            for (int k = lo + lane; k < hi; k += 32) mx = fmaxf(mx, z[k]);
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            float se = 0.0f;
+            for (int k = lo + lane; k < hi; k += 32) se += __expf(z[k] - mx);
+            for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+            const float lse = mx + __logf(se);
+            total += lse - z[tgt];
+            __syncwarp();  // the zeros above and the columns of the last head come from other lanes
+            for (int k = lo + lane; k < hi; k += 32) {
+                const float g = (__expf(z[k] - lse) - (k == tgt ? 1.0f : 0.0f)) / (float)Bsz;
+                gb[k] = __float2bfloat16(g);
+                acc[k] += g;
+            }
+        }
+        __syncwarp();
+    }
+    if (lane == 0 && total != 0.0f) atomicAdd(loss, total);
+#pragma unroll
+    for (int i = 0; i < V; ++i)
+        if (lane + 32 * i < n4) reinterpret_cast<float4*>(acc)[lane + 32 * i] = sum[i];
+    __syncthreads();
+    for (int k = (int)threadIdx.x; k < n_out; k += (int)blockDim.x) {
+        float t = 0.0f;
+        for (int w = 0; w < warps; ++w) t += s_sum[(size_t)w * n_out + k];
+        if (t != 0.0f) atomicAdd(&db[k], t);
+    }
+}
+
+template <int V>
+cudaError_t softmax_ce_rows(const float* logits, int n_out, int nA, int nB, int nC, int S, const int* tA, const int* tB,
+                            const int* tC, int Bsz, __nv_bfloat16* dlogb, float* db, float* loss, cudaStream_t s) {
+    const int warps = V <= 12 ? 16 : 12;
+    const size_t smem = (size_t)warps * n_out * sizeof(float);
+    int dev = 0, nsm = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(softmax_ce_rows_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+            cudaSuccess)
+        return e;
+    softmax_ce_rows_kernel<V><<<std::min((Bsz + warps - 1) / warps, nsm), warps * 32, smem, s>>>(
+        logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb, db, loss);
+    return cudaGetLastError();
+}
+
 cudaError_t softmax_ce(const float* logits, int n_out, int nA, int nB, int nC, int S, const int* tA, const int* tB,
                        const int* tC, int Bsz, __nv_bfloat16* dlogb, float* db, float* loss, cudaStream_t s) {
+    // rows that fit a warp's registers and, 16 at a time, a block's shared memory
+    // (grids of up to 341 bins); the heads' columns one by one otherwise
+    if (nA % 4 == 0 && n_out % 4 == 0 && nA <= 2048 && n_out <= 3200) {
+        const auto rows = nA <= 512 ? softmax_ce_rows<4>
+                                    : (nA <= 1024 ? softmax_ce_rows<8> : (nA <= 1536 ? softmax_ce_rows<12> : softmax_ce_rows<16>));
+        return rows(logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb, db, loss, s);
+    }
     // at most 64 KiB of column sums a block (three blocks per SM), 8 warps while they fit
     const size_t row = (size_t)n_out * sizeof(float);
     const int warps = (int)std::max<size_t>(1, std::min<size_t>(8, (64u * 1024u) / row));

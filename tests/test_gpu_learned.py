@@ -250,3 +250,61 @@ def test_network_gradients_for_narrow_and_wide_heads(n_out, nA, nB):
     worst = int(np.argmax(err / bound))
     assert np.all(err <= bound), (n_out, worst, g[worst], g_ref[worst], g_abs[worst],
                                   float((err / (g_abs + 1e-30)).max()))
+
+
+@pytest.mark.parametrize("nA,nC", [(4, 0), (512, 24), (516, 24), (1024, 0), (1536, 150), (1540, 150), (2048, 24),
+                                   (2052, 24), (222, 24)])
+@pytest.mark.parametrize("batch", [64, 192])
+def test_logit_gradients_at_the_edges_of_the_row_widths(nA, nC, batch):
+    """Heads at the widths up to which a row is held in a warp's registers and
+    past them, with the slice head C, ignored samples and a batch that is not a
+    power of two: loss, BF16 logit gradients and their column sums against FP64
+    on the device's own FP32 logits (both lie in the work buffer)."""
+    B.build()
+    nB, S = 32, max(1, nC // 6)
+    n_out = (nA + nB + nC + 15) // 16 * 16
+    rng = np.random.default_rng(nA + batch)
+    n_par = R.mlp_param_count(n_out)
+    wf = torch.tensor(rng.normal(0.0, 0.1, n_par).astype(np.float32), device="cuda")
+    wb = torch.empty(n_par, dtype=torch.bfloat16, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    R.mlp_to_bf16(n_out, wf.data_ptr(), wb.data_ptr(), s)
+    X = torch.tensor(rng.normal(0.0, 1.0, (batch, 16)), dtype=torch.bfloat16, device="cuda")
+    tA, tB = rng.integers(0, nA, batch), rng.integers(0, nB, batch)
+    tA[::7] = -1
+    tC = rng.integers(-1, nC, batch) if nC else np.full(batch, -1)
+    dev = [torch.tensor(t, dtype=torch.int32, device="cuda") for t in (tA, tB, tC)]
+    work = torch.empty(R.mlp_work_bytes(batch, n_out), dtype=torch.uint8, device="cuda")
+    grad = torch.empty(n_par, dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    R.mlp_loss_grad(n_out, nA, nB, wf.data_ptr(), wb.data_ptr(), X.data_ptr(), dev[0].data_ptr(), dev[1].data_ptr(),
+                    batch, work.data_ptr(), grad.data_ptr(), loss.data_ptr(), s, nC=nC, S=S if nC else 0,
+                    d_tc=dev[2].data_ptr() if nC else 0)
+    R.mlp_status(s)
+    up = lambda v: (v + 255) // 256 * 256
+    o = 5 * up(batch * 256)
+    z = work[o:o + batch * n_out * 4].view(torch.float32).view(batch, n_out).double().cpu().numpy()
+    o += up(batch * n_out * 4)
+    got = work[o:o + batch * n_out * 2].view(torch.bfloat16).view(batch, n_out).double().cpu().numpy()
+    prob, hot, ref_loss = np.zeros_like(z), np.zeros_like(z), 0.0
+    for r in np.flatnonzero(tA >= 0):
+        heads = [(0, nA, tA[r]), (nA, nA + nB, nA + tB[r])]
+        if tC[r] >= 0:
+            lo = nA + nB + (tC[r] // S) * S
+            heads.append((lo, lo + S, nA + nB + tC[r]))
+        for lo, hi, t in heads:
+            e = np.exp(z[r, lo:hi] - z[r, lo:hi].max())
+            prob[r, lo:hi] = e / e.sum()
+            hot[r, t] += 1.0
+            ref_loss -= np.log(prob[r, t])
+    g = (prob - hot) / batch
+    # the fast exponential of arguments above -20 (26 ulp) and the FP32 log-sum:
+    # 1e-5 of a probability; p - 1 in FP32: 1e-7.  Rounding to BF16 is monotone, so
+    # the stored value lies between the two ends' roundings
+    tol = (1e-5 * prob + 1e-7 * hot) / batch
+    assert np.all((_bf16(g - tol) <= got) & (got <= _bf16(g + tol)))
+    assert np.all(got[(prob == 0.0) & (hot == 0.0)] == 0.0)
+    # column sums: the terms' own errors and one FP32 rounding per addition
+    db = grad[n_par - n_out:].double().cpu().numpy()
+    assert np.all(np.abs(db - g.sum(axis=0)) <= tol.sum(axis=0) + 2.0 ** -23 * batch * np.abs(g).sum(axis=0))
+    assert float(loss.item()) == pytest.approx(ref_loss, rel=1e-5)

@@ -368,9 +368,9 @@ cudaError_t launch(const rddmc_batch* b, BatchParams& P, const rddmc_run_opts* o
     int ctas = o->ctas_per_sm ? o->ctas_per_sm : full;
     P.lanes = 32;
     if (few) {
-        const uint64_t per = 128ull * nsm;
-        ctas = (int)((P.total + per - 1) / per);
-        if (ctas <= 2) P.lanes = (unsigned)((P.total + 4ull * ctas * nsm - 1) / (4ull * ctas * nsm));
+        const Spread f = spread(P.total, 2 * full, nsm);
+        ctas = f.ctas;
+        P.lanes = f.lanes;
     }
     batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
     return cudaGetLastError();

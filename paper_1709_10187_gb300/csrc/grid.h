@@ -6,6 +6,25 @@
 #include "../../include/rddmc.h"
 #include "rddmc_internal.cuh"
 
+namespace rddmc {
+// Few packets (fewer than a launch that fills the chip has lanes) on CTAs of 128
+// threads, one warp per scheduler: as many CTAs per SM as they need, at most
+// `most`, and the lanes of a warp that take packets, so that one or two warps
+// per scheduler share them evenly.
+struct Spread {
+    int ctas;
+    unsigned lanes;
+    bool all;  // every packet has a lane at once
+};
+inline Spread spread(uint64_t n, int most, int sms) {
+    const uint64_t per = 128ull * (unsigned)sms, need = (n + per - 1) / per;
+    Spread f{(int)(need < (uint64_t)most ? need : (uint64_t)most), 32u, need <= (uint64_t)most};
+    const uint64_t warps = 4ull * (unsigned)sms * (unsigned)f.ctas;
+    if (f.all && f.ctas <= 2) f.lanes = (unsigned)((n + warps - 1) / warps);
+    return f;
+}
+}  // namespace rddmc
+
 struct rddmc_grid {
     int ndim = 1;
     int n[3] = {1, 1, 1};

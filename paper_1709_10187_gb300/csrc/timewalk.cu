@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
     const unsigned J = (unsigned)P.J;
     const unsigned nr1 = (unsigned)P.n_rows - 1u;
     const unsigned ns1 = (unsigned)T.n_states - 1u;
-    bool have = false, exhausted = false;
+    bool have = false, exhausted = lane >= P.lanes;
     unsigned long long pid = 0, t = 0, e = 0, d = 0;
     unsigned cell = 0, cls = 0, s = 0;  // s = cls * J + bin: the row of the state
     unsigned st = 0;                    // cell * J + bin: the state of the tallies
@@ -448,23 +448,38 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
         }
 }
 
+// Fewer packets than lanes are spread over the schedulers, as in the persistent
+// walk: 12 steps of 1.8 diffusion times, 2.6e4 packets on a 140 x 22 slab, 25.0 ->
+// 18.6 ms (steps of a few transitions are no faster).
 template <int NDIM, bool SMEM_TALLY, int MINB, bool LEAK, bool WEIGHT>
-cudaError_t launch_time_minb(const WalkParams& P, const TimeParams& T, int threads, size_t smem, int ctas, int nsm,
+cudaError_t launch_time_minb(WalkParams& P, const TimeParams& T, int threads, size_t smem, int ctas, int nsm,
                              cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(time_kernel<NDIM, SMEM_TALLY, MINB, LEAK, WEIGHT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const auto kernel = time_kernel<NDIM, SMEM_TALLY, MINB, LEAK, WEIGHT>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    const bool chosen = !threads && !ctas;
+    if (!threads) threads = 256;
     if (!ctas) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, time_kernel<NDIM, SMEM_TALLY, MINB, LEAK, WEIGHT>, threads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem);
         if (e != cudaSuccess) return e;
     }
     if (ctas < 1) ctas = 1;
-    time_kernel<NDIM, SMEM_TALLY, MINB, LEAK, WEIGHT><<<(unsigned)(ctas * nsm), threads, smem, s>>>(P, T);
+    if (chosen && P.n_packets < (uint64_t)ctas * threads * nsm) {
+        int most = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, 128, smem)) != cudaSuccess) return e;
+        const Spread f = spread(P.n_packets, std::max(1, most), nsm);
+        if (f.all) {
+            threads = 128;
+            ctas = f.ctas;
+            P.lanes = f.lanes;
+        }
+    }
+    kernel<<<(unsigned)(ctas * nsm), threads, smem, s>>>(P, T);
     return cudaGetLastError();
 }
 
 template <int NDIM, bool SMEM_TALLY>
-cudaError_t launch_time(const WalkParams& P, const TimeParams& T, int threads, size_t smem, int ctas, int nsm,
+cudaError_t launch_time(WalkParams& P, const TimeParams& T, int threads, size_t smem, int ctas, int nsm,
                         cudaStream_t s) {
     // default and ctas_per_sm >= 3: the 24-warp variant (faster on short steps);
     // ctas_per_sm 1 or 2: the spill-free 16-warp one
@@ -556,7 +571,7 @@ extern "C" int rddmc_time_step_launch(const rddmc_grid* g, const void* d_table, 
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return RDDMC_ERR_CUDA;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RDDMC_ERR_CUDA;
-    const int threads = ts->threads_per_cta ? ts->threads_per_cta : 256;
+    const int threads = ts->threads_per_cta;
     size_t smem = (size_t)(kCounters + 8 + kNsb) * 8;
     if (P.hist_in_smem) smem += (size_t)(g->J + 2) * 8;
     // per-state tallies in shared memory while they fit the budget (u32 bin

@@ -866,14 +866,12 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem)) != cudaSuccess)
         return e;
     if (ctas < 1) ctas = 1;
-    P.lanes = 32;
     if (few) {
-        const uint64_t n = P.n_packets, per = (uint64_t)threads * L.sms;
-        ctas = (int)std::min<uint64_t>((uint64_t)ctas, (n + per - 1) / per);
-        const uint64_t warps = (uint64_t)ctas * per / 32;
-        if (ctas <= 2) P.lanes = (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps);
+        const Spread f = spread(P.n_packets, ctas, L.sms);
+        ctas = f.ctas;
+        P.lanes = f.lanes;
         // no lane waits for a new packet, so the queue is asked less often
-        if (!PROPOSE && !P.time_slice_ns && L.chunk == 0 && n <= warps * 32) P.chunk = 4096;
+        if (!PROPOSE && !P.time_slice_ns && L.chunk == 0 && f.all) P.chunk = 4096;
     }
     kernel<<<(unsigned)(ctas * L.sms), threads, smem, s>>>(P);
     return cudaGetLastError();
@@ -1399,6 +1397,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.chunk = o.chunk ? o.chunk : 256;
     P.resume = o.resume;
     P.save_state = (o.steps_per_launch != 0 || o.resume || o.time_slice_us > 0) ? 1 : 0;
+    P.lanes = 32;
     P.hist_in_smem = (g.J + 2 <= kSmemHistMax) ? 1 : 0;
     P.moving = g.moving ? 1 : 0;
     for (int a = 0; a < 3; ++a) {

@@ -285,6 +285,7 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
     std::vector<ClassDesc> cd(g->n_class);
     std::vector<Rebin> rb((size_t)g->n_class * g->nfaces);
     const double dx0 = g->edges[1] - g->edges[0];
+    g->tau_cell = 0.0;
     for (int k = 0; k < g->n_class; ++k) {
         const int64_t c = g->class_rep[k];
         int idx[3];
@@ -292,6 +293,7 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
         ClassDesc& D = cd[k];
         std::memset(&D, 0, sizeof(D));
         D.k0 = g->tau0 / g->R * g->n_rel[c];
+        g->tau_cell = std::fmax(g->tau_cell, D.k0 * 2.0 * g->R / g->n[0]);
         D.ks = p->dust_scat / g->R * g->n_rel[c];
         D.ka = p->dust_abs / g->R * g->n_rel[c];
         D.moving = (!g->v.empty() && (g->v[3 * c] != 0.0 || g->v[3 * c + 1] != 0.0 || g->v[3 * c + 2] != 0.0)) ? 1 : 0;

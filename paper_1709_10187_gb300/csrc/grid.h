@@ -57,6 +57,7 @@ struct rddmc_grid {
              off_margin = 0, table_bytes = 0;
     // leakage parameters of the last precompute
     rddmc_leak_params params{};
+    double tau_cell = 0.0;  // largest line-centre optical depth of a cell (last precompute)
     bool precomputed = false;
     // dust absorption as an outcome of the draw, or by packet weights (Sec. 2.6)
     bool dusty() const { return params.dust_abs > 0.0 && params.dust_method == RDDMC_DUST_PROBABILISTIC; }

@@ -313,8 +313,10 @@ enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CO
              L_EVENT_BLK = 6, L_EVENT = 7, kLoc32Events = 11 };  // the event words kept for rebins (3D)  // the block of event words kept for rebins
 
 // How a kernel instantiation reads frequency moves: fast heads through L1 or
-// from shared memory, or pairs through L1.
-enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2 };
+// from shared memory, pairs through L1, or not at all (every transition on its
+// row: a moving grid of thin cells, where most transitions cross a Doppler shift
+// and speculative frequency moves are gathers in vain).
+enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2, ROWS = 3 };
 
 // What bounds it: dispatch.  A Philox block costs 17 wide products (3.65 cycles
 // of the multiply pipe each) and 19 xors, measured at 81 cycles per warp and
@@ -327,8 +329,8 @@ enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2 };
 // Two 4096-step slices of 4e6 packets on the 256 x 512 slab: 32.6 ms with heads,
 // 27.7 ms with pairs, 26.1 ms with the rows in groups too; 2e6 packets on its
 // wide-core grid to escape: 205, 184 and 98-103 ms.
-template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
-__global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : RDDMC_WALK_MIN_BLOCKS) walk_kernel(const __grid_constant__ WalkParams P) {
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT, int MINB>
+__global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__ WalkParams P) {
     constexpr int RW = NDIM == 1 ? 1 : 2;  // uint4 per row
     constexpr bool SMEM_ROWS = PATH == HEADS_SMEM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -720,6 +722,10 @@ __global__ void __launch_bounds__(256, HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : R
                 goto slow;                                                                    \
             }                                                                                 \
         }
+                    if constexpr (PATH == ROWS) {
+                        q = 0u;
+                        goto slow;
+                    }
                     if (!WEIGHT) {
                         // The group's four transitions as one branch-free chain: each
                         // head is loaded at the state the previous transition would
@@ -837,9 +843,14 @@ struct LaunchShape {
     int threads, ctas_per_sm, chunk, sms;
     size_t smem, smem_per_thread;
 
-    // Fewer packets than the lanes of a launch that fills the chip.
-    bool few(const WalkParams& P) const {
-        return !threads && !ctas_per_sm && P.n_packets < 256ull * RDDMC_WALK_MIN_BLOCKS * (unsigned)sms;
+    // Fewer packets than the lanes of a launch that fills the chip with `blocks`
+    // CTAs of 256 threads per SM.
+    bool few(const WalkParams& P, int blocks = RDDMC_WALK_MIN_BLOCKS) const {
+        return !threads && !ctas_per_sm && P.n_packets < 256ull * blocks * (unsigned)sms;
+    }
+    // More than that, and at most two rounds of four CTAs per SM.
+    bool two_rounds(const WalkParams& P) const {
+        return !threads && !ctas_per_sm && !few(P) && P.n_packets <= 2048ull * (unsigned)sms;
     }
 };
 
@@ -853,10 +864,11 @@ struct LaunchShape {
 // slab, 2e4 packets 3.6 -> 3.3 ms; 2048 steps on the hybrid sphere, 2e4 packets
 // 4.6 -> 2.6 ms.  With every packet in a lane from the start the default chunk is
 // 4096 transitions (2048 packets 69 -> 64 ms; 1024: 65, 16384: 64).
-template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT>
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT,
+          int MINB = HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : RDDMC_WALK_MIN_BLOCKS>
 cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
-    const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT>;
-    const bool few = L.few(P);
+    const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT, MINB>;
+    const bool few = L.few(P, std::max(MINB, RDDMC_WALK_MIN_BLOCKS));
     const int threads = L.threads ? L.threads : (few ? 128 : 256);
     const size_t smem = L.smem + (size_t)threads * L.smem_per_thread;
     int ctas = L.ctas_per_sm;
@@ -877,11 +889,18 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
     return cudaGetLastError();
 }
 
+// A 3D walk of one to two rounds of packets takes four CTAs per SM (64
+// registers): its second round is short, and more of the packets are in the
+// first (two 944-step slices of 1.3e5 packets on a 14^3 moving sphere: 3.1 -> 2.3 ms;
+// more packets are faster with three).
 template <int NDIM, int PATH>
 cudaError_t launch_path(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
-    if (NDIM == 3 && P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, L, s);
-    if constexpr (NDIM == 1 || PATH != PAIRS)
+    if constexpr (NDIM == 3 && PATH != ROWS)
+        if (P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, L, s);
+    if constexpr (NDIM == 1 || PATH == HEADS)
         if (P.hybrid) return launch_variant<NDIM, PATH, true, false, false>(P, L, s);
+    if constexpr (NDIM == 3)
+        if (L.two_rounds(P)) return launch_variant<NDIM, PATH, false, false, false, 4>(P, L, s);
     return launch_variant<NDIM, PATH, false, false, false>(P, L, s);
 }
 
@@ -891,15 +910,19 @@ cudaError_t launch_path(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
 // transition that is not a frequency move without reading rows (2048 steps of
 // 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7 against 6.7
 // in a 20 km/s outflow).  A moving 3D grid leaves them for its rebins: pairs
-// where the launch fills the chip (two 4096-step slices of 1e6 packets on the
-// sphere: 11.2 against 11.9 ms), heads where the latency counts (16384 steps of
-// 2e4 packets 5.0 against 5.4 ms, of 6e4 6.4 against 6.8).
+// where its cells are thick and the launch fills the chip (two 4096-step slices
+// of 1e6 packets on the sphere: 11.2 against 11.9 ms), heads where the latency
+// counts (16384 steps of 2e4 packets 5.0 against 5.4 ms, of 6e4 6.4 against 6.8),
+// rows alone below kThinCell (2e4 packets to escape from a 13^3 sphere of
+// tau_cell 82, where 99 % of the transitions rebin: 96 against 120 ms).
 template <int NDIM>
 cudaError_t launch_mode(WalkParams& P, bool smem_heads, const LaunchShape& L, cudaStream_t s) {
     if (P.weights)
         return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, L, s)
                           : launch_variant<NDIM, HEADS, false, false, true>(P, L, s);
-    const bool pairs = P.pair && !(NDIM == 3 && (P.hybrid || (P.moving && L.few(P))));
+    if constexpr (NDIM == 3)
+        if (P.thin && !P.prop_b && !P.hybrid) return launch_path<NDIM, ROWS>(P, L, s);
+    const bool pairs = P.pair && !(NDIM == 3 && (P.hybrid || (P.moving && (L.few(P, 4) || !P.thick))));
     return pairs ? launch_path<NDIM, PAIRS>(P, L, s) : launch_path<NDIM, HEADS>(P, L, s);
 }
 
@@ -1398,6 +1421,8 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.resume = o.resume;
     P.save_state = (o.steps_per_launch != 0 || o.resume || o.time_slice_us > 0) ? 1 : 0;
     P.lanes = 32;
+    P.thin = g.moving && g.tau_cell < kThinCell ? 1 : 0;
+    P.thick = g.tau_cell >= kThickCell ? 1 : 0;
     P.hist_in_smem = (g.J + 2 <= kSmemHistMax) ? 1 : 0;
     P.moving = g.moving ? 1 : 0;
     for (int a = 0; a < 3; ++a) {

@@ -150,3 +150,24 @@ def test_small_launches_walk_every_packet_as_full_ones_do(moving):
         _same(second, b.read(1), 2 * w.ndim)
         _same(first, p.run(m, w.seed), 2 * w.ndim)
     p.close()
+
+
+@pytest.mark.parametrize("tau0", [1.0e3, 4.0e3, 1.2e4])
+def test_moving_grids_of_thin_and_thick_cells_match_the_oracle(tau0):
+    # cells of optical depth 250, 1000 and 3000: rows only, and either side of the
+    # line between heads and pairs, in launches below, at and past one round
+    w = W.Workload(f"cells_{tau0:.0f}", 3, (8, 8, 8), 12, -7.0, 7.0, tau0, 1.0e4, 1, 0x5EED0B06, sphere=True,
+                   vmax_kms=40.0)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = C.Grid(w)
+    ot = g.table()
+    p = R.Problem(w)
+    thr, _ = p.rows()
+    sel = np.repeat(w.mask().astype(bool), w.J)
+    ot["thr"][sel] = thr[sel]
+    for n in (3000, 800 * sms, 2100 * sms):
+        p.reset()
+        p.launch(n, w.seed, steps_per_launch=40)
+        p.launch(n, w.seed, steps_per_launch=40, resume=1, max_steps=77)
+        _same(p.read(), C.walk(g, ot, w.seed, 0, n, max_steps=77), 6)
+    p.close()

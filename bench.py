@@ -31,9 +31,9 @@ from paper_1709_10187_gb300 import workloads as W  # noqa: E402
 
 METRIC = "packet transitions/s (rDDMC walk, tau0=1e7 slab)"
 UNIT = "transitions/s"
-# Gather bytes per transition of the slab walk: the 8-byte fast head of the
-# state's row (a frequency move, ~all transitions at this resolution); the
-# generic step's 16-byte row is read on the rare other outcomes.
+# Gather bytes per transition of the slab walk: one 16-byte pair decides two
+# frequency moves (~all transitions at this resolution); the rows are read on
+# the rare other outcomes.
 GATHER_BYTES = 8
 PEAK_SM_MHZ = 2070.0  # maximum SM clock of a GB300
 N_SM = 152
@@ -265,7 +265,9 @@ def run_native(args, rank, world, local_rank):
         # to the host (rddmc_read_tallies, synchronising).
         e2e_steps = max(1, min(args.steps, 5))
         sz = R.grid_sizes(prob.grid, 1)
-        h2d = int(sz.table_bytes - prob.J * sz.row_bytes * sz.n_class)
+        # per step: the header, the cells' classes and margins, the class
+        # descriptors, the rebins of each class's two faces and the bin edges
+        h2d = int(200 + 5 * w.ncell + sz.n_class * (224 + 2 * 8) + 8 * (prob.J + 1))
         t0 = time.perf_counter()
         e2e_trans = 0
         for i in range(e2e_steps):
@@ -305,13 +307,13 @@ def run_native(args, rank, world, local_rank):
     if world == 1 and not args.no_gather:
         with torch.cuda.stream(stream):
             gp = _gather_peaks(R, torch)
-        l1 = gp["l1_8B_32KiB"]
+        l1 = gp["l1_16B_32KiB"]
         gather_gbs = GATHER_BYTES * trans_per_launch / mean_launch_s / 1e9
         roof["gather"] = {"achieved": gather_gbs, "peak": l1["GB_per_s"], "unit": "GB/s",
                           "frac": gather_gbs / l1["GB_per_s"],
-                          "note": f"{GATHER_BYTES}-byte fast heads per transition against the measured random "
-                                  "dependent-gather rate of 8-byte rows from a 32 KiB table through L1 (the "
-                                  "C2 table's footprint; rddmc_gather_probe, best of two occupancies)",
+                          "note": "a 16-byte pair per two transitions against the measured random "
+                                  "dependent-gather rate of 16-byte rows from a 32 KiB table through L1 (the "
+                                  "C2 pairs' footprint; rddmc_gather_probe, best of two occupancies)",
                           "probe": gp}
         roof["gather_frac"] = roof["gather"]["frac"]
     line = {

@@ -465,9 +465,7 @@ cudaError_t launch_time_minb(WalkParams& P, const TimeParams& T, int threads, si
     }
     if (ctas < 1) ctas = 1;
     if (chosen && P.n_packets < (uint64_t)ctas * threads * nsm) {
-        int most = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, 128, smem)) != cudaSuccess) return e;
-        const Spread f = spread(P.n_packets, std::max(1, most), nsm);
+        const Spread f = spread(P.n_packets, ctas, nsm);  // as many of half the size fit for certain
         if (f.all) {
             threads = 128;
             ctas = f.ctas;

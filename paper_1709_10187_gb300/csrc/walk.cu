@@ -909,7 +909,10 @@ cudaError_t launch_path(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
 // hybrid, which leaves most groups for an excursion: heads name the first
 // transition that is not a frequency move without reading rows (2048 steps of
 // 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7 against 6.7
-// in a 20 km/s outflow).  A moving 3D grid leaves them for its rebins: pairs
+// in a 20 km/s outflow); hybrid slabs do below cells of kThickHybrid (two slices
+// of 2856 steps, 5.3e4 packets at tau_cell 1.9e3 9.4 against 11.7 ms; at 2.4e4 1.6
+// against 1.9; at 5.8e4 pairs 5.1 against 5.3, at 4.5e5 3.9 against 4.5).  A moving
+// 3D grid leaves them for its rebins: pairs
 // where its cells are thick and the launch fills the chip (two 4096-step slices
 // of 1e6 packets on the sphere: 11.2 against 11.9 ms), heads where the latency
 // counts (16384 steps of 2e4 packets 5.0 against 5.4 ms, of 6e4 6.4 against 6.8),
@@ -922,7 +925,9 @@ cudaError_t launch_mode(WalkParams& P, bool smem_heads, const LaunchShape& L, cu
                           : launch_variant<NDIM, HEADS, false, false, true>(P, L, s);
     if constexpr (NDIM == 3)
         if (P.thin && !P.prop_b && !P.hybrid) return launch_path<NDIM, ROWS>(P, L, s);
-    const bool pairs = P.pair && !(NDIM == 3 && (P.hybrid || (P.moving && (L.few(P, 4) || !P.thick))));
+    const bool heads = (P.hybrid && (NDIM == 3 || !P.thick_hybrid)) ||
+                       (NDIM == 3 && P.moving && (L.few(P, 4) || !P.thick));
+    const bool pairs = P.pair && !heads;
     return pairs ? launch_path<NDIM, PAIRS>(P, L, s) : launch_path<NDIM, HEADS>(P, L, s);
 }
 
@@ -1423,6 +1428,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.lanes = 32;
     P.thin = g.moving && g.tau_cell < kThinCell ? 1 : 0;
     P.thick = g.tau_cell >= kThickCell ? 1 : 0;
+    P.thick_hybrid = g.tau_cell >= kThickHybrid ? 1 : 0;
     P.hist_in_smem = (g.J + 2 <= kSmemHistMax) ? 1 : 0;
     P.moving = g.moving ? 1 : 0;
     for (int a = 0; a < 3; ++a) {

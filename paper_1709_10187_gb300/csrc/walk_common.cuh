@@ -41,7 +41,7 @@ struct WalkParams {
     uint8_t* st_status;
     unsigned long long* tally;
     unsigned long long n_packets, max_steps, slice, mc_cap;
-    int thin, thick;  // a moving grid of cells below kThinCell; a grid of cells of kThickCell or more
+    int thin, thick, thick_hybrid;  // a moving grid of cells below kThinCell; cells of kThickCell, kThickHybrid or more
     unsigned lanes;  // lanes of a warp that take packets (the persistent walk)
     static constexpr bool kDust = true;  // may walk a dusty grid
     unsigned long long time_slice_ns;  // wall-time slice of the launch (0 = none)

@@ -283,7 +283,8 @@ __global__ void __launch_bounds__(256, MINB) time_kernel(const WalkParams P, con
     auto pass = [&]() -> int {
         const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
         const unsigned k0 = (unsigned)t & 3u;
-        const unsigned long long room = P.max_steps - t;
+        // none for a packet resumed past a limit lower than the last step's
+        const unsigned long long room = t < P.max_steps ? P.max_steps - t : 0ull;
         const unsigned k1 = room < 4ull - k0 ? k0 + (unsigned)room : 4u;
         const uint4 rn = trans_block(t >> 2, pl, ph, P);
         // dwell words w .. w + 3 with w = d - k0 (d >= t: a packet draws a dwell

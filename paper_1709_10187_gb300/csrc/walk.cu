@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
         unsigned long long lim = PROPOSE ? (t / (unsigned long long)P.chunk + 1ull) * (unsigned long long)P.chunk : ~0ull;
         lim = lim < t_stop ? lim : t_stop;
         lim = lim < P.max_steps ? lim : P.max_steps;
+        lim = lim > t ? lim : t;  // resumed past a limit lower than the last launch's: no transition
         const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
         if (have) {
             const unsigned long long lim0 = lim;

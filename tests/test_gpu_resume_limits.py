@@ -60,3 +60,47 @@ def test_time_step_with_a_lower_limit_aborts_at_once(w):
     assert left["aborted"] - t["aborted"] + esc + stay == alive
     assert int(bins[2].sum()) == stay and left["steps"] - t["steps"] == moves
     p.close()
+
+
+PATHS = ["pairs", "heads", "hybrid", "hybrid thick", "weights", "cube", "rows", "thick moving", "proposal"]
+
+
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("limit", [1, 63, 64, 97])
+def test_walk_with_a_lower_limit_aborts_at_once(path, limit):
+    # every way of reading transitions: pairs, heads (a table past the pairs' row
+    # count, a hybrid slab, the weight method), rows, and parking for a proposal
+    cube = W.Workload("limit_cube", 3, (8, 8, 8), 16, -9.0, 9.0, 2.0e5, 1.0e4, 1, 0x5EED0C01)
+    kw = {}
+    if path == "pairs":
+        w = W.C1
+    elif path == "heads":
+        w, kw = W.Workload("limit_dense", 1, (2050, 1, 1), 512, -60.0, 60.0, 1.0e8, 1.0e4, 1, 1), dict(
+            layout=R.LAYOUT_DENSE)
+    elif path.startswith("hybrid"):
+        w, kw = W.C1.with_(tau0=2.0e6 if path == "hybrid thick" else 1.0e5), dict(mode=R.MODE_HYBRID)
+    elif path == "weights":
+        w, kw = W.C1, dict(dust_abs=1e-3, dust_weights=True)
+    else:
+        w = {"rows": cube.with_(tau0=1.0e3, vmax_kms=30.0), "thick moving": cube.with_(vmax_kms=30.0)}.get(path, cube)
+    n, first = 3000, 128
+    p = R.Problem(w, **kw)
+    prop, keep = None, []
+    if path == "proposal":  # one whole brick whose packets are never served (no eligible brick)
+        t = lambda *a, **k: keep.append(torch.tensor(*a, device="cuda", **k)) or keep[-1].data_ptr()  # noqa: E731
+        prop = R.Proposal()
+        prop.brick, prop.margin, prop.n_bricks = 8, 1, 1
+        prop.d_brick_lk, prop.d_lp, prop.d_xc = t([-1e30]), t([0.0] * 16), t([0.0] * 16)
+        prop.d_queue_count, prop.d_queue_pid = t([0], dtype=torch.int64), t([0] * n, dtype=torch.int64)
+    p.reset()
+    p.launch(n, 5, steps_per_launch=first, proposal=prop)
+    a, s = p.read(), p.packet_states(n, 0, n)
+    flying = s["status"] == 1
+    assert flying.sum() > 100 and np.all(s["steps"][flying] == first)
+    p.launch(n, 5, steps_per_launch=first, resume=1, max_steps=limit, proposal=prop)
+    b = p.read()
+    assert b["aborted"] - a["aborted"] == flying.sum()
+    for k in ("emitted", "escaped", "steps", "mc_events", "event_draws", "absorbed"):
+        assert a[k] == b[k], k
+    assert np.all(p.packet_states(n, 0, n)["status"] == 2)
+    p.close()

@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                     TransitionStream ts;
                     ts.init((uint32_t)blk - left, bh, pl, ph, P);
                     uint4 ra = ts.next(P), rb;
-                    uint32_t o = 16u * s;
+                    uint32_t o = pair_offset(s, nr1);
                     // one group of four on r while the next block is drawn into rn;
                     // true when the packet finished
                     auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
@@ -682,7 +682,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                         }
                         s = o >> 4;
                         if (walk_four_rows<NDIM>(P, nr1, J, r, s, cell, cls)) {
-                            o = 16u * s;
+                            o = min(16u * s, omax);
                             return false;
                         }
                         if (m.ok2) s = (m.o2 - 32u) >> 4;

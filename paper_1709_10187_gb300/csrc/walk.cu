@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                             // a thin source state starts as MC
                             const uint4 a0 = __ldg(&rows[min(s, nr1) * RW]);
                             if (a0.w & FLAG_THIN) {
-                                if (after_mc(excursion(min(bin, J - 1u), -1))) release();
+                                if (after_mc(excursion(min(bin, J - 1u), -1))) done_with();
                             }
                         }
                     }

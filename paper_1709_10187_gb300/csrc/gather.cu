@@ -89,8 +89,7 @@ template <int RB, bool SMEM>
 cudaError_t launch_chase(const void* table, uint32_t mask, uint32_t chain, int ctas_per_sm, int threads,
                          uint32_t seed, unsigned long long* sink, cudaStream_t s, uint64_t* n_threads) {
     const size_t smem = SMEM ? (size_t)(mask + 1u) * RB : 0;
-    cudaError_t e = cudaFuncSetAttribute(gather_chase_kernel<RB, SMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(gather_chase_kernel<RB, SMEM>, SMEM ? kSmemMost : 0);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, fit = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -123,7 +122,7 @@ extern "C" int rddmc_gather_probe(void* d_table, uint64_t table_bytes, int row_b
     const uint64_t rows = table_bytes / (uint64_t)row_bytes;
     if (rows < 64 || rows > (1ull << 32) || (rows & (rows - 1)) || rows * (uint64_t)row_bytes != table_bytes)
         return RDDMC_ERR_ARG;
-    if (in_smem && table_bytes > 200u * 1024u) return RDDMC_ERR_SIZE;
+    if (in_smem && table_bytes > kSmemMost) return RDDMC_ERR_SIZE;
     const uint32_t mask = (uint32_t)(rows - 1ull);
     cudaStream_t s = (cudaStream_t)stream;
     if (fill) {

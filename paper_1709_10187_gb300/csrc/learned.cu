@@ -401,8 +401,7 @@ cudaError_t softmax_ce_rows(const float* logits, int n_out, int nA, int nB, int 
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(softmax_ce_rows_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
+        (e = allow_smem(softmax_ce_rows_kernel<V>, kSmemMost)) != cudaSuccess)
         return e;
     softmax_ce_rows_kernel<V><<<std::min((Bsz + warps - 1) / warps, nsm), warps * 32, smem, s>>>(
         logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb, db, loss);
@@ -421,14 +420,13 @@ cudaError_t softmax_ce(const float* logits, int n_out, int nA, int nB, int nC, i
     // at most 64 KiB of column sums a block (three blocks per SM), 8 warps while they fit
     const size_t row = (size_t)n_out * sizeof(float);
     const int warps = (int)std::max<size_t>(1, std::min<size_t>(8, (64u * 1024u) / row));
-    if (row > 200u * 1024u) {
+    if (row > kSmemMost) {
         softmax_ce_kernel<false><<<(Bsz + 7) / 8, 256, 0, s>>>(logits, n_out, nA, nB, nC, S, tA, tB, tC, Bsz, dlogb,
                                                               db, loss);
         return cudaGetLastError();
     }
     const size_t smem = row * warps;
-    cudaError_t e = cudaFuncSetAttribute(softmax_ce_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(softmax_ce_kernel<true>, kSmemMost);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
@@ -526,7 +524,7 @@ cudaError_t gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const 
     const int kpanels = (K + umma::kPanel - 1) / umma::kPanel;
     const int per_split = (kpanels + ksplit - 1) / ksplit;
     int nstage = staged ? 2 : std::min(per_split, ksplit > 1 ? 3 : umma::kMaxStages);
-    while (nstage > 2 && umma::smem_bytes(NT, nstage, MNB) > 200u * 1024u) --nstage;
+    while (nstage > 2 && umma::smem_bytes(NT, nstage, MNB) > kSmemMost) --nstage;
     // at least 80 KiB of shared memory: at most two CTAs per SM, so their TMEM
     // accumulators (<= 256 columns each) always fit the SM's 512 columns
     const size_t smem = std::max<size_t>(umma::smem_bytes(NT, nstage, MNB), 80 * 1024);
@@ -542,7 +540,7 @@ cudaError_t gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const 
     auto kern = umma::gemm_tc_kernel<EPI, true, MNA, MNB>;
     if constexpr (!MNA && !MNB)
         if (staged) kern = umma::gemm_tc_kernel<EPI, false, false, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kSmemMost);
     if (e != cudaSuccess) return e;
     kern<<<grid, umma::kThreads, smem, s>>>(M, N, K, NT, A, lda, W, ldw, mapA, mapW, bias, mask, ldmask, outb, outf,
                                             ldc, colsum, nstage, err);

@@ -132,6 +132,17 @@ __device__ __forceinline__ uint32_t event_word(uint64_t p, uint64_t n, uint32_t 
     return l == 0 ? r.x : (l == 1 ? r.y : (l == 2 ? r.z : r.w));
 }
 
+// Lets a kernel's blocks take up to `most` bytes of dynamic shared memory.  The
+// limit belongs to the kernel, which every host thread and stream shares, so each
+// launch sets the same: set to a call's own size, a smaller call could lower it
+// between another thread's set and its launch, which is then refused.
+constexpr size_t kSmemBlock = 227 * 1024;  // what a block of a kernel without static shared memory may take (sm_103a)
+constexpr size_t kSmemMost = 200 * 1024;   // the largest that the kernels with some ask for
+template <class... A>
+inline cudaError_t allow_smem(void (*kernel)(A...), size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 __host__ __device__ __forceinline__ uint64_t align256(uint64_t v) { return (v + 255ull) & ~255ull; }
 
 }  // namespace rddmc

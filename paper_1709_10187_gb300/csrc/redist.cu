@@ -232,12 +232,11 @@ extern "C" int rddmc_precompute_redistribution(const rddmc_grid* g, const void* 
     if (n_sub < 1 || n_sub > kMaxSub || g->J < 2) return RDDMC_ERR_ARG;
     if (bytes < (size_t)g->J * (size_t)(g->J - 1) * 4u) return RDDMC_ERR_SIZE;
     if (!g->precomputed) return RDDMC_ERR_TABLE;  // the bin edges are read from the table
-    if ((size_t)n_sub * (size_t)(g->J - 1) * 8u > 200u * 1024u) return RDDMC_ERR_UNSUPPORTED;
+    if ((size_t)n_sub * (size_t)(g->J - 1) * 8u > kSmemMost) return RDDMC_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     const double* edges = (const double*)((const char*)d_table + g->off_edges);
     const size_t smem = (size_t)(g->J - 1) * 8u;  // a block's node
-    if (cudaFuncSetAttribute(redist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return RDDMC_ERR_CUDA;
+    if (allow_smem(redist_kernel, kSmemMost) != cudaSuccess) return RDDMC_ERR_CUDA;
     cudaLaunchAttribute cluster;
     cluster.id = cudaLaunchAttributeClusterDimension;
     cluster.val.clusterDim.x = (unsigned)n_sub;

@@ -456,7 +456,7 @@ template <int NDIM, bool SMEM_TALLY, int MINB, bool LEAK, bool WEIGHT>
 cudaError_t launch_time_minb(WalkParams& P, const TimeParams& T, int threads, size_t smem, int ctas, int nsm,
                              cudaStream_t s) {
     const auto kernel = time_kernel<NDIM, SMEM_TALLY, MINB, LEAK, WEIGHT>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, kSmemBlock);
     if (e != cudaSuccess) return e;
     const bool chosen = !threads && !ctas;
     if (!threads) threads = 256;

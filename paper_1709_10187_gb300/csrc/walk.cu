@@ -873,7 +873,7 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
     const int threads = L.threads ? L.threads : (few ? 128 : 256);
     const size_t smem = L.smem + (size_t)threads * L.smem_per_thread;
     int ctas = L.ctas_per_sm;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, kSmemBlock);
     if (e != cudaSuccess) return e;
     if (!ctas &&
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem)) != cudaSuccess)

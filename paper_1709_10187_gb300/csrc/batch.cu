@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                 auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
                     unsigned q = 0;
                     if (pair) {
-                        const uint32_t o = pair_offset(s, nr1);
+                        const uint32_t o = pair_offset(s, 16u * nr1);
                         const FourMoves m = walk_four(pair, r, o);
                         rn = ts.next(P);
                         if (m.ok4) {

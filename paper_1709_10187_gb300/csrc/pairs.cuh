@@ -36,11 +36,8 @@ struct alignas(16) Pair {
 constexpr int kPairPad = 32;
 
 // Offset of the pair of state s.  A saved state that names a cell in vacuum has
-// the class 0xffffffff and an s far past the table: it reads the last row, nr1, as
-// it does on the rows.  (The walk's loop keeps min(16 s, 16 nr1) after its row
-// groups, bounded as well and a register less: with the clamps two 4096-step slices
-// of 4e6 packets on the 256 x 512 slab take 26.1 ms, without 25.9.)
-__host__ __device__ __forceinline__ uint32_t pair_offset(uint32_t s, uint32_t nr1) { return 16u * (s < nr1 ? s : nr1); }
+// the class 0xffffffff and an s far past the table: it gets at most `last`, the last row's.
+__host__ __device__ __forceinline__ uint32_t pair_offset(uint32_t s, uint32_t last) { return min(16u * s, last); }
 
 __host__ __device__ __forceinline__ Pair load_pair(const Pair* base, uint32_t offset, int shift) {
     const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(base) + offset + shift);
@@ -81,7 +78,11 @@ __host__ __device__ __forceinline__ FourMoves walk_four(const Pair* base, const 
 // move leaves the row as it is, so a transition is one row's thresholds against
 // its word, and the rows' flags say that every outcome is a plain move
 // (FLAG_FASTX, FLAG_FASTZ); nearer the class's edge the outcome's own action is
-// looked at and the class follows the cell.  Moves s, cell and cls and returns
+// looked at and the class follows the cell.  s is a row of the table, and inside a
+// class it moves by one row at a time: rows up to three beyond the ends are read
+// there without a clamp, and they lie in the table buffer's neighbouring blocks of
+// 256 bytes or more (the profile before the rows, the heads after them).  The
+// clamps cost 2 % of the wide-core slab.  Moves s, cell and cls and returns
 // true; returns false with all as they were when a transition is not a plain
 // move, and on moving grids, which the caller walks outcome by outcome.
 // Such groups took 520 of 650 cycles per warp on the wide-core slab when every
@@ -94,8 +95,8 @@ __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const unsigned w = q == 0 ? r.x : (q == 1 ? r.y : (q == 2 ? r.z : r.w));
-        const unsigned row = min(s1, nr1);
-        const uint4 a = __ldg(&P.rows[NDIM == 1 ? row : 2u * row]);
+        const int row = INSIDE ? (int)s1 : (int)min(s1, nr1);
+        const uint4 a = __ldg(&P.rows[NDIM == 1 ? row : 2 * row]);
         const bool spatial = w >= a.y;  // thresholds of j-1 | j+1 | -x | +x ...
         unsigned move, outcome;
         if (NDIM == 1) {
@@ -103,7 +104,7 @@ __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, 
             move = up ? 1u : 0xffffffffu;
             outcome = (spatial ? 2u : 0u) + (up ? 1u : 0u);
         } else {
-            const uint4 b = __ldg(&P.rows[2u * row + 1u]);  // ... | -y | +y | -z | +z
+            const uint4 b = __ldg(&P.rows[2 * row + 1]);  // ... | -y | +y | -z | +z
             const bool y = w >= b.x, z = w >= b.z;
             const bool up = w >= (spatial ? (z ? b.w : (y ? b.y : a.z)) : a.x);
             const unsigned stride = !spatial ? 1u : (z ? (unsigned)P.n01 : (y ? (unsigned)P.n0 : 1u));

@@ -602,7 +602,10 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                         cell = min(cell, (unsigned)P.ncell - 1u);
                         cls = __ldg(&P.cell_class[cell]);
                         s = cls * J + min(bin, J - 1u);
-                        t_stop = P.slice ? t + P.slice : ~0ull;
+                        // the slice's end or the watchdog's limit, not before t: a packet
+                        // resumed past a limit lower than the last launch's takes no transition
+                        t_stop = P.slice && P.slice < P.max_steps ? min(t + P.slice, P.max_steps) : P.max_steps;
+                        t_stop = max(t_stop, t);
                         if (HYBRID && st == PK_FRESH) {
                             // a thin source state starts as MC
                             const uint4 a0 = __ldg(&rows[min(s, nr1) * RW]);
@@ -651,8 +654,6 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
         // checkpoints do not depend on slicing)
         unsigned long long lim = PROPOSE ? (t / (unsigned long long)P.chunk + 1ull) * (unsigned long long)P.chunk : ~0ull;
         lim = lim < t_stop ? lim : t_stop;
-        lim = lim < P.max_steps ? lim : P.max_steps;
-        lim = lim > t ? lim : t;  // resumed past a limit lower than the last launch's: no transition
         const uint32_t pl = (uint32_t)pid, ph = (uint32_t)(pid >> 32);
         if (have) {
             const unsigned long long lim0 = lim;
@@ -670,7 +671,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                     TransitionStream ts;
                     ts.init((uint32_t)blk - left, bh, pl, ph, P);
                     uint4 ra = ts.next(P), rb;
-                    uint32_t o = pair_offset(s, nr1);
+                    uint32_t o = pair_offset(s, omax);
                     // one group of four on r while the next block is drawn into rn;
                     // true when the packet finished
                     auto group = [&](const uint4& r, uint4& rn, unsigned behind) -> bool {
@@ -682,12 +683,12 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                         }
                         s = o >> 4;
                         if (walk_four_rows<NDIM>(P, nr1, J, r, s, cell, cls)) {
-                            o = min(16u * s, omax);
+                            o = pair_offset(s, omax);
                             return false;
                         }
                         if (m.ok2) s = (m.o2 - 32u) >> 4;
                         const unsigned q = by_rows(r, m.ok2 ? 2u : 0u);
-                        o = min(16u * s, omax);
+                        o = pair_offset(s, omax);
                         t = 4ull * (blk - behind) + q + 1ull;
                         return q < 4u;
                     };

@@ -31,7 +31,7 @@ int main() {
         for (int i = 0; i < 200; ++i) states.push_back(rnd());
         for (uint32_t s : states)
             for (int k = 0; k < 50; ++k) {
-                const uint32_t o = pair_offset(s, n - 1u);
+                const uint32_t o = pair_offset(s, 16u * (n - 1u));
                 if (o % 16u || o > 16u * (n - 1u) || (s < n && o != 16u * s)) return 1;
                 uint4 r = make_uint4(rnd(), rnd(), rnd(), rnd());
                 if (k & 1) r = make_uint4(0u, 0u, 0u, 0u);           // always down

@@ -876,9 +876,13 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
     int ctas = L.ctas_per_sm;
     cudaError_t e = allow_smem(kernel, kSmemBlock);
     if (e != cudaSuccess) return e;
-    if (!ctas &&
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem)) != cudaSuccess)
-        return e;
+    if (!ctas || P.time_slice_ns) {
+        int fit = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, threads, smem)) != cudaSuccess) return e;
+        // more CTAs than are resident would begin wall-time slices of their own
+        // when the first have ended theirs
+        ctas = ctas ? std::min(ctas, fit) : fit;
+    }
     if (ctas < 1) ctas = 1;
     if (few) {
         const Spread f = spread(P.n_packets, ctas, L.sms);

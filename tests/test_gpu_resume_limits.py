@@ -1,5 +1,6 @@
-"""Watchdog limits that change between the launches of a run: a packet resumed
-past the limit is aborted before it takes another transition."""
+"""Limits of the launches of a run.  Watchdog limits that change between them: a
+packet resumed past the limit is aborted before it takes another transition.
+Wall-time slices end on time whatever number of CTAs is asked for."""
 import numpy as np
 import pytest
 
@@ -103,4 +104,22 @@ def test_walk_with_a_lower_limit_aborts_at_once(path, limit):
     for k in ("emitted", "escaped", "steps", "mc_events", "event_draws", "absorbed"):
         assert a[k] == b[k], k
     assert np.all(p.packet_states(n, 0, n)["status"] == 2)
+    p.close()
+
+
+@pytest.mark.parametrize("ctas,threads", [(0, 0), (4, 256), (12, 256), (24, 128)])
+def test_wall_time_slices_are_not_repeated_by_waiting_ctas(ctas, threads):
+    p, n, ms = R.Problem(W.C1), 500_000, 20.0
+    p.reset()
+    p.launch(n, 5, steps_per_launch=64)
+    took = []
+    for _ in range(3):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        p.launch(n, 5, resume=1, time_slice_us=int(1e3 * ms), ctas_per_sm=ctas, threads_per_cta=threads)
+        b.record()
+        torch.cuda.synchronize()
+        took.append(a.elapsed_time(b))
+    assert ms <= min(took) < 1.6 * ms, took
+    assert (p.packet_states(n, 0, n)["status"] == 1).sum() > n // 2
     p.close()

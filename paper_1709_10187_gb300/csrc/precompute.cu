@@ -2,10 +2,11 @@
 //
 // Kernel 1: phi[j] = bin mean of H(a,x) over bin j (k_ij = k0_i phi_j).  Half a
 // warp sums one edge's Dawson series, a lane per term, in the series' order.
-// Kernel 2, a thread per (class, bin) row; on a moving grid a block per class
-// and 127 of its rows, each thread first taking one bin edge, shifted by every
-// face's velocity difference in turn (faces with the same shift once), then its
-// row: leakage coefficients of
+// Kernel 2, a thread per (class, bin) row; on a moving grid a block takes 127
+// rows of a class, or as many whole classes of fewer bins as it has threads for
+// their edges, each thread first taking one bin edge, shifted by every face's
+// velocity difference in turn (faces with the same shift once), then its row:
+// leakage coefficients of
 //   eq. x-leakage and eq. z-leakage, the boundary / thin-neighbour form
 //   2/(3 dz (k dz + 2 lambda)), probabilities p_X = k_X / sum k accumulated in
 //   outcome order, 32-bit thresholds round-half-even(C 2^32) saturated at
@@ -62,21 +63,39 @@ __device__ __forceinline__ uint32_t quantise_dev(double C) {
 // Bound by FP64 issue where cells move: the neighbour's opacity over the shifted
 // bin takes one Dawson series (32 exponentials and divisions) per edge and
 // distinct shift.  16^3 cells x 64 bins, every cell its own shifts: 4.7 ms (12.8 ms
-// with two series of 34 terms per row and face).
+// with two series of 34 terms per row and face).  Classes of few bins share a
+// block: 64^3 cells x 1 and x 8 bins 23 and 50 ms, 136 and 142 ms with a block each
+// (29 and 129 ms with a thread per row).
 template <int NDIM, bool MOVING>
 __global__ void __launch_bounds__(kRowEdges)
     rows_kernel(const TableHeader h, const ClassDesc* __restrict__ cdesc, const double* __restrict__ edges,
                 const double* __restrict__ phi, uint32_t* __restrict__ rows, uint2* __restrict__ fast,
                 float* __restrict__ tau_row, float* __restrict__ rk, uint32_t* __restrict__ abs_thr, int dusty,
-                unsigned long long* __restrict__ wq, float* __restrict__ ka_row, int weighted, int tiles, int64_t nrow) {
+                unsigned long long* __restrict__ wq, float* __restrict__ ka_row, int weighted, int tiles,
+                int per_block, int64_t nrow) {
     constexpr int K = 2 + 2 * NDIM;
     constexpr int W = NDIM == 1 ? 4 : 8;  // words per row, the last holding the flags
     __shared__ VoigtEdge s_edge[MOVING ? kRowEdges : 1];
     const int J = h.J, tid = (int)threadIdx.x;
     const int64_t lin = (int64_t)blockIdx.x * kRowEdges + tid;
-    const int cls = MOVING ? (int)(blockIdx.x / (unsigned)tiles) : (int)(min(lin, nrow - 1) / J);
-    const int j = MOVING ? (int)(blockIdx.x % (unsigned)tiles) * (kRowEdges - 1) + tid
-                         : (int)(lin - (int64_t)cls * J);
+    // static: rows in a line; moving: `per_block` classes, or a tile of one
+    int cls, j;
+    bool edge = true, row = lin < nrow;  // this thread has an edge, a row
+    if (!MOVING) {
+        cls = (int)(min(lin, nrow - 1) / J);
+        j = (int)(lin - (int64_t)cls * J);
+    } else if (per_block > 1) {
+        const int64_t c = (int64_t)blockIdx.x * per_block + tid / (J + 1), last = nrow / J - 1;
+        cls = (int)min(c, last);
+        j = tid % (J + 1);
+        edge = tid < per_block * (J + 1) && c <= last;
+        row = edge && j < J;
+    } else {
+        cls = (int)(blockIdx.x / (unsigned)tiles);
+        j = (int)(blockIdx.x % (unsigned)tiles) * (kRowEdges - 1) + tid;
+        edge = j <= J;
+        row = tid < kRowEdges - 1 && j < J;
+    }
     const ClassDesc& D = cdesc[cls];
     // bin-mean profile over the bin shifted by each face's velocity difference
     double phi_nb[2 * NDIM];
@@ -85,29 +104,24 @@ __global__ void __launch_bounds__(kRowEdges)
         for (int f = 0; f < 2 * NDIM; ++f) {
             const double delta = D.face[f].delta;
             phi_nb[f] = 0.0;
-            if (D.face[f].exterior || delta == 0.0) continue;  // one class per block: uniform
             int same = -1;
 #pragma unroll
             for (int g = 0; g < f; ++g)
                 if (same < 0 && !D.face[g].exterior && D.face[g].delta == delta) same = g;
-            if (same >= 0) {
 #pragma unroll
-                for (int g = 0; g < f; ++g)
-                    if (g == same) phi_nb[f] = phi_nb[g];
-                continue;
-            }
-            __syncthreads();  // the last face's readers
-            if (j <= J) {
+            for (int g = 0; g < f; ++g)
+                if (g == same) phi_nb[f] = phi_nb[g];
+            const bool shifted = !D.face[f].exterior && delta != 0.0 && same < 0;  // the same in all of a class
+            if (!__syncthreads_or(shifted)) continue;  // also: the last face's readers are done
+            if (shifted && edge) {
                 const double x = edges[j] + delta;
                 s_edge[tid] = voigt_edge(x, dawson_f64(x));
             }
             __syncthreads();
-            if (tid < kRowEdges - 1 && j < J) phi_nb[f] = voigt_bin_mean_f64(h.a, s_edge[tid], s_edge[tid + 1]);
+            if (shifted && row) phi_nb[f] = voigt_bin_mean_f64(h.a, s_edge[tid], s_edge[tid + 1]);
         }
-        if (tid == kRowEdges - 1 || j >= J) return;
-    } else if (lin >= nrow) {
-        return;
     }
+    if (!row) return;
     const int64_t r = (int64_t)cls * J + j;
     const bool hybrid = h.mode == RDDMC_MODE_HYBRID;
     double dzmin = h.dz[0];
@@ -285,7 +299,10 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     for (int a = 0; a < 3; ++a) h.dz[a] = 2.0 * g.R / g.n[a];
     const int64_t nrow = (int64_t)g.n_class * g.J;
     const int tiles = (g.J + kRowEdges - 2) / (kRowEdges - 1);
-    const int64_t blocks = g.moving ? (int64_t)g.n_class * tiles : (nrow + kRowEdges - 1) / kRowEdges;
+    const int per_block = kRowEdges / (g.J + 1);  // whole classes of a block's edges
+    const int64_t blocks = !g.moving ? (nrow + kRowEdges - 1) / kRowEdges
+                           : per_block > 1 ? (g.n_class + per_block - 1) / per_block
+                                           : (int64_t)g.n_class * tiles;
     const ClassDesc* cd = (const ClassDesc*)(base + g.off_cdesc);
     uint32_t* rows = (uint32_t*)(base + g.off_rows);
     uint2* fast = (uint2*)(base + g.off_fast);
@@ -299,7 +316,7 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
     auto rows_k = g.ndim == 1 ? (g.moving ? rows_kernel<1, true> : rows_kernel<1, false>)
                               : (g.moving ? rows_kernel<3, true> : rows_kernel<3, false>);
     rows_k<<<(unsigned)blocks, kRowEdges, 0, s>>>(h, cd, edges, phi, rows, fast, tau_row, rk, abs_thr, dusty, wq,
-                                                  ka_row, weighted, tiles, nrow);
+                                                  ka_row, weighted, tiles, per_block, nrow);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.pairs()) {
         pair_kernel<<<(unsigned)((nrow + 255) / 256), 256, 0, s>>>(fast, (Pair*)(base + g.off_pair), g.J, nrow);

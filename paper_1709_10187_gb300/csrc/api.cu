@@ -25,32 +25,6 @@ uint32_t quantise(double C) {
     return (uint32_t)t;
 }
 
-// Per cell, the number of spatial moves after which a packet is certainly still
-// in a cell of the same class: the cells' distance (moves along the axes) to the
-// nearest cell with a neighbour of another class, in vacuum or outside the grid,
-// at most 254.  One pass along the cells and one back give these distances.
-std::vector<uint8_t> class_margins(const rddmc_grid& g) {
-    std::vector<uint8_t> m((size_t)g.ncell, 254);
-    const int64_t stride[3] = {1, g.n[0], (int64_t)g.n[0] * g.n[1]};
-    auto nearer = [&](int64_t c, int64_t n) { m[c] = m[n] + 1 < m[c] ? (uint8_t)(m[n] + 1) : m[c]; };
-    int idx[3] = {0, 0, 0};
-    for (int64_t c = 0; c < g.ncell; ++c) {
-        for (int ax = 0; ax < g.ndim; ++ax) {
-            if (idx[ax] == 0 || idx[ax] + 1 == g.n[ax]) m[c] = 0;
-            if (idx[ax] + 1 < g.n[ax] && g.cell_class[c + stride[ax]] != g.cell_class[c]) m[c] = m[c + stride[ax]] = 0;
-        }
-        for (int ax = 0; ax < g.ndim; ++ax)
-            if (idx[ax] > 0) nearer(c, c - stride[ax]);
-        for (int ax = 0; ax < 3 && ++idx[ax] == g.n[ax]; ++ax) idx[ax] = 0;
-    }
-    for (int64_t c = g.ncell - 1; c >= 0; --c) {
-        for (int ax = 0; ax < 3 && --idx[ax] < 0; ++ax) idx[ax] = g.n[ax] - 1;
-        for (int ax = 0; ax < g.ndim; ++ax)
-            if (idx[ax] + 1 < g.n[ax]) nearer(c, c + stride[ax]);
-    }
-    return m;
-}
-
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? RDDMC_OK : RDDMC_ERR_CUDA; }
 
 }  // namespace
@@ -225,8 +199,6 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     g->n_class = (int)g->class_rep.size();
     if ((uint64_t)g->n_class * (uint64_t)J > (1ull << 40)) { delete g; return RDDMC_ERR_UNSUPPORTED; }
 
-    if (g->pairs() && !g->moving) g->margin = class_margins(*g);
-
     // Table layout.
     uint64_t off = align256(sizeof(TableHeader));
     g->off_class = off; off += align256((uint64_t)ncell * 4);
@@ -243,7 +215,7 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     g->off_abs = off; off += align256((uint64_t)g->n_class * J * 4);
     g->off_wq = off; off += align256((uint64_t)g->n_class * J * 8);
     g->off_ka = off; off += align256((uint64_t)g->n_class * J * 4);
-    g->off_margin = off; off += align256(g->margin.size());
+    g->off_inside = off; off += g->inside() ? align256((uint64_t)ncell) : 0;
     g->off_pair = off + 256; off += g->pairs() ? 256 + align256((uint64_t)g->n_class * J * 16 + kPairPad) : 0;
     g->table_bytes = off;
     *out = g;
@@ -344,9 +316,6 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
         return cuda_status(e);
     if ((e = cudaMemcpyAsync(base + g->off_rebin, rb.data(), rb.size() * sizeof(Rebin), cudaMemcpyHostToDevice, s)) !=
         cudaSuccess)
-        return cuda_status(e);
-    if (!g->margin.empty() && (e = cudaMemcpyAsync(base + g->off_margin, g->margin.data(), g->margin.size(),
-                                                   cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return cuda_status(e);
     if (g->moving && (e = cudaMemcpyAsync(base + g->off_vel, g->v.data(), g->v.size() * 8, cudaMemcpyHostToDevice,
                                           s)) != cudaSuccess)

@@ -35,7 +35,7 @@ struct InstDesc {
     const uint4* rows;
     const uint2* fast;
     const Pair* pair;               // null for a large table
-    const uint8_t* margin;          // with pair
+    const uint8_t* inside;          // with pair, static grids
     const uint32_t* cell_class;
     const Rebin* rebin;
     const double* edges;
@@ -94,7 +94,7 @@ struct LaneInst {
     const uint4* rows;
     const uint2* fast;
     const uint32_t* cell_class;
-    const uint8_t* margin;
+    const uint8_t* inside;
     unsigned J, ncls1, n0, n01, ndim;
     int ncell;
     static constexpr bool kDust = false;  // instances have none
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                         pair = D.pair;
                         nr1 = (unsigned)D.n_rows - 1u;
                         L.rows = D.rows; L.fast = D.fast; L.cell_class = D.cell_class;
-                        L.margin = D.margin; L.J = (unsigned)D.J; L.ncell = D.ncell; L.ncls1 = (unsigned)D.n_class - 1u;
+                        L.inside = D.inside; L.J = (unsigned)D.J; L.ncell = D.ncell; L.ncls1 = (unsigned)D.n_class - 1u;
                         L.n0 = (unsigned)D.n0; L.n01 = (unsigned)D.n01; L.ndim = (unsigned)D.ndim;
                     }
                     gid = D.pkt_begin + (q - P.off[inst]);
@@ -431,7 +431,7 @@ int rddmc_batch_create(const rddmc_grid* const* grids, const void* const* d_tabl
         D.rows = (const uint4*)(tb + g->off_rows);
         D.fast = (const uint2*)(tb + g->off_fast);
         D.pair = g->pairs() ? (const Pair*)(tb + g->off_pair) : nullptr;
-        D.margin = !g->margin.empty() ? (const uint8_t*)(tb + g->off_margin) : nullptr;
+        D.inside = g->inside() ? (const uint8_t*)(tb + g->off_inside) : nullptr;
         D.cell_class = (const uint32_t*)(tb + g->off_class);
         D.rebin = (const Rebin*)(tb + g->off_rebin);
         D.edges = (const double*)(tb + g->off_edges);

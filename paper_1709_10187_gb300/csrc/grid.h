@@ -41,7 +41,6 @@ struct rddmc_grid {
     std::vector<double> edges;
     std::vector<uint32_t> cell_class;   // UINT32_MAX for vacuum cells
     std::vector<int64_t> class_rep;     // a representative cell per class
-    std::vector<uint8_t> margin;        // per cell: spatial moves that stay in its class (pairs and a static grid; else empty)
     std::vector<double> n_rel;          // per cell (copied)
     std::vector<double> v;              // per cell x3, km/s (empty if static)
     double vth = 12.85;                 // thermal velocity, km/s
@@ -54,7 +53,7 @@ struct rddmc_grid {
     // table layout (byte offsets)
     uint64_t off_class = 0, off_cdesc = 0, off_rebin = 0, off_vel = 0, off_edges = 0, off_phi = 0,
              off_rows = 0, off_fast = 0, off_tau = 0, off_upar = 0, off_rk = 0, off_abs = 0, off_wq = 0, off_ka = 0, off_pair = 0,
-             off_margin = 0, table_bytes = 0;
+             off_inside = 0, table_bytes = 0;
     // leakage parameters of the last precompute
     rddmc_leak_params params{};
     double tau_cell = 0.0;  // largest line-centre optical depth of a cell (last precompute)
@@ -65,6 +64,8 @@ struct rddmc_grid {
 
     // the table holds the walk's pairs (pairs.cuh)
     bool pairs() const { return (int64_t)n_class * J <= rddmc::kPairRows; }
+    // and which cells lie four moves inside their class (walk_rows)
+    bool inside() const { return pairs() && !moving; }
 
     bool in_medium(const int idx[3]) const;
     int64_t cell_of(const int idx[3]) const { return idx[0] + (int64_t)n[0] * (idx[1] + (int64_t)n[1] * idx[2]); }

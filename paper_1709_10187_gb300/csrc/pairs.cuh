@@ -74,7 +74,7 @@ __host__ __device__ __forceinline__ FourMoves walk_four(const Pair* base, const 
 }
 
 // Four transitions of any plain moves on the rows, without a branch on their
-// outcomes.  In a cell at least four moves inside its class (margin) a spatial
+// outcomes.  In a cell at least four moves inside its class (P.inside) a spatial
 // move leaves the row as it is, so a transition is one row's thresholds against
 // its word, and the rows' flags say that every outcome is a plain move
 // (FLAG_FASTX, FLAG_FASTZ); nearer the class's edge the outcome's own action is
@@ -136,10 +136,10 @@ __device__ __forceinline__ bool walk_rows(const K& P, unsigned nr1, unsigned J, 
 template <int NDIM, class K>
 __device__ __forceinline__ bool walk_four_rows(const K& P, unsigned nr1, unsigned J, const uint4& r, unsigned& s,
                                                unsigned& cell, unsigned& cls) {
-    if (!P.margin) return false;
+    if (!P.inside) return false;
     if constexpr (K::kDust)
         if (P.dust) return walk_rows<NDIM, false, true>(P, nr1, J, r, s, cell, cls);
-    return __ldg(&P.margin[cell]) >= 4u ? walk_rows<NDIM, true, false>(P, nr1, J, r, s, cell, cls)
+    return __ldg(&P.inside[cell]) ? walk_rows<NDIM, true, false>(P, nr1, J, r, s, cell, cls)
                                         : walk_rows<NDIM, false, false>(P, nr1, J, r, s, cell, cls);
 }
 

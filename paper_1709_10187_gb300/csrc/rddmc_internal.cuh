@@ -6,8 +6,7 @@
 //    | fast heads uint2[n_class*J] | tau f32[n_class*J] | u_par split points f32x2[kUparN]
 //    | 1/K_s f32[n_class*J] | dust absorption thresholds u32[n_class*J] | dust weights u64[n_class*J]
 //    | dust opacities f32[n_class*J] | pairs 16 B[n_class*J] with pads (tables up to kPairRows rows)
-//    | margins u8[ncell] (with the pairs, static grids): spatial moves a packet can make from a cell and stay in its class,
-//    at most 254]
+//    | inside u8[ncell] (with the pairs, static grids): whether four spatial moves from a cell stay in its class]
 // With dust absorption (Sec. 2.6) the categorical draw has one more outcome,
 // absorption, after the leakage outcomes: the row thresholds are cumulative over
 // the leakage rates plus k_a, and the absorption threshold (where absorption

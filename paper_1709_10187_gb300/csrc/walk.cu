@@ -1373,7 +1373,7 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.rows = (const uint4*)(tb + g.off_rows);
     P.fast = (const uint2*)(tb + g.off_fast);
     P.pair = g.pairs() ? (const Pair*)(tb + g.off_pair) : nullptr;
-    P.margin = g.margin.empty() ? nullptr : (const uint8_t*)(tb + g.off_margin);
+    P.inside = g.inside() ? (const uint8_t*)(tb + g.off_inside) : nullptr;
     P.tau_row = (const float*)(tb + g.off_tau);
     P.upar = (const float2*)(tb + g.off_upar);
     P.cdesc = (const ClassDesc*)(tb + g.off_cdesc);

@@ -17,7 +17,7 @@ struct WalkParams {
     const uint4* rows;
     const uint2* fast;
     const Pair* pair;         // two frequency moves per gather (null for large tables)
-    const uint8_t* margin;    // per cell: spatial moves that stay in the cell's class (with the pairs)
+    const uint8_t* inside;    // per cell: whether four spatial moves stay in its class (with the pairs, static grids)
     const float* tau_row;     // tau_ij = k_ij dz per row (hybrid conversions)
     const float2* upar;       // u_par envelope split points
     const ClassDesc* cdesc;

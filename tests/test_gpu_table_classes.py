@@ -57,3 +57,20 @@ def test_tables_of_few_bins_take_less_time():
 
     small, large = ms(2), ms(62)
     assert small < 0.25 * large, (small, large)
+
+
+@pytest.mark.parametrize("n,J", [(10, 2), (10, 40), (12, 31), (18, 62), (22, 31)])
+def test_rows_do_not_depend_on_how_blocks_share_classes(n, J):
+    # every cell a class of its own: few classes go one to a block, more fill its
+    # threads
+    x = max(4.0, J / 2.0)
+    w = W.Workload(f"shared_{n}_{J}", 3, (n, n, n), J, -x, x, 1.0e5, 1.0e4, 1, 1, vmax_kms=60.0)
+    n_rel = W.clumpy_medium(n=n, J=J, brick=1).n_rel
+    ot = C.Grid(w, n_rel=n_rel).table()
+    p = R.Problem(w, n_rel=n_rel)
+    thr, flags = p.rows()
+    assert p.sizes.n_class == w.ncell
+    p.close()
+    assert np.array_equal(flags, ot["flags"])
+    d = thr.astype(np.int64) - ot["thr"].astype(np.int64)
+    assert np.abs(d).max() <= 1 and (d != 0).sum() <= max(2, 1e-4 * d.size)

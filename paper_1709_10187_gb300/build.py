@@ -31,7 +31,7 @@ def nvcc() -> str:
 
 
 def _flags():
-    # RDDMC_NVCC_EXTRA: extra nvcc options for tuning builds (e.g. -DRDDMC_WALK_MIN_BLOCKS=4)
+    # RDDMC_NVCC_EXTRA: extra nvcc options for tuning builds (e.g. -Xptxas -v)
     extra = os.environ.get("RDDMC_NVCC_EXTRA", "").split()
     return ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
                    "-I", os.path.join(ROOT, "include"), "-I", CSRC] + extra

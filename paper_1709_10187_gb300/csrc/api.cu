@@ -120,7 +120,15 @@ int rddmc_build_grid(const rddmc_grid_desc* d, rddmc_grid** out) {
     for (int j = 0; j < J; ++j)
         if (std::fabs((g->edges[j + 1] - g->edges[j]) - dx0) > 1e-9 * std::fabs(dx0)) g->uniform_bins = false;
     g->n_rel.resize(ncell);
-    for (int64_t c = 0; c < ncell; ++c) g->n_rel[c] = d->n_rel ? d->n_rel[c] : 1.0;
+    double sum_rel = 0.0;
+    int64_t n_med = 0;
+    for (int64_t c = 0; c < ncell; ++c) {
+        g->n_rel[c] = d->n_rel ? d->n_rel[c] : 1.0;
+        if (d->mask && !d->mask[c]) continue;
+        sum_rel += g->n_rel[c];
+        ++n_med;
+    }
+    g->mean_rel = n_med ? sum_rel / (double)n_med : 0.0;
     if (d->mask) g->mask.assign(d->mask, d->mask + ncell);
     g->vth = 12.85 * std::sqrt(d->T / 1.0e4);  // Sec. 2.1
     if (d->v_kms) {
@@ -257,7 +265,6 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
     std::vector<ClassDesc> cd(g->n_class);
     std::vector<Rebin> rb((size_t)g->n_class * g->nfaces);
     const double dx0 = g->edges[1] - g->edges[0];
-    g->tau_cell = 0.0;
     for (int k = 0; k < g->n_class; ++k) {
         const int64_t c = g->class_rep[k];
         int idx[3];
@@ -265,7 +272,6 @@ int rddmc_precompute_leakage(rddmc_grid* g, const rddmc_leak_params* p, void* d_
         ClassDesc& D = cd[k];
         std::memset(&D, 0, sizeof(D));
         D.k0 = g->tau0 / g->R * g->n_rel[c];
-        g->tau_cell = std::fmax(g->tau_cell, D.k0 * 2.0 * g->R / g->n[0]);
         D.ks = p->dust_scat / g->R * g->n_rel[c];
         D.ka = p->dust_abs / g->R * g->n_rel[c];
         D.moving = (!g->v.empty() && (g->v[3 * c] != 0.0 || g->v[3 * c + 1] != 0.0 || g->v[3 * c + 2] != 0.0)) ? 1 : 0;

@@ -56,11 +56,20 @@ struct rddmc_grid {
              off_inside = 0, table_bytes = 0;
     // leakage parameters of the last precompute
     rddmc_leak_params params{};
-    double tau_cell = 0.0;  // largest line-centre optical depth of a cell (last precompute)
+    double mean_rel = 0.0;  // mean of n_rel over the medium's cells
     bool precomputed = false;
     // dust absorption as an outcome of the draw, or by packet weights (Sec. 2.6)
     bool dusty() const { return params.dust_abs > 0.0 && params.dust_method == RDDMC_DUST_PROBABILISTIC; }
     bool weighted() const { return params.dust_abs > 0.0 && params.dust_method == RDDMC_DUST_WEIGHTS; }
+
+    // Mean line-centre optical depth of a cell, and what decides how often a packet
+    // moves in frequency rather than in space: that depth against the fourth power of
+    // the mean bin width.
+    double tau_cell() const { return tau0 * mean_rel * 2.0 / n[0]; }
+    double freq_share() const {
+        const double dx = (edges.back() - edges.front()) / J;
+        return tau_cell() / (dx * dx * dx * dx);
+    }
 
     // the table holds the walk's pairs (pairs.cuh)
     bool pairs() const { return (int64_t)n_class * J <= rddmc::kPairRows; }

@@ -38,10 +38,6 @@ constexpr int kHistOff = 22;
 constexpr int kNsb = 64;            // impact-parameter bins over b/R in [0, kSbMax)
 constexpr double kSbMax = 1.28;
 constexpr int64_t kPairRows = 1 << 20;  // tables up to this many rows carry the walk's pairs (pairs.cuh)
-// Line-centre optical depth of a cell below which a moving 3D walk reads
-// rows only, from which its frequency moves are worth reading in pairs, and those
-// of a hybrid slab.
-constexpr double kThinCell = 500.0, kThickCell = 1000.0, kThickHybrid = 4.0e4;
 constexpr int kUparN = 1024;        // |x| grid of the u_par envelope split points
 constexpr float kUparStep = 1.0f / 16.0f;
 

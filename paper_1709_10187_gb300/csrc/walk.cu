@@ -43,20 +43,6 @@ namespace {
 // weight method: -ln(1e-10) in 2^-40 units, the elimination weight of Sec. 2.6
 constexpr unsigned long long kLwMin = 25317190836906ull;
 
-// Resident 256-thread CTAs per SM the register budget targets.  Three (80
-// registers) keep the pair loop's two blocks of words and its stream constants
-// in registers; four (64) spill them: 27.7 against 28.2 ms on two 4096-step
-// slices of 4e6 packets (256 x 512 slab), 0.56 against 0.67 s on 1e5 packets of
-// the 64 x 128 slab to escape, 46 against 53 ms on the 32^3 clumpy medium.
-#ifndef RDDMC_WALK_MIN_BLOCKS
-#define RDDMC_WALK_MIN_BLOCKS 3
-#endif
-// The hybrid kernel's excursions need more: two (128 registers) 10.6 ms, three
-// 11.7 ms on two 4096-step slices of 5e5 packets, 256 x 512 hybrid slab.
-#ifndef RDDMC_WALK_HYBRID_MIN_BLOCKS
-#define RDDMC_WALK_HYBRID_MIN_BLOCKS 2
-#endif
-
 // ---------------------------------------------------------------- hybrid MC
 // Continuous MC of a packet in thin states (Sec. 5.1, Sec. 5.2), in FP32.  It
 // runs from a DDMC hand-off until the packet converts back to DDMC, escapes or
@@ -310,7 +296,7 @@ __device__ __forceinline__ bool prop_takes(const WalkParams& P, unsigned cell, u
 // Per-thread counters in shared memory.
 enum Loc64 { L_STEPS = 0, L_EDRAW = 1, L_MC = 2, kLoc64 = 3 };
 enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6,
-             L_EVENT_BLK = 6, L_EVENT = 7, kLoc32Events = 11 };  // the event words kept for rebins (3D)  // the block of event words kept for rebins
+             L_EVENT_BLK = 6, L_EVENT = 7, kLoc32Events = 11 };  // from L_EVENT_BLK: the event words kept for rebins (3D)
 
 // How a kernel instantiation reads frequency moves: fast heads through L1 or
 // from shared memory, pairs through L1, or not at all (every transition on its
@@ -340,13 +326,17 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
     unsigned long long* s_hist = s_sb + kNsb;                                     // J+2 if in smem
     const int nhist = P.J + 2;
     // this thread's counters: touched once per packet or event, so they live in
-    // shared memory and leave their registers to the transition loop
+    // shared memory and leave their registers to the transition loop; but not where
+    // the excursions' stacks of four CTAs want that L1 (REGS)
+    constexpr bool REGS = HYBRID && MINB == 4;
     unsigned long long* loc64 = s_hist + (P.hist_in_smem ? ((nhist + 1) & ~1) : 0) + threadIdx.x;
     unsigned* loc32 = reinterpret_cast<unsigned*>(loc64 - threadIdx.x + kLoc64 * blockDim.x) + threadIdx.x;
     constexpr int kSlots = NDIM == 3 ? kLoc32Events : kLoc32;
     uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + kSlots * blockDim.x);
-    auto cnt64 = [&](int i) -> unsigned long long& { return loc64[i * blockDim.x]; };
-    auto cnt32 = [&](int i) -> unsigned& { return loc32[i * blockDim.x]; };
+    unsigned long long reg64[kLoc64];
+    unsigned reg32[kLoc32];
+    auto cnt64 = [&](int i) -> unsigned long long& { return REGS ? reg64[i] : loc64[i * blockDim.x]; };
+    auto cnt32 = [&](int i) -> unsigned& { return REGS ? reg32[i] : loc32[i * blockDim.x]; };
 #pragma unroll
     for (int i = 0; i < kLoc64; ++i) cnt64(i) = 0ull;
 #pragma unroll
@@ -422,22 +412,26 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
         return false;
     };
 
+    // Whether the event words of Doppler rebins are kept (rebin_word).
+    constexpr bool KEEP = NDIM == 3 && !REGS;
+
     // The next event word, for a Doppler rebin of a 3D walk: every fourth draws a
     // block, kept in shared memory with its index (event indices grow by a few per
     // transition, so the index's low word names the block).  Drawing one per rebin
     // cost the sphere in outflow 4 %.
     auto rebin_word = [&]() -> unsigned {
+        if (!KEEP) return event_word(pid, e++, P.k0, P.k1);
         const unsigned long long b = e >> 2;
-        if (cnt32(L_EVENT_BLK) != (unsigned)b) {
+        if (loc32[L_EVENT_BLK * blockDim.x] != (unsigned)b) {
             const uint4 v = philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), (uint32_t)pid,
                                                  (uint32_t)(pid >> 32) | 0x80000000u), P);
-            cnt32(L_EVENT) = v.x;
-            cnt32(L_EVENT + 1) = v.y;
-            cnt32(L_EVENT + 2) = v.z;
-            cnt32(L_EVENT + 3) = v.w;
-            cnt32(L_EVENT_BLK) = (unsigned)b;
+            loc32[L_EVENT * blockDim.x] = v.x;
+            loc32[(L_EVENT + 1) * blockDim.x] = v.y;
+            loc32[(L_EVENT + 2) * blockDim.x] = v.z;
+            loc32[(L_EVENT + 3) * blockDim.x] = v.w;
+            loc32[L_EVENT_BLK * blockDim.x] = (unsigned)b;
         }
-        return cnt32(L_EVENT + (int)((unsigned)e++ & 3u));
+        return loc32[(L_EVENT + ((unsigned)e++ & 3u)) * blockDim.x];
     };
 
     // Outcome of word w in the current state's row, and the row's flags.
@@ -504,7 +498,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
         unsigned nbin = bin;
         if (act == ACT_REBIN) {
             const Rebin rb = P.rebin[min(cls, (unsigned)P.n_class - 1u) * (2u * NDIM) + face];
-            const unsigned w1 = NDIM == 3 ? rebin_word() : event_word(pid, e++, P.k0, P.k1);
+            const unsigned w1 = rebin_word();
             int jn = (int)bin + rb.m + (w1 >= rb.thr ? 1 : 0);
             if (jn < 0) { jn = 0; ++cnt32(L_CLAMP); }
             if (jn > (int)J - 1) { jn = (int)J - 1; ++cnt32(L_CLAMP); }
@@ -598,7 +592,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                         have = true;
                     }
                     if (have) {
-                        if (NDIM == 3) cnt32(L_EVENT_BLK) = ~(unsigned)(e >> 2);  // not the next event's block
+                        if (KEEP) loc32[L_EVENT_BLK * blockDim.x] = ~(unsigned)(e >> 2);  // not the next event's block
                         cell = min(cell, (unsigned)P.ncell - 1u);
                         cls = __ldg(&P.cell_class[cell]);
                         s = cls * J + min(bin, J - 1u);
@@ -840,20 +834,20 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
 }
 
 // A launch's threads per CTA and CTAs per SM (0: chosen by launch_variant), the
-// SMs, and the shared memory of a CTA and of each of its threads.
+// SMs, the shared memory of a CTA and of each of its threads, and the grid's depth
+// of a cell and share of frequency moves (rddmc_grid::freq_share).
 struct LaunchShape {
     int threads, ctas_per_sm, chunk, sms;
     size_t smem, smem_per_thread;
+    double tau_cell, share;
 
     // Fewer packets than the lanes of a launch that fills the chip with `blocks`
     // CTAs of 256 threads per SM.
-    bool few(const WalkParams& P, int blocks = RDDMC_WALK_MIN_BLOCKS) const {
+    bool few(const WalkParams& P, int blocks = 3) const {
         return !threads && !ctas_per_sm && P.n_packets < 256ull * blocks * (unsigned)sms;
     }
-    // More than that, and at most two rounds of four CTAs per SM.
-    bool two_rounds(const WalkParams& P) const {
-        return !threads && !ctas_per_sm && !few(P) && P.n_packets <= 2048ull * (unsigned)sms;
-    }
+    // Packets that four CTAs per SM hold at once and three do not.
+    bool fourth(const WalkParams& P) const { return few(P, 4) && !few(P); }
 };
 
 // Few packets crowd on the CTAs that start first, two to six warps on one
@@ -866,13 +860,12 @@ struct LaunchShape {
 // slab, 2e4 packets 3.6 -> 3.3 ms; 2048 steps on the hybrid sphere, 2e4 packets
 // 4.6 -> 2.6 ms.  With every packet in a lane from the start the default chunk is
 // 4096 transitions (2048 packets 69 -> 64 ms; 1024: 65, 16384: 64).
-template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT,
-          int MINB = HYBRID ? RDDMC_WALK_HYBRID_MIN_BLOCKS : RDDMC_WALK_MIN_BLOCKS>
+template <int NDIM, int PATH, bool HYBRID, bool PROPOSE, bool WEIGHT, int MINB>
 cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
     const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT, MINB>;
-    const bool few = L.few(P, std::max(MINB, RDDMC_WALK_MIN_BLOCKS));
+    const bool few = L.few(P, std::max(MINB, 3));
     const int threads = L.threads ? L.threads : (few ? 128 : 256);
-    const size_t smem = L.smem + (size_t)threads * L.smem_per_thread;
+    const size_t smem = L.smem + (HYBRID && MINB == 4 ? 0 : (size_t)threads * L.smem_per_thread);
     int ctas = L.ctas_per_sm;
     cudaError_t e = allow_smem(kernel, kSmemBlock);
     if (e != cudaSuccess) return e;
@@ -895,46 +888,103 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
     return cudaGetLastError();
 }
 
-// A 3D walk of one to two rounds of packets takes four CTAs per SM (64
-// registers): its second round is short, and more of the packets are in the
-// first (two 944-step slices of 1.3e5 packets on a 14^3 moving sphere: 3.1 -> 2.3 ms;
-// more packets are faster with three).
-template <int NDIM, int PATH>
-cudaError_t launch_path(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
-    if constexpr (NDIM == 3 && PATH != ROWS)
-        if (P.prop_b) return launch_variant<NDIM, PATH, false, true, false>(P, L, s);
-    if constexpr (NDIM == 1 || PATH == HEADS)
-        if (P.hybrid) return launch_variant<NDIM, PATH, true, false, false>(P, L, s);
-    if constexpr (NDIM == 3)
-        if (L.two_rounds(P)) return launch_variant<NDIM, PATH, false, false, false, 4>(P, L, s);
-    return launch_variant<NDIM, PATH, false, false, false>(P, L, s);
+// How a walk reads its transitions (Path) and how many CTAs per SM it targets.
+// The lines lie where the sweeps cross: cells of depth 5 to 1e6, 2e4 to 1.6e6
+// packets, slabs of 16-256 cells, static, moving and dusty grids of 16^3-128^3
+// cells, 64-256 bins, against heads at four CTAs per SM.
+// Below, the mean depth of a cell is tau and the share of frequency moves tau / dx^4.
+// A grid whose cells move leaves pairs and heads for its rebins.  Pairs pay from a
+// share of 5e4 on, where the launch fills the chip (1e6 packets, 512 steps, pairs
+// and heads: 16^3 x 64 bins, dx = 1, tau 2e4 1.18 and 0.84 ms, 8e4 0.75 and 0.73;
+// 32^3 x 128, dx = 1.25, tau 3e5 0.64 and 0.69; 24^3 x 256, dx = 0.47, tau 5e3 0.99
+// both, 2e4 0.78 and 0.85; slab of 64 x 128, tau 5e3 0.74 and 0.78).  Rows alone read
+// nothing in vain where almost every transition rebins: below a depth of 500 in 3D
+// (2e4 packets to escape from a 13^3 sphere of tau 82: 96 ms, heads 120), of 100 in a
+// slab.  Static 3D grids read rows below a depth and a share of 100 (tau 50, 1e6
+// packets: 16^3 x 64, share 50, 1.92 ms, pairs 4.1, heads 2.0; 24^3 x 256, share 1000,
+// pairs 1.42, rows 1.95); static slabs always pairs.  A dusty 3D grid's groups on the
+// rows look at the absorption of every
+// transition: heads once the lanes are full, up to the same share (tau 1e3, 1e6
+// packets: 0.98 ms, pairs 1.25).
+constexpr double kFrequent = 5.0e4, kThinMoving = 500.0, kThin = 100.0;
+
+template <int NDIM>
+int path_of(const WalkParams& P, const LaunchShape& L) {
+    const bool rows = !P.prop_b;  // there is no proposal walk on rows alone
+    if (P.moving) {
+        if (rows && L.tau_cell < (NDIM == 3 ? kThinMoving : kThin)) return ROWS;
+        return P.pair && L.share >= kFrequent && !L.few(P, 4) ? PAIRS : HEADS;
+    }
+    if (!P.pair) return HEADS;
+    if (NDIM == 1) return PAIRS;
+    if (rows && L.tau_cell < kThin && L.share < kThin) return ROWS;
+    return P.dust && !L.few(P, 4) && L.share < kFrequent ? HEADS : PAIRS;
 }
 
-// Pairs where the table has them, heads otherwise.  The weight method reads
-// heads (its weight is checked before every transition), and so does the 3D
-// hybrid, which leaves most groups for an excursion: heads name the first
-// transition that is not a frequency move without reading rows (2048 steps of
-// 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7 against 6.7
-// in a 20 km/s outflow); hybrid slabs do below cells of kThickHybrid (two slices
-// of 2856 steps, 5.3e4 packets at tau_cell 1.9e3 9.4 against 11.7 ms; at 2.4e4 1.6
-// against 1.9; at 5.8e4 pairs 5.1 against 5.3, at 4.5e5 3.9 against 4.5).  A moving
-// 3D grid leaves them for its rebins: pairs
-// where its cells are thick and the launch fills the chip (two 4096-step slices
-// of 1e6 packets on the sphere: 11.2 against 11.9 ms), heads where the latency
-// counts (16384 steps of 2e4 packets 5.0 against 5.4 ms, of 6e4 6.4 against 6.8),
-// rows alone below kThinCell (2e4 packets to escape from a 13^3 sphere of
-// tau_cell 82, where 99 % of the transitions rebin: 96 against 120 ms).
+// Three CTAs per SM (80 registers) keep the pair loop's two blocks of words and its
+// stream constants in registers, four (64) spill them: 27.7 against 28.2 ms on two
+// 4096-step slices of 4e6 packets (256 x 512 slab), 0.56 against 0.67 s on 1e5 packets
+// of the 64 x 128 slab to escape.  Four pay where the
+// packets fit four CTAs and not three (1.3e5 packets on a 24^3 x 256 sphere of tau
+// 30: 1.38 ms, with three 1.92); on static 3D grids of cells below 3e4, whose lanes
+// wait for rows (32^3 x 128, tau 300, 1e6 packets: 1.70 against 2.30 ms); on thin
+// moving slabs; and on heads of tables far past L2, whose lanes wait for memory
+// (16384 steps of 4e5 packets on a moving 128^3 x 256 medium: 53 against 58 ms; a
+// moving table pays from 2^24 rows on, a static one from 2^26).
+template <int NDIM>
+int blocks_of(const WalkParams& P, const LaunchShape& L, int path) {
+    if (L.few(P)) return 3;
+    if (NDIM == 1) return path == ROWS ? 4 : 3;
+    if ((L.fourth(P) && !P.prop_b) || (!P.moving && L.tau_cell < 3.0e4)) return 4;
+    return path == HEADS && (unsigned)P.n_rows > (P.moving ? 1u << 24 : 1u << 26) ? 4 : 3;
+}
+
+template <int NDIM, int PATH, bool PROPOSE>
+cudaError_t launch_blocks(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
+    return blocks_of<NDIM>(P, L, PATH) == 4 ? launch_variant<NDIM, PATH, false, PROPOSE, false, 4>(P, L, s)
+                                            : launch_variant<NDIM, PATH, false, PROPOSE, false, 3>(P, L, s);
+}
+
+// The hybrid walk.  In 3D it reads heads: most groups leave for an excursion, and
+// heads name the first transition that is not a frequency move without reading rows
+// (2048 steps of 2e5 packets on the 64^3 sphere: 3.5 ms against 4.6 ms static, 5.7
+// against 6.7 in a 20 km/s outflow); slabs do below cells of 4e4 (two slices of 2856
+// steps, 5.3e4 packets at tau 1.9e3 9.4 against 11.7 ms; at 2.4e4 1.6 against 1.9; at
+// 5.8e4 pairs 5.1 against 5.3, at 4.5e5 3.9 against 4.5).  Two CTAs per SM (128
+// registers) hold the excursion without spills; with more packets than they hold and
+// cells below 5e3, where excursions are what a packet does, four are faster (256
+// steps of 3e5 packets, 16^3 x 64: tau 1e3 8.3 -> 6.4 ms; tau 2e4 0.72 both).
+template <int NDIM>
+cudaError_t launch_hybrid(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
+    if constexpr (NDIM == 1)
+        if (P.pair && L.tau_cell >= 4.0e4) return launch_variant<1, PAIRS, true, false, false, 2>(P, L, s);
+    return P.n_packets > 512ull * (unsigned)L.sms && L.tau_cell < 5.0e3
+               ? launch_variant<NDIM, HEADS, true, false, false, 4>(P, L, s)
+               : launch_variant<NDIM, HEADS, true, false, false, 2>(P, L, s);
+}
+
+// The weight method reads heads: its weight is checked before every transition.
+// Four CTAs per SM pay on thin slabs whose packets they hold at once (1024 steps of
+// 1.3e5 packets, 256 x 128, tau 50: 0.72 against 0.88 ms).
+template <int NDIM, int PATH>
+cudaError_t launch_weights(WalkParams& P, const LaunchShape& L, cudaStream_t s) {
+    if constexpr (NDIM == 1)
+        if (L.fourth(P) && L.tau_cell < kThin) return launch_variant<1, PATH, false, false, true, 4>(P, L, s);
+    return launch_variant<NDIM, PATH, false, false, true, 3>(P, L, s);
+}
+
 template <int NDIM>
 cudaError_t launch_mode(WalkParams& P, bool smem_heads, const LaunchShape& L, cudaStream_t s) {
-    if (P.weights)
-        return smem_heads ? launch_variant<NDIM, HEADS_SMEM, false, false, true>(P, L, s)
-                          : launch_variant<NDIM, HEADS, false, false, true>(P, L, s);
+    if (P.weights) return smem_heads ? launch_weights<NDIM, HEADS_SMEM>(P, L, s) : launch_weights<NDIM, HEADS>(P, L, s);
+    if (P.hybrid) return launch_hybrid<NDIM>(P, L, s);
+    const int path = path_of<NDIM>(P, L);
     if constexpr (NDIM == 3)
-        if (P.thin && !P.prop_b && !P.hybrid) return launch_path<NDIM, ROWS>(P, L, s);
-    const bool heads = (P.hybrid && (NDIM == 3 || !P.thick_hybrid)) ||
-                       (NDIM == 3 && P.moving && (L.few(P, 4) || !P.thick));
-    const bool pairs = P.pair && !heads;
-    return pairs ? launch_path<NDIM, PAIRS>(P, L, s) : launch_path<NDIM, HEADS>(P, L, s);
+        if (P.prop_b)
+            return path == PAIRS ? launch_blocks<3, PAIRS, true>(P, L, s) : launch_blocks<3, HEADS, true>(P, L, s);
+    if (path == ROWS) return launch_blocks<NDIM, ROWS, false>(P, L, s);
+    if (path == HEADS) return launch_blocks<NDIM, HEADS, false>(P, L, s);
+    if constexpr (NDIM == 1) return launch_variant<1, PAIRS, false, false, false, 3>(P, L, s);
+    else return launch_blocks<3, PAIRS, false>(P, L, s);
 }
 
 // One scattering per thread at x_in with incoming direction +e_z; sample i
@@ -1432,9 +1482,6 @@ void fill_walk_params(const rddmc_grid& g, const WalkLaunch& w, WalkParams& P) {
     P.resume = o.resume;
     P.save_state = (o.steps_per_launch != 0 || o.resume || o.time_slice_us > 0) ? 1 : 0;
     P.lanes = 32;
-    P.thin = g.moving && g.tau_cell < kThinCell ? 1 : 0;
-    P.thick = g.tau_cell >= kThickCell ? 1 : 0;
-    P.thick_hybrid = g.tau_cell >= kThickHybrid ? 1 : 0;
     P.hist_in_smem = (g.J + 2 <= kSmemHistMax) ? 1 : 0;
     P.moving = g.moving ? 1 : 0;
     for (int a = 0; a < 3; ++a) {
@@ -1476,7 +1523,7 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return e;
     LaunchShape L{o.threads_per_cta, o.ctas_per_sm, o.chunk, nsm, (size_t)(kCounters + 8 + kNsb) * 8,
-                  kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4};
+                  kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4, g.tau_cell(), g.freq_share()};
     if (P.hist_in_smem) L.smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads
     const size_t counters = (size_t)(L.threads ? L.threads : 256) * L.smem_per_thread;

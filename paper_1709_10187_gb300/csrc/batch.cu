@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "escape.cuh"
@@ -34,8 +35,9 @@ constexpr unsigned FULL = 0xffffffffu;
 struct InstDesc {
     const uint4* rows;
     const uint2* fast;
-    const Pair* pair;               // null for a large table
+    const Pair* pair;               // null for a large table, and for a moving grid that reads heads
     const uint8_t* inside;          // with pair, static grids
+    static constexpr bool kDust = false;  // instances have none
     const uint32_t* cell_class;
     const Rebin* rebin;
     const double* edges;
@@ -55,9 +57,9 @@ struct BatchParams {
     unsigned long long* tally;
     unsigned long long total, max_steps;
     uint32_t k0, k1;
-    uint32_t rk0[10], rk1[10];
     int chunk;
     unsigned lanes;  // lanes of a warp that take packets
+    uint32_t rk0[10], rk1[10];  // 8 bytes past a multiple of 16, as in WalkParams
 };
 
 __device__ __forceinline__ unsigned bword(const uint4& r, unsigned q) {
@@ -95,19 +97,26 @@ struct LaneInst {
     const uint2* fast;
     const uint32_t* cell_class;
     const uint8_t* inside;
-    unsigned J, ncls1, n0, n01, ndim;
-    int ncell;
+    int J, n_class, ncell, n0, n01, ndim;
     static constexpr bool kDust = false;  // instances have none
 };
 
 // Bound by dispatch in the pair loop and by its lanes in thin media, which leave
 // it for the rows (the 64-instance study: 20.0 ms with heads, 11.5 ms).
-__global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ BatchParams P) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    LaneInst& L = reinterpret_cast<LaneInst*>(smem_raw)[threadIdx.x];
+// MOVES: some instance moves, and a lane reads what it needs of its instance from
+// the description: copies in shared memory take L1 that rebins and escapes want (8
+// moving spheres of 8^3 cells, tau 50, 1e5 packets each: 9.1 -> 8.8 ms; the study,
+// where none moves, 11.5 ms with copies, 11.8 without).
+template <bool MOVES, int MINB>
+__global__ void __launch_bounds__(256, MINB) batch_kernel(const __grid_constant__ BatchParams P) {
     const unsigned lane = threadIdx.x & 31u;
     bool have = false, exhausted = lane >= P.lanes;
     int inst = -1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LaneInst* copy = reinterpret_cast<LaneInst*>(smem_raw) + threadIdx.x;
+    const std::conditional_t<MOVES, InstDesc, LaneInst>* L;
+    if constexpr (MOVES) L = P.desc;
+    else L = copy;
     const Pair* pair = nullptr;
     unsigned nr1 = 0;
     unsigned long long gid = 0, t = 0, e = 0;
@@ -131,12 +140,12 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
     // One full transition on word w: every threshold, the outcome's action.
     // Returns true when the packet has finished.
     auto transition = [&](unsigned w) -> bool {
-        const bool slab = L.ndim == 1u;
+        const bool slab = L->ndim == 1;
         const unsigned ri = min(s, nr1);
-        const uint4 a = __ldg(&L.rows[slab ? ri : 2u * ri]);
+        const uint4 a = __ldg(&L->rows[slab ? ri : 2u * ri]);
         unsigned o = (unsigned)(w >= a.x) + (unsigned)(w >= a.y) + (unsigned)(w >= a.z);
         if (!slab) {
-            const uint4 b = __ldg(&L.rows[2u * ri + 1u]);
+            const uint4 b = __ldg(&L->rows[2u * ri + 1u]);
             o += (unsigned)(w >= b.x) + (unsigned)(w >= b.y) + (unsigned)(w >= b.z) + (unsigned)(w >= b.w);
         }
         const unsigned fl = a.w;
@@ -148,7 +157,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
         }
         const unsigned face = o - 2u;
         if (act == ACT_TO_MC) { ++n_abort; return true; }
-        const unsigned J = L.J;
+        const unsigned J = (unsigned)L->J;
         unsigned bin = min(s - cls * J, J - 1u);
         if (act == ACT_ESCAPE) {
             batch_escape(P, P.desc[inst], cell, bin, face, gid, e, (fl & FLAG_MOVING) != 0u);
@@ -157,7 +166,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
             return true;
         }
         if (act == ACT_REBIN) {
-            const Rebin rb = P.desc[inst].rebin[min(cls, L.ncls1) * (2u * L.ndim) + face];
+            const Rebin rb = P.desc[inst].rebin[min(cls, (unsigned)L->n_class - 1u) * (2u * (unsigned)L->ndim) + face];
             const unsigned w1 = event_word(gid, e++, P.k0, P.k1);
             int jn = (int)bin + rb.m + (w1 >= rb.thr ? 1 : 0);
             if (jn < 0) { jn = 0; ++n_clamp; }
@@ -165,9 +174,9 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
             bin = (unsigned)jn;
         }
         const unsigned ax = face >> 1;
-        const unsigned stride = ax == 0 ? 1u : (ax == 1 ? L.n0 : L.n01);
-        cell = min((face & 1u) ? cell + stride : cell - stride, (unsigned)L.ncell - 1u);
-        cls = __ldg(&L.cell_class[cell]);
+        const unsigned stride = ax == 0 ? 1u : (unsigned)(ax == 1 ? L->n0 : L->n01);
+        cell = min((face & 1u) ? cell + stride : cell - stride, (unsigned)L->ncell - 1u);
+        cls = __ldg(&L->cell_class[cell]);
         s = cls * J + bin;
         return false;
     };
@@ -195,9 +204,11 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                         inst = lo;
                         pair = D.pair;
                         nr1 = (unsigned)D.n_rows - 1u;
-                        L.rows = D.rows; L.fast = D.fast; L.cell_class = D.cell_class;
-                        L.inside = D.inside; L.J = (unsigned)D.J; L.ncell = D.ncell; L.ncls1 = (unsigned)D.n_class - 1u;
-                        L.n0 = (unsigned)D.n0; L.n01 = (unsigned)D.n01; L.ndim = (unsigned)D.ndim;
+                        if constexpr (MOVES)
+                            L = &D;
+                        else
+                            *copy = LaneInst{D.rows, D.fast, D.cell_class, D.inside, D.J,
+                                             D.n_class, D.ncell, D.n0, D.n01, D.ndim};
                     }
                     gid = D.pkt_begin + (q - P.off[inst]);
                     const unsigned w = event_word(gid, 0, P.k0, P.k1);
@@ -205,10 +216,10 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
                         idx[a] = (unsigned)D.src_cand[a][(D.src_ncand[a] == 2) ? ((w >> (31 - a)) & 1u) : 0u];
-                    cell = min(idx[0] + L.n0 * idx[1] + L.n01 * idx[2], (unsigned)L.ncell - 1u);
+                    cell = min(idx[0] + (unsigned)D.n0 * idx[1] + (unsigned)D.n01 * idx[2], (unsigned)L->ncell - 1u);
                     const unsigned bin = (unsigned)D.src_bin[(D.src_nbin == 2) ? ((w >> 28) & 1u) : 0u];
-                    cls = __ldg(&L.cell_class[cell]);
-                    s = cls * L.J + min(bin, L.J - 1u);
+                    cls = __ldg(&L->cell_class[cell]);
+                    s = cls * (unsigned)D.J + min(bin, (unsigned)D.J - 1u);
                     t = 0;
                     e = 1;
                     ++n_emit;
@@ -249,8 +260,8 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                             return false;
                         }
                         s = o >> 4;
-                        if (L.ndim == 1u ? walk_four_rows<1>(L, nr1, L.J, r, s, cell, cls)
-                                         : walk_four_rows<3>(L, nr1, L.J, r, s, cell, cls))
+                        if (L->ndim == 1 ? walk_four_rows<1>(*L, nr1, (unsigned)L->J, r, s, cell, cls)
+                                         : walk_four_rows<3>(*L, nr1, (unsigned)L->J, r, s, cell, cls))
                             return false;
                         if (m.ok2) {
                             s = (m.o2 - 32u) >> 4;
@@ -261,7 +272,7 @@ __global__ void __launch_bounds__(256, 3) batch_kernel(const __grid_constant__ B
                         // head loads (clamped speculative states), checked at its
                         // end, as in the single-grid walk
                         rn = ts.next(P);
-                        const uint2* fast = L.fast;
+                        const uint2* fast = L->fast;
                         const unsigned s0 = s;
                         const uint2 f0 = __ldg(&fast[min(s0, nr1)]);
                         const unsigned s1 = s0 + ((r.x >= f0.x) ? 1u : 0xffffffffu);
@@ -328,12 +339,30 @@ struct rddmc_batch {
     std::vector<uint64_t> n_packets;
     uint64_t tally_words = 0, total = 0;
     uint64_t desc_bytes = 0;
-    int default_ctas = 0;
+    bool moves = false;  // some instance moves
+    bool thin = false;   // most packets walk static 3D instances of cells below a depth of 3e4
+    int ctas = 0, ctas_full = 0;  // resident CTAs of 256 threads, per SM, of few packets' kernel and a full launch's
 };
 
 namespace {
 
-size_t lane_bytes(int threads) { return (size_t)threads * sizeof(LaneInst); }
+// The kernel of a batch: three CTAs per SM, and four where static 3D grids of thin
+// cells, whose lanes wait for rows, fill the chip, as in the single-grid walk (8
+// cubes of 8^3 cells, tau 500, 1e5 packets each: 2.7 -> 2.5 ms).
+using Kernel = void (*)(const BatchParams);
+Kernel kernel_of(const rddmc_batch* b, bool full) {
+    if (b->moves) return batch_kernel<true, 3>;
+    return b->thin && full ? batch_kernel<false, 4> : batch_kernel<false, 3>;
+}
+
+size_t lane_bytes(const rddmc_batch* b, int threads) { return b->moves ? 0 : (size_t)threads * sizeof(LaneInst); }
+
+int resident(const rddmc_batch* b, bool full, int threads) {
+    int ctas = 0;
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel_of(b, full), threads, lane_bytes(b, threads));
+    return e == cudaSuccess ? std::max(1, ctas) : 1;
+}
 
 uint64_t off_array_bytes(size_t n_inst) { return align256((n_inst + 1) * 8ull); }
 
@@ -362,17 +391,16 @@ void fill_params(const rddmc_batch* b, const void* d_desc, bool trial, const rdd
 // Launches the batch on s.  Fewer packets than the lanes of a launch that fills
 // the chip are spread over its schedulers as in the single-grid walk.
 cudaError_t launch(const rddmc_batch* b, BatchParams& P, const rddmc_run_opts* o, int nsm, cudaStream_t s) {
-    const int full = std::max(1, b->default_ctas);  // of 256 threads, per SM
-    const bool few = !o->threads_per_cta && !o->ctas_per_sm && P.total < 256ull * full * nsm;
+    const bool few = !o->threads_per_cta && !o->ctas_per_sm && P.total < 256ull * b->ctas * nsm;
     const int threads = o->threads_per_cta ? o->threads_per_cta : (few ? 128 : 256);
-    int ctas = o->ctas_per_sm ? o->ctas_per_sm : full;
+    int ctas = o->ctas_per_sm ? o->ctas_per_sm : b->ctas_full;
     P.lanes = 32;
     if (few) {
-        const Spread f = spread(P.total, 2 * full, nsm);
+        const Spread f = spread(P.total, 2 * b->ctas, nsm);
         ctas = f.ctas;
         P.lanes = f.lanes;
     }
-    batch_kernel<<<(unsigned)(ctas * nsm), threads, lane_bytes(threads), s>>>(P);
+    kernel_of(b, !few)<<<(unsigned)(ctas * nsm), threads, lane_bytes(b, threads), s>>>(P);
     return cudaGetLastError();
 }
 
@@ -458,9 +486,21 @@ int rddmc_batch_create(const rddmc_grid* const* grids, const void* const* d_tabl
     b->tally_words = tw;
     b->total = b->off.back();
     b->desc_bytes = align256(b->desc.size() * sizeof(InstDesc)) + 2 * off_array_bytes(b->desc.size());
-    int ctas = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, batch_kernel, 256, lane_bytes(256)) != cudaSuccess) ctas = 1;
-    b->default_ctas = std::max(1, ctas);
+    uint64_t thin = 0;
+    for (int i = 0; i < n_inst; ++i) {
+        b->moves = b->moves || grids[i]->moving;
+        if (grids[i]->ndim == 3 && grids[i]->tau_cell() < 3.0e4) thin += n_packets[i];
+    }
+    b->thin = 2 * thin > b->total;
+    b->ctas = resident(b, false, 256);
+    b->ctas_full = resident(b, true, 256);
+    // moving grids read heads where the packets fill the chip
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        b->total >= 256ull * b->ctas * nsm)
+        for (int i = 0; i < n_inst; ++i)
+            if (grids[i]->reads_heads()) b->desc[i].pair = nullptr;
     *out = b;
     return RDDMC_OK;
 }
@@ -585,15 +625,14 @@ int rddmc_batch_autotune(const rddmc_batch* b, const void* d_desc, const rddmc_r
     cudaStream_t s = (cudaStream_t)stream;
     const int threads_c[] = {128, 256};
     const int chunk_c[] = {64, 256, 1024};
-    int occ128 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ128, batch_kernel, 128, lane_bytes(128)) != cudaSuccess) occ128 = 6;
+    const int occ128 = resident(b, true, 128);
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return RDDMC_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return RDDMC_ERR_CUDA; }
     double best_r = -1.0;
     rddmc_run_opts bo = *base;
     for (int th : threads_c) {
-        const int occ = th == 128 ? std::max(1, occ128) : std::max(1, b->default_ctas);
+        const int occ = th == 128 ? occ128 : b->ctas_full;
         for (int ctas : {occ, std::max(1, occ - 1)}) {
             for (int ch : chunk_c) {
                 rddmc_run_opts o = *base;

@@ -71,6 +71,11 @@ struct rddmc_grid {
         return tau_cell() / (dx * dx * dx * dx);
     }
 
+    // A moving grid, too thick to walk on rows alone, whose share of frequency moves
+    // is too small for pairs (the lines stand at walk.cu's path_of).
+    bool thin_moving() const { return moving && tau_cell() < (ndim == 3 ? rddmc::kThinMoving : rddmc::kThin); }
+    bool reads_heads() const { return moving && !thin_moving() && freq_share() < rddmc::kFrequent; }
+
     // the table holds the walk's pairs (pairs.cuh)
     bool pairs() const { return (int64_t)n_class * J <= rddmc::kPairRows; }
     // and which cells lie four moves inside their class (walk_rows)

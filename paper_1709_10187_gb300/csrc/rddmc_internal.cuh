@@ -38,6 +38,10 @@ constexpr int kHistOff = 22;
 constexpr int kNsb = 64;            // impact-parameter bins over b/R in [0, kSbMax)
 constexpr double kSbMax = 1.28;
 constexpr int64_t kPairRows = 1 << 20;  // tables up to this many rows carry the walk's pairs (pairs.cuh)
+// Where walks change how they read transitions (walk.cu, path_of): share of frequency
+// moves from which pairs pay on a moving grid, mean depth of a cell below which rows
+// alone do (moving 3D grids; slabs and static grids).
+constexpr double kFrequent = 5.0e4, kThinMoving = 500.0, kThin = 100.0;
 constexpr int kUparN = 1024;        // |x| grid of the u_par envelope split points
 constexpr float kUparStep = 1.0f / 16.0f;
 

@@ -906,8 +906,6 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
 // rows look at the absorption of every
 // transition: heads once the lanes are full, up to the same share (tau 1e3, 1e6
 // packets: 0.98 ms, pairs 1.25).
-constexpr double kFrequent = 5.0e4, kThinMoving = 500.0, kThin = 100.0;
-
 template <int NDIM>
 int path_of(const WalkParams& P, const LaunchShape& L) {
     const bool rows = !P.prop_b;  // there is no proposal walk on rows alone

@@ -94,3 +94,35 @@ def test_hybrid_walk_does_not_depend_on_its_register_budget(w):
         fly = (few["status"] == 1) & (many["status"] == 1)
         assert np.array_equal(few["status"], many["status"]) and np.array_equal(few[k][fly], many[k][fly]), k
     p.close()
+
+
+@pytest.mark.parametrize("depth", [60.0, 700.0, 6.0e4])
+@pytest.mark.parametrize("moving", [False, True])
+def test_batches_match_the_oracle_on_every_route(depth, moving):
+    # batches of static cubes (thin and thick) and with a moving grid (pairs, or heads
+    # where the packets fill the chip), few packets and more than fit at once
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ws = [CUBE.with_(tau0=depth * 4.0, vmax_kms=30.0 if moving else 0.0),
+          SLAB.with_(tau0=depth * 4.0), CUBE.with_(tau0=depth * 4.0, J=9, seed=3)]
+    ps, ots, gs = [R.Problem(w) for w in ws], [], []
+    for w, p in zip(ws, ps):
+        g = C.Grid(w)
+        ot = g.table()
+        thr, _ = p.rows()
+        sel = np.ones(w.ncell * w.J, bool) if w.mask() is None else np.repeat(w.mask().astype(bool), w.J)
+        ot["thr"][sel] = thr[sel]
+        gs.append(g)
+        ots.append(ot)
+    for total in (3000, 1100 * sms):
+        n = [total // 2, total // 6, total // 3]
+        b = R.Batch(ps, n)
+        b.launch(R.RunOpts(0x5EED, 0, 45))
+        first = 0
+        for i, w in enumerate(ws):
+            got, want = b.read(i), C.walk(gs[i], ots[i], 0x5EED, first, n[i], max_steps=45)
+            for k in ("emitted", "escaped", "aborted", "steps", "clamps", "event_draws"):
+                assert got[k] == want[k], (total, i, k)
+            assert np.array_equal(got["hist"], want["hist"]) and np.array_equal(got["sb"], want["sb"])
+            first += n[i]
+    for p in ps:
+        p.close()

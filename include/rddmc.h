@@ -138,7 +138,16 @@ typedef struct rddmc_leak_params {
  *   ctas_per_sm, threads_per_cta, chunk  launch schedule (0 = library default):
  *                 persistent grid of ctas_per_sm * #SM CTAs of threads_per_cta
  *                 threads (a multiple of 32, at most 256); `chunk` transitions
- *                 (multiple of 4) between warp refills.
+ *                 (multiple of 4) between warp refills.  Library defaults: 256
+ *                 threads, the CTAs that are resident (two to four by the kind of
+ *                 walk), chunk 256.  A launch with both shape fields 0 and fewer
+ *                 packets than those CTAs have lanes uses CTAs of 128 threads, as
+ *                 many as the packets need, lets only some lanes of each warp take
+ *                 packets while one or two warps per scheduler hold them all, and
+ *                 with chunk 0 and no wall-time slice or proposal looks for new
+ *                 packets every 4096 transitions only; any explicit shape turns
+ *                 that off.  With time_slice_us, ctas_per_sm is cut to the resident
+ *                 CTAs.  No result depends on the schedule.
  *   table_in_smem 1: stage the fast row heads in shared memory when they fit
  *                 (the dust weight method; the other walks read a denser table
  *                 through L1, which measured faster); 0: gather them from
@@ -414,7 +423,8 @@ typedef struct rddmc_time_step {
                                0: packets resume from the state buffer */
     int32_t chunk;          /* transitions a thread runs between refills: multiple of 4, 0 = 256 */
     int32_t threads_per_cta; /* multiple of 32, at most 256; 0 = 256 */
-    int32_t ctas_per_sm;    /* 0 = occupancy limit */
+    int32_t ctas_per_sm;    /* 0 = occupancy limit; with both 0, fewer packets than lanes go to CTAs of 128
+                               threads, as many as they need (results do not change) */
     int32_t regroup;        /* lanes still walking their packets break off, so that the lanes whose
                                packets reached t_end take new ones, once fewer than this many of a
                                warp's lanes are walking (packets keep their state in registers and

@@ -53,7 +53,8 @@ enum Counter : int {
 
 // 2-bit actions per outcome in the flags word.
 constexpr uint32_t ACT_MOVE = 0u, ACT_ESCAPE = 1u, ACT_TO_MC = 2u, ACT_REBIN = 3u;
-constexpr uint32_t FLAG_FASTZ = 1u << 28;   // every spatial outcome is a plain move, and there is no absorption
+constexpr uint32_t FLAG_FASTZ = 1u << 28;   // every spatial outcome is a plain move (of a packet that is not absorbed: dusty
+                                           // grids look at abs_thr as well)
 constexpr uint32_t FLAG_FASTX = 1u << 29;   // both frequency outcomes are plain moves
 constexpr uint32_t FLAG_MOVING = 1u << 30;
 constexpr uint32_t FLAG_THIN = 1u << 31;

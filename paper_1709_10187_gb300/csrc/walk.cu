@@ -14,9 +14,10 @@
 // four, checked at its end, and a transition whose word reaches its pair's
 // guard is taken row by row with the rest of its group, plain moves (frequency
 // or spatial) in a short step and other outcomes in the generic one.  Larger
-// tables and the dust weight method read the 8-byte fast heads {thr0, thr1 or
-// 0}: four transitions run as a chain of head loads (w < thr1: one bin down
-// when w < thr0, else up).
+// tables, the dust weight method and walks with fewer frequency moves read the
+// 8-byte fast heads {thr0, thr1 or 0}: four transitions run as a chain of head
+// loads (w < thr1: one bin down when w < thr0, else up).  Grids of thin cells are
+// walked on their rows alone.  path_of says which and why.
 // Everything else -- spatial moves, Doppler rebins, escapes through exterior
 // faces, and frequency outcomes that are not plain moves (their head holds 0)
 // -- goes through one generic step that reads the full row (through L1) and
@@ -300,8 +301,8 @@ enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CO
 
 // How a kernel instantiation reads frequency moves: fast heads through L1 or
 // from shared memory, pairs through L1, or not at all (every transition on its
-// row: a moving grid of thin cells, where most transitions cross a Doppler shift
-// and speculative frequency moves are gathers in vain).
+// row: grids of thin cells, where most transitions are spatial and speculative
+// frequency moves are gathers in vain).
 enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2, ROWS = 3 };
 
 // What bounds it: dispatch.  A Philox block costs 17 wide products (3.65 cycles
@@ -903,9 +904,8 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
 // slab.  Static 3D grids read rows below a depth and a share of 100 (tau 50, 1e6
 // packets: 16^3 x 64, share 50, 1.92 ms, pairs 4.1, heads 2.0; 24^3 x 256, share 1000,
 // pairs 1.42, rows 1.95); static slabs always pairs.  A dusty 3D grid's groups on the
-// rows look at the absorption of every
-// transition: heads once the lanes are full, up to the same share (tau 1e3, 1e6
-// packets: 0.98 ms, pairs 1.25).
+// rows look at the absorption of every transition: heads once the lanes are full, up
+// to the same share (tau 1e3, 1e6 packets: 0.98 ms, pairs 1.25).
 template <int NDIM>
 int path_of(const WalkParams& P, const LaunchShape& L) {
     const bool rows = !P.prop_b;  // there is no proposal walk on rows alone
@@ -922,13 +922,13 @@ int path_of(const WalkParams& P, const LaunchShape& L) {
 // Three CTAs per SM (80 registers) keep the pair loop's two blocks of words and its
 // stream constants in registers, four (64) spill them: 27.7 against 28.2 ms on two
 // 4096-step slices of 4e6 packets (256 x 512 slab), 0.56 against 0.67 s on 1e5 packets
-// of the 64 x 128 slab to escape.  Four pay where the
-// packets fit four CTAs and not three (1.3e5 packets on a 24^3 x 256 sphere of tau
-// 30: 1.38 ms, with three 1.92); on static 3D grids of cells below 3e4, whose lanes
-// wait for rows (32^3 x 128, tau 300, 1e6 packets: 1.70 against 2.30 ms); on thin
-// moving slabs; and on heads of tables far past L2, whose lanes wait for memory
-// (16384 steps of 4e5 packets on a moving 128^3 x 256 medium: 53 against 58 ms; a
-// moving table pays from 2^24 rows on, a static one from 2^26).
+// of the 64 x 128 slab to escape.  Four pay in 3D where the packets fit four CTAs and
+// not three (1.3e5 packets on a 24^3 x 256 sphere of tau 30: 1.38 ms, with three
+// 1.92); on static 3D grids of cells below 3e4, whose lanes wait for rows (32^3 x
+// 128, tau 300, 1e6 packets: 1.70 against 2.30 ms); on thin moving slabs; and on heads
+// of tables far past L2, whose lanes wait for memory (16384 steps of 4e5 packets on a
+// moving 128^3 x 256 medium: 53 against 58 ms; a moving table pays from 2^24 rows on,
+// a static one from 2^26).
 template <int NDIM>
 int blocks_of(const WalkParams& P, const LaunchShape& L, int path) {
     if (L.few(P)) return 3;

@@ -205,9 +205,7 @@ __global__ void __launch_bounds__(kRowEdges)
 
 // The walk's pair of each row (pairs.cuh) from the fast heads of the three rows
 // around it in its class block.
-__global__ void pair_kernel(const uint2* __restrict__ fast, Pair* __restrict__ pair, int J, int64_t nrow) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrow) return;
+__device__ __forceinline__ Pair pair_of(const uint2* __restrict__ fast, int J, int64_t r) {
     const int j = (int)(r % J);
     uint32_t t[3], guard = 0xffffffffu;
 #pragma unroll
@@ -217,31 +215,38 @@ __global__ void pair_kernel(const uint2* __restrict__ fast, Pair* __restrict__ p
         t[i + 1] = f.x;
         guard = min(guard, f.y);
     }
-    pair[r] = Pair{t[0], t[1], t[2], guard};
+    return Pair{t[0], t[1], t[2], guard};
 }
 
-// Per cell, whether every cell within four moves along the axes lies in the grid
-// and in its class, so that four transitions leave a packet's class as it is.  Up
-// to 129 loads per cell, of L1: 1.4 ms for 256^3 cells, where a pass over the cells
-// on the host took 230 ms of the 1.3 s that the grid takes.
+// Whether every cell within four moves of cell c along the axes lies in the grid and
+// in its class, so that four transitions leave a packet's class as it is: up to 129
+// loads per cell, of L1.
 template <int NDIM>
-__global__ void inside_kernel(const uint32_t* __restrict__ cell_class, uint8_t* __restrict__ inside, int n0, int n1,
-                              int n2, int64_t ncell) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncell) return;
+__device__ __forceinline__ bool inside_class(const uint32_t* __restrict__ cell_class, int64_t c, int n0, int n1, int n2) {
     constexpr int M = 4, MY = NDIM == 3 ? M : 0;
     const int i0 = (int)(c % n0), i1 = (int)(c / n0 % n1), i2 = (int)(c / ((int64_t)n0 * n1));
     bool in = i0 >= M && i0 + M < n0 && (NDIM == 1 || (i1 >= M && i1 + M < n1 && i2 >= M && i2 + M < n2));
-    if (in) {
-        const uint32_t k = cell_class[c];
-        for (int z = -MY; z <= MY && in; ++z)
-            for (int y = abs(z) - MY; y <= MY - abs(z) && in; ++y) {
-                const int m = M - abs(z) - abs(y);
-                const uint32_t* row = cell_class + c + ((int64_t)z * n1 + y) * n0;
-                for (int x = -m; x <= m; ++x) in = in && row[x] == k;
-            }
-    }
-    inside[c] = in ? 1 : 0;
+    if (!in) return false;
+    const uint32_t k = cell_class[c];
+    for (int z = -MY; z <= MY && in; ++z)
+        for (int y = abs(z) - MY; y <= MY - abs(z) && in; ++y) {
+            const int m = M - abs(z) - abs(y);
+            const uint32_t* row = cell_class + c + ((int64_t)z * n1 + y) * n0;
+            for (int x = -m; x <= m; ++x) in = in && row[x] == k;
+        }
+    return in;
+}
+
+// A thread per row's pair and, on static grids, per cell's mark, in one launch: a
+// few microseconds for small grids, 1.4 ms for 256^3 cells, where a pass over the cells
+// on the host took 230 ms of the 1.3 s that the grid takes.
+template <int NDIM>
+__global__ void pair_kernel(const uint2* __restrict__ fast, Pair* __restrict__ pair, int J, int64_t nrow,
+                            const uint32_t* __restrict__ cell_class, uint8_t* __restrict__ inside, int n0, int n1,
+                            int n2, int64_t nmark) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nrow) pair[i] = pair_of(fast, J, i);
+    if (i < nmark) inside[i] = inside_class<NDIM>(cell_class, i, n0, n1, n2) ? 1 : 0;
 }
 
 // Split points (u1, u0) of the three-part rejection envelope of the parallel
@@ -353,14 +358,11 @@ cudaError_t launch_precompute(const rddmc_grid& g, void* d_table, cudaStream_t s
                                                   ka_row, weighted, tiles, per_block, nrow);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.pairs()) {
-        pair_kernel<<<(unsigned)((nrow + 255) / 256), 256, 0, s>>>(fast, (Pair*)(base + g.off_pair), g.J, nrow);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (g.inside()) {
-        const auto inside_k = g.ndim == 1 ? inside_kernel<1> : inside_kernel<3>;
-        inside_k<<<(unsigned)((g.ncell + 255) / 256), 256, 0, s>>>((const uint32_t*)(base + g.off_class),
-                                                                   (uint8_t*)(base + g.off_inside), g.n[0], g.n[1],
-                                                                   g.n[2], g.ncell);
+        const int64_t nmark = g.inside() ? g.ncell : 0;
+        const auto pair_k = g.ndim == 1 ? pair_kernel<1> : pair_kernel<3>;
+        pair_k<<<(unsigned)((std::max(nrow, nmark) + 255) / 256), 256, 0, s>>>(
+            fast, (Pair*)(base + g.off_pair), g.J, nrow, (const uint32_t*)(base + g.off_class),
+            (uint8_t*)(base + g.off_inside), g.n[0], g.n[1], g.n[2], nmark);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // the u_par envelope table serves only the continuous MC of the hybrid scheme

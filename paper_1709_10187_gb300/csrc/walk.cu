@@ -294,16 +294,33 @@ __device__ __forceinline__ bool prop_takes(const WalkParams& P, unsigned cell, u
     return l >= P.prop_llo && l <= P.prop_lhi;
 }
 
-// Per-thread counters in shared memory.
+// Per-thread counters, and the block of event words that a 3D walk keeps for its
+// rebins with its index.
 enum Loc64 { L_STEPS = 0, L_EDRAW = 1, L_MC = 2, kLoc64 = 3 };
-enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6,
-             L_EVENT_BLK = 6, L_EVENT = 7, kLoc32Events = 11 };  // from L_EVENT_BLK: the event words kept for rebins (3D)
+enum Loc32 { L_EMIT = 0, L_ESC = 1, L_ABORT = 2, L_CLAMP = 3, L_STATUS = 4, L_CONV = 5, kLoc32 = 6 };
+constexpr int kEvent = 5;  // index, four words
 
 // How a kernel instantiation reads frequency moves: fast heads through L1 or
 // from shared memory, pairs through L1, or not at all (every transition on its
 // row: grids of thin cells, where most transitions are spatial and speculative
 // frequency moves are gathers in vain).
 enum Path { HEADS = 0, HEADS_SMEM = 1, PAIRS = 2, ROWS = 3 };
+
+// Where an instantiation's counters and kept event words lie.  They are touched once
+// per packet or event, so with pairs (and in the weight and hybrid walks) they live
+// in shared memory and leave their registers to the transition loop.  Heads and rows
+// count in registers: 48 bytes a thread in shared memory are 36-48 KiB of the L1 that
+// their gathers, and the stacks of excursions at four CTAs, want.  Late slices of
+// 4e5 packets: moving 128^3 x 256 medium 53 ms, 68 with everything in shared memory;
+// static 64^3 x 256 14.9 and 17.1; moving 32^3 x 128 17.0 and 19.7.  The event words
+// stay there (the sphere in outflow 4 %), but not for heads at four CTAs, the large
+// tables' choice (moving 64^3 x 256 29 ms with them, 26 without).
+template <int NDIM, int PATH, bool HYBRID, bool WEIGHT, int MINB>
+struct Local {
+    static constexpr bool regs = HYBRID ? MINB == 4 : !WEIGHT && (PATH == HEADS || PATH == ROWS);
+    static constexpr bool keep = NDIM == 3 && !(PATH == HEADS && MINB == 4);
+    static constexpr int bytes = (regs ? 0 : kLoc64 * 8 + kLoc32 * 4) + (keep ? kEvent * 4 : 0);  // of shared memory, a thread
+};
 
 // What bounds it: dispatch.  A Philox block costs 17 wide products (3.65 cycles
 // of the multiply pipe each) and 19 xors, measured at 81 cycles per warp and
@@ -326,18 +343,22 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
     unsigned long long* s_sb = s_face + 8;                                        // kNsb
     unsigned long long* s_hist = s_sb + kNsb;                                     // J+2 if in smem
     const int nhist = P.J + 2;
-    // this thread's counters: touched once per packet or event, so they live in
-    // shared memory and leave their registers to the transition loop; but not where
-    // the excursions' stacks of four CTAs want that L1 (REGS)
-    constexpr bool REGS = HYBRID && MINB == 4;
+    using Loc = Local<NDIM, PATH, HYBRID, WEIGHT, MINB>;
+    constexpr bool REGS = Loc::regs, KEEP = Loc::keep;
     unsigned long long* loc64 = s_hist + (P.hist_in_smem ? ((nhist + 1) & ~1) : 0) + threadIdx.x;
-    unsigned* loc32 = reinterpret_cast<unsigned*>(loc64 - threadIdx.x + kLoc64 * blockDim.x) + threadIdx.x;
-    constexpr int kSlots = NDIM == 3 ? kLoc32Events : kLoc32;
-    uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + kSlots * blockDim.x);
+    unsigned* loc32 = reinterpret_cast<unsigned*>(loc64 - threadIdx.x + (REGS ? 0 : kLoc64) * blockDim.x) + threadIdx.x;
+    uint2* s_fast = reinterpret_cast<uint2*>(loc32 - threadIdx.x + ((REGS ? 0 : kLoc32) + (KEEP ? kEvent : 0)) * blockDim.x);
     unsigned long long reg64[kLoc64];
     unsigned reg32[kLoc32];
-    auto cnt64 = [&](int i) -> unsigned long long& { return REGS ? reg64[i] : loc64[i * blockDim.x]; };
-    auto cnt32 = [&](int i) -> unsigned& { return REGS ? reg32[i] : loc32[i * blockDim.x]; };
+    auto cnt64 = [&](int i) -> unsigned long long& {
+        if constexpr (REGS) return reg64[i];
+        else return loc64[i * blockDim.x];
+    };
+    auto cnt32 = [&](int i) -> unsigned& {
+        if constexpr (REGS) return reg32[i];
+        else return loc32[i * blockDim.x];
+    };
+    auto event = [&](int i) -> unsigned& { return loc32[((REGS ? 0 : kLoc32) + i) * blockDim.x]; };
 #pragma unroll
     for (int i = 0; i < kLoc64; ++i) cnt64(i) = 0ull;
 #pragma unroll
@@ -413,9 +434,6 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
         return false;
     };
 
-    // Whether the event words of Doppler rebins are kept (rebin_word).
-    constexpr bool KEEP = NDIM == 3 && !REGS;
-
     // The next event word, for a Doppler rebin of a 3D walk: every fourth draws a
     // block, kept in shared memory with its index (event indices grow by a few per
     // transition, so the index's low word names the block).  Drawing one per rebin
@@ -423,16 +441,16 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
     auto rebin_word = [&]() -> unsigned {
         if (!KEEP) return event_word(pid, e++, P.k0, P.k1);
         const unsigned long long b = e >> 2;
-        if (loc32[L_EVENT_BLK * blockDim.x] != (unsigned)b) {
+        if (event(0) != (unsigned)b) {
             const uint4 v = philox_rk(make_uint4((uint32_t)b, (uint32_t)(b >> 32), (uint32_t)pid,
                                                  (uint32_t)(pid >> 32) | 0x80000000u), P);
-            loc32[L_EVENT * blockDim.x] = v.x;
-            loc32[(L_EVENT + 1) * blockDim.x] = v.y;
-            loc32[(L_EVENT + 2) * blockDim.x] = v.z;
-            loc32[(L_EVENT + 3) * blockDim.x] = v.w;
-            loc32[L_EVENT_BLK * blockDim.x] = (unsigned)b;
+            event(1) = v.x;
+            event(2) = v.y;
+            event(3) = v.z;
+            event(4) = v.w;
+            event(0) = (unsigned)b;
         }
-        return loc32[(L_EVENT + ((unsigned)e++ & 3u)) * blockDim.x];
+        return event(1 + (int)((unsigned)e++ & 3u));
     };
 
     // Outcome of word w in the current state's row, and the row's flags.
@@ -593,7 +611,7 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
                         have = true;
                     }
                     if (have) {
-                        if (KEEP) loc32[L_EVENT_BLK * blockDim.x] = ~(unsigned)(e >> 2);  // not the next event's block
+                        if (KEEP) event(0) = ~(unsigned)(e >> 2);  // not the next event's block
                         cell = min(cell, (unsigned)P.ncell - 1u);
                         cls = __ldg(&P.cell_class[cell]);
                         s = cls * J + min(bin, J - 1u);
@@ -835,11 +853,11 @@ __global__ void __launch_bounds__(256, MINB) walk_kernel(const __grid_constant__
 }
 
 // A launch's threads per CTA and CTAs per SM (0: chosen by launch_variant), the
-// SMs, the shared memory of a CTA and of each of its threads, and the grid's depth
-// of a cell and share of frequency moves (rddmc_grid::freq_share).
+// SMs, the shared memory of a CTA but for its threads' own (Local), and the grid's
+// depth of a cell and share of frequency moves (rddmc_grid::freq_share).
 struct LaunchShape {
     int threads, ctas_per_sm, chunk, sms;
-    size_t smem, smem_per_thread;
+    size_t smem;
     double tau_cell, share;
 
     // Fewer packets than the lanes of a launch that fills the chip with `blocks`
@@ -866,7 +884,7 @@ cudaError_t launch_variant(WalkParams& P, const LaunchShape& L, cudaStream_t s) 
     const auto kernel = walk_kernel<NDIM, PATH, HYBRID, PROPOSE, WEIGHT, MINB>;
     const bool few = L.few(P, std::max(MINB, 3));
     const int threads = L.threads ? L.threads : (few ? 128 : 256);
-    const size_t smem = L.smem + (HYBRID && MINB == 4 ? 0 : (size_t)threads * L.smem_per_thread);
+    const size_t smem = L.smem + (size_t)threads * Local<NDIM, PATH, HYBRID, WEIGHT, MINB>::bytes;
     int ctas = L.ctas_per_sm;
     cudaError_t e = allow_smem(kernel, kSmemBlock);
     if (e != cudaSuccess) return e;
@@ -926,9 +944,9 @@ int path_of(const WalkParams& P, const LaunchShape& L) {
 // not three (1.3e5 packets on a 24^3 x 256 sphere of tau 30: 1.38 ms, with three
 // 1.92); on static 3D grids of cells below 3e4, whose lanes wait for rows (32^3 x
 // 128, tau 300, 1e6 packets: 1.70 against 2.30 ms); on thin moving slabs; and on heads
-// of tables far past L2, whose lanes wait for memory (16384 steps of 4e5 packets on a
-// moving 128^3 x 256 medium: 53 against 58 ms; a moving table pays from 2^24 rows on,
-// a static one from 2^26).
+// of tables far past L2, whose lanes wait for memory (a late slice of 16384 steps, 4e5
+// packets on a moving 128^3 x 256 medium: 53 against 55 ms, 1.5e6 packets 43 against
+// 49; a moving table pays from 2^24 rows on, a static one from 2^26).
 template <int NDIM>
 int blocks_of(const WalkParams& P, const LaunchShape& L, int path) {
     if (L.few(P)) return 3;
@@ -1521,10 +1539,11 @@ cudaError_t launch_walk(const rddmc_grid& g, const WalkLaunch& w, cudaStream_t s
     if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return e;
     LaunchShape L{o.threads_per_cta, o.ctas_per_sm, o.chunk, nsm, (size_t)(kCounters + 8 + kNsb) * 8,
-                  kLoc64 * 8 + (g.ndim == 3 ? kLoc32Events : kLoc32) * 4, g.tau_cell(), g.freq_share()};
+                  g.tau_cell(), g.freq_share()};
     if (P.hist_in_smem) L.smem += (size_t)((g.J + 2 + 1) & ~1) * 8;
     const size_t rows_bytes = (size_t)P.n_rows * 8;  // fast heads
-    const size_t counters = (size_t)(L.threads ? L.threads : 256) * L.smem_per_thread;
+    const int local = g.ndim == 1 ? Local<1, HEADS_SMEM, false, true, 3>::bytes : Local<3, HEADS_SMEM, false, true, 3>::bytes;
+    const size_t counters = (size_t)(L.threads ? L.threads : 256) * local;
     const bool smem_heads = P.weights && o.table_in_smem && L.smem + counters + rows_bytes <= (size_t)smem_optin;
     if (smem_heads) L.smem += rows_bytes;
     if ((e = cudaMemsetAsync(P.cursor, 0, 8, s)) != cudaSuccess) return e;
